@@ -135,7 +135,10 @@ int variant_for_full(const K32 &a, int prec, int gf) {
         auto it = g_var.find(var_key(a.V, a.k, prec, gf));
         if (it != g_var.end()) return it->second;
     }
-    return variant_ok(1, a.k, gf) ? 1 : 0;
+    // not tuned yet (products before the first solve with this shape): the pipelined pair over
+    // the tiled order for batches, direct loads for one RHS.  24^3x64 FP32, per product:
+    // k = 16 0.87 ms (staged 1.64), k = 1 68 us (staged 124)
+    return variant_ok(19, a.k, gf) ? 19 : 2;
 }
 
 template <typename S, int GF, bool DAG, int EPI>
