@@ -424,7 +424,7 @@ static void apply_A64(eig_op_s *op, Field in, Field out, cudaStream_t s) {
     apply_M(op, u, out, true, true, s);
 }
 
-// natural (host or device) -> internal FP64 field
+// natural (host or device) -> internal field of any storage precision
 static void load_natural(eig_op_s *op, const double *nat, Field dst, cudaStream_t s) {
     const size_t bytes = (size_t)dst.v.V * 12 * 16 * dst.v.k;
     const double *src = nat;
@@ -1162,14 +1162,14 @@ static void ay_run(eig_basis_s *B, const ColSet &A, const double *Y, const ColSe
     CUDA_CK(launch_gemm_ay(A, Y, Out, beta, nrow, s));
 }
 
-// x64 <- x64 + U H^{-1} U^H r64 for k RHS (r64 given in FP64).
-static void deflate_into(eig_basis_s *B, Field r64, Field x64, cudaStream_t s) {
+// xsv <- U H^{-1} U^H rsv for k RHS, both in the basis precision (op->rsv, op->xsv).  The
+// host copy of the coefficients is read by an asynchronous copy: the caller synchronises
+// the stream before Yr goes out of scope.
+static void deflate_core(eig_basis_s *B, int k, std::vector<cd> &Yr, cudaStream_t s) {
     eig_op_s *op = B->op;
-    const int l = B->l, k = r64.v.k;
-    if (l == 0) return;
+    const int l = B->l;
     if (!B->chol_ok) throw Error{EIG_ERR_BREAKDOWN, "H = U^H A U is not positive definite"};
     Field rsv = op->rsv.view(k);
-    CUDA_CK(launch_combine(rsv, 1.0, r64, 0.0, null_field(), s));
     const bool f64 = op->wprec == P64;
     ColSet R = field_cols(rsv.v.data, f64, k, B->fsize(), k, true);
     const cd *Cc = ahb_to_host(B, basis_cols(B, 0, l), R, op->ncomplex(), s);
@@ -1178,7 +1178,7 @@ static void deflate_into(eig_basis_s *B, Field r64, Field x64, cudaStream_t s) {
     for (int a = 0; a < l; a++)
         for (int q = 0; q < k; q++) Yc[(size_t)q * l + a] = Cc[(size_t)a * k + q];
     dense::chol_solve(l, B->Lc.data(), Yc.data(), k);
-    std::vector<cd> Yr((size_t)l * k);
+    Yr.resize((size_t)l * k);
     for (int a = 0; a < l; a++)
         for (int q = 0; q < k; q++) Yr[(size_t)a * k + q] = Yc[(size_t)q * l + a];
     B->Y.ensure((size_t)l * k * 16);
@@ -1186,8 +1186,18 @@ static void deflate_into(eig_basis_s *B, Field r64, Field x64, cudaStream_t s) {
     Field xsv = op->xsv.view(k);
     ColSet X = field_cols(xsv.v.data, f64, k, B->fsize(), k, true);
     ay_run(B, basis_cols(B, 0, l), B->Y.as<double>(), X, 0.0, op->ncomplex(), s);
-    CUDA_CK(launch_combine(x64, 1.0, x64, 1.0, xsv, s));
-    sync(s);  // Yr must outlive the async copy
+}
+
+// x64 <- x64 + U H^{-1} U^H r64 for k RHS (r64 given in FP64).
+static void deflate_into(eig_basis_s *B, Field r64, Field x64, cudaStream_t s) {
+    eig_op_s *op = B->op;
+    const int k = r64.v.k;
+    if (B->l == 0) return;
+    std::vector<cd> Yr;
+    CUDA_CK(launch_combine(op->rsv.view(k), 1.0, r64, 0.0, null_field(), s));
+    deflate_core(B, k, Yr, s);
+    CUDA_CK(launch_combine(x64, 1.0, x64, 1.0, op->xsv.view(k), s));
+    sync(s);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1479,11 +1489,10 @@ eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int
     std::lock_guard<std::mutex> lk(op->mu);
     ensure_workspace(op);
     cudaStream_t s = (cudaStream_t)stream;
-    Field x64 = op->x64.view(k);
-    load_natural(op, in, x64, s);
     if (which == 3) {  // A = M^H M in double-float arithmetic
         const long n = op->Vf * 12 * (long)k;
-        Field t1 = op->u64.view(k), t2 = op->r64.view(k);
+        Field x64 = op->x64.view(k), t1 = op->u64.view(k), t2 = op->r64.view(k);
+        load_natural(op, in, x64, s);
         CUDA_CK(launch_to_dd(x64.v.data, t1.v.data, n, s));
         CUDA_CK(launch_dslash_dd(op->call(x64, t2, false, true), op->gauge_dd.p, t1.v.data, t2.v.data, s));
         CUDA_CK(launch_dslash_dd(op->call(x64, t1, true, true), op->gauge_dd.p, t2.v.data, t1.v.data, s));
@@ -1492,8 +1501,10 @@ eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int
         sync(s);
         return EIG_OK;
     }
+    // the vectors go straight between the natural layout and the op's storage precision (the
+    // same roundings as through an FP64 field, without its passes over memory)
     Field a = op->p.view(k), b = op->u.view(k), c = op->r.view(k);
-    CUDA_CK(launch_combine(a, 1.0, x64, 0.0, null_field(), s));
+    load_natural(op, in, a, s);
     const bool f64 = op->prec == P64;
     if (which == 0) apply_M(op, a, b, false, f64, s);
     else if (which == 1) apply_M(op, a, b, true, f64, s);
@@ -1501,8 +1512,7 @@ eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int
         apply_M(op, a, c, false, f64, s);
         apply_M(op, c, b, true, f64, s);
     }
-    CUDA_CK(launch_combine(x64, 1.0, b, 0.0, null_field(), s));
-    store_natural(op, x64, out, s);
+    store_natural(op, b, out, s);
     sync(s);
     API_END
 }
@@ -1880,6 +1890,16 @@ eig_status eig_basis_deflate(eig_basis B, const double *b, const double *x_in, d
     ensure_workspace(op);
     cudaStream_t s = (cudaStream_t)stream;
     Field b64 = op->b64.view(k), x64 = op->x64.view(k), r64 = (op->prec == P64 ? op->r : op->r64).view(k);
+    if (!x_in && B->l > 0) {
+        // zero guess: the residual is b and the result is the correction itself, so both go
+        // straight between the natural layout and the basis precision
+        std::vector<cd> Yr;
+        load_natural(op, b, op->rsv.view(k), s);
+        deflate_core(B, k, Yr, s);
+        store_natural(op, op->xsv.view(k), x0, s);
+        sync(s);
+        return EIG_OK;
+    }
     load_natural(op, b, b64, s);
     if (x_in) {
         load_natural(op, x_in, x64, s);
