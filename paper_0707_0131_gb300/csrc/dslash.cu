@@ -23,6 +23,7 @@
 #include <mutex>
 #include <unordered_map>
 
+#include "dslash_split.cuh"
 #include "kernels.cuh"
 #include "prof.h"
 
@@ -290,51 +291,13 @@ __global__ void __launch_bounds__(128) k_dslash(const KArgs a) {
     double *const h_alpha = a.h_alpha, *const h_beta = a.h_beta, *const h_rho = a.h_rho;
     const int iter = a.iter + (a.jbase ? *a.jbase : 0), set_rho = a.set_rho;
     grid_reduce_rhs(bs, k, a.partials, a.counter, smem, [=](int r, double tot) {
-        CGScalars &st = sts[r];
-        const long hi = (long)iter * k + r;
-        if (EPI == EPI_NORM) {
-            if (st.active) {
-                st.pAp = tot;
-                if (!(tot > 0.0) || !isfinite(tot)) {
-                    st.breakdown = 1;
-                    st.active = 0;
-                    st.alpha = 0.0;
-                } else {
-                    st.alpha = st.rho / tot;
-                }
-                h_alpha[hi] = st.alpha;
-                st.x_pending = st.active;
-            } else {
-                st.alpha = 0.0;
-                st.x_pending = 0;
-            }
-        } else if (EPI == EPI_CG) {
-            if (st.active) {
-                if (!isfinite(tot)) {
-                    st.breakdown = 1;
-                    st.active = 0;
-                    return;
-                }
-                st.iters = iter;
-                st.nit++;
-                st.rho_prev = st.rho;
-                st.rho = tot;
-                st.beta = tot / st.rho_prev;
-                h_rho[hi] = tot;
-                h_beta[hi + k] = st.beta;
-                if (tot <= st.target) st.active = 0;
-            }
-        } else {  // EPI_RESID
-            st.aux = tot;
-            if (set_rho) {
-                st.rho = tot;
-                st.beta = tot / st.rho_prev;
-                h_rho[hi] = tot;
-                h_beta[hi + k] = st.beta;
-            }
-        }
+        finish_scalars<EPI>(sts, h_alpha, h_beta, h_rho, iter, k, set_rho, r, tot);
     });
 }
+
+static_assert((int)EPI_PLAIN == (int)SPL_PLAIN && (int)EPI_NORM == (int)SPL_NORM && (int)EPI_CG == (int)SPL_CG &&
+                  (int)EPI_RESID == (int)SPL_RESID,
+              "epilogue numbers shared with dslash_split.cuh");
 
 // ------------------------------------------------------------------------------------
 // launch plumbing
@@ -430,11 +393,49 @@ static std::string dslash_name(int epi, Prec p, int k) {
     return n;
 }
 
+// FP64 launches of n (site, RHS) pairs: spread the hops over lanes (dslash_split.cuh) while
+// the FP64 issue time of the fullest SM sub-partition is shorter that way.  One thread per
+// pair costs ~912 FP64 warp instructions per 32 pairs, the split form ~62 per 2 pairs; both
+// run in whole warps per sub-partition.
+static bool split64(long n) {
+    if (n > SPLIT_MAX) return false;
+    const long smsp = 4L * device_sm_count();
+    const long one = ((n + 31) / 32 + smsp - 1) / smsp * 912;
+    const long spl = ((n + 1) / 2 + smsp - 1) / smsp * 68;
+    return spl < one;
+}
+
+bool dslash_takes_natural(const DslashCall &c) {
+    return c.in.prec == P64 && c.eo_parity < 0 && split64(c.V * c.k);
+}
+
 template <int EPI>
 static cudaError_t dispatch(const DslashCall &c, KArgs &a, int cap, cudaStream_t s) {
     const long work = a.V * c.k;
     const int block = 128;
     ProfScope prof(dslash_name(EPI, c.in.prec, c.k).c_str(), dslash_bytes<EPI>(c, a), s);
+    if (c.in.prec == P64 && c.gformat == GF_F64_18 && split64(work)) {
+        SplitArgs b;
+        split_args(b, c);
+        if (EPI != EPI_PLAIN) {
+            History h;
+            h.alpha = a.h_alpha;
+            h.beta = a.h_beta;
+            h.rho = a.h_rho;
+            h.jbase = a.jbase;
+            RedScratch red;
+            red.partials = a.partials;
+            red.counter = a.counter;
+            split_reduction(b, a.st, h, a.iter, red);
+        }
+        b.r = a.r.data;
+        b.b = a.b.data;
+        b.tsave = a.tsave.data;
+        b.save_t = a.save_t;
+        b.set_rho = a.set_rho;
+        return split_launch<double, GF_F64_18, EPI>(c.dagger, b, cap, s);
+    }
+    if (c.nat_in || c.nat_out) return cudaErrorInvalidValue;
 #define EIG_LAUNCH(S, GF)                                                                   \
     do {                                                                                    \
         if (c.dagger) {                                                                     \

@@ -1,0 +1,393 @@
+// Internal header: the Wilson stencil with the hops of a site spread over lanes, for
+// launches with too few (site, RHS) pairs to fill the GPU one thread each.
+//
+// Same operator, layouts and epilogues as dslash.cu / dslash32.cuh.  There one thread
+// walks the eight hops of a site: on a small lattice that is one long serial chain on a
+// few SMs (4^4: two blocks; GB300 issues an FP64 warp instruction about every 64 cycles,
+// so the ~900 FP64 instructions of a site took 37 us with 150 SMs idle; in FP32 the chain
+// is eight dependent rounds of loads, 5-7 us).  Here 16 lanes share a (site, RHS): lane
+// 2 h + s forms spin component s of the half spinor of hop h (three colours), multiplies it
+// by the link and leaves the product in shared memory; lanes 0..11 then each sum one
+// complex component of the output over the eight hops and run the epilogue on it.  The
+// arithmetic per site is the same but for the reduction, about 31 FP64 warp instructions
+// per site against 28.5, so the one-thread form stays for lattices that fill the GPU.
+#pragma once
+#include <cstring>
+
+#include "fastdiv.h"
+#include "kernels.cuh"
+
+namespace eig {
+
+struct SplitArgs {
+    const void *in;
+    const float *in_s;
+    void *out;
+    float *out_s;
+    const void *cen;  // centre-term input (odd-even form), else in; null: hops only
+    const float *cen_s;
+    void *r;
+    float *r_s;
+    const void *b;    // residual epilogue
+    void *tsave;
+    const void *g;
+    // complex-component, site and RHS strides of in and out, in chunks (FP64: one complex
+    // per chunk, so the natural layout of the API can be read and written as it is)
+    unsigned in_c, in_x, in_r, out_c, out_x, out_r;
+    unsigned L0, L1, L2, L3, V, Vg, lh;
+    FastDiv d0, d1, d2, dh;
+    int eo;
+    unsigned k, kshift;
+    double diag, hcoef;
+    int save_t, set_rho;
+    CGScalars *st;
+    double *h_alpha, *h_beta, *h_rho;
+    int iter;
+    const int *jbase;
+    double *partials;
+    unsigned *counter;
+};
+
+// largest number of (site, RHS) pairs the split launchers take (32-bit offsets)
+constexpr long SPLIT_MAX = 1L << 20;
+
+// epilogues: the numbers of dslash.cu's Epi and dslash32.cuh's E_*
+enum { SPL_PLAIN = 0, SPL_NORM = 1, SPL_CG = 2, SPL_RESID = 3 };
+
+namespace {
+
+// the scalar updates of RHS r after a grid reduction gave tot (Fig. 1 steps 12, 4, 8; see
+// kernels.cuh for the launches they belong to)
+template <int EPI>
+__device__ __forceinline__ void finish_scalars(CGScalars *sts, double *h_alpha, double *h_beta, double *h_rho, int iter,
+                                               int k, int set_rho, int r, double tot) {
+    CGScalars &st = sts[r];
+    const long hi = (long)iter * k + r;
+    if (EPI == SPL_NORM) {
+        if (st.active) {
+            st.pAp = tot;
+            if (!(tot > 0.0) || !isfinite(tot)) {
+                st.breakdown = 1;
+                st.active = 0;
+                st.alpha = 0.0;
+            } else {
+                st.alpha = st.rho / tot;
+            }
+            h_alpha[hi] = st.alpha;
+            st.x_pending = st.active;
+        } else {
+            st.alpha = 0.0;
+            st.x_pending = 0;
+        }
+    } else if (EPI == SPL_CG) {
+        if (st.active) {
+            if (!isfinite(tot)) {
+                st.breakdown = 1;
+                st.active = 0;
+                return;
+            }
+            st.iters = iter;
+            st.nit++;
+            st.rho_prev = st.rho;
+            st.rho = tot;
+            st.beta = tot / st.rho_prev;
+            h_rho[hi] = tot;
+            h_beta[hi + k] = st.beta;
+            if (tot <= st.target) st.active = 0;
+        }
+    } else if (EPI == SPL_RESID) {
+        st.aux = tot;
+        if (set_rho) {
+            st.rho = tot;
+            st.beta = tot / st.rho_prev;
+            h_rho[hi] = tot;
+            h_beta[hi + k] = st.beta;
+        }
+    }
+}
+
+// one complex component e of the spinor at (site, RHS) offset o = site stride * site + RHS
+// stride * RHS (in chunks), chunk stride cs
+template <typename S>
+struct Comp;
+template <>
+struct Comp<double> {
+    using C = double;
+    __device__ static __forceinline__ Cx<double> load(const void *p, const float *, unsigned cs, unsigned o, int e) {
+        const double2 d = static_cast<const double2 *>(p)[(unsigned)e * cs + o];
+        return cmk<double>(d.x, d.y);
+    }
+    __device__ static __forceinline__ void store(void *p, unsigned cs, unsigned o, int e, Cx<double> z) {
+        static_cast<double2 *>(p)[(unsigned)e * cs + o] = make_double2(z.re, z.im);
+    }
+};
+template <>
+struct Comp<float> {
+    using C = float;
+    __device__ static __forceinline__ Cx<float> load(const void *p, const float *, unsigned cs, unsigned o, int e) {
+        const float2 d = static_cast<const float2 *>(p)[((unsigned)(e >> 1) * cs + o) * 2 + (e & 1)];
+        return cmk<float>(d.x, d.y);
+    }
+    __device__ static __forceinline__ void store(void *p, unsigned cs, unsigned o, int e, Cx<float> z) {
+        static_cast<float2 *>(p)[((unsigned)(e >> 1) * cs + o) * 2 + (e & 1)] = make_float2(z.re, z.im);
+    }
+};
+template <>
+struct Comp<__half> {
+    using C = float;
+    __device__ static __forceinline__ Cx<float> load(const void *p, const float *sc, unsigned cs, unsigned o, int e) {
+        const float2 d = __half22float2(static_cast<const __half2 *>(p)[((unsigned)(e >> 2) * cs + o) * 4 + (e & 3)]);
+        const float s = sc[o];
+        return cmk<float>(d.x * s, d.y * s);
+    }
+};
+
+// the rows of the link this lane multiplies by: u[a][b] = U[a][b] (bwd = false) or
+// conj(U[b][a]) (bwd = true)
+template <int GF, typename C>
+__device__ __forceinline__ void load_link_for(const void *g, unsigned Vg, int mu, unsigned s, bool bwd, Cx<C> (&u)[3][3]) {
+    GaugeView gv;
+    gv.data = g;
+    gv.V = Vg;
+    Link<C> U;
+    GaugeLoad<GF>::load(gv, mu, s, U);
+#pragma unroll
+    for (int a = 0; a < 3; a++)
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            u[a][b].re = bwd ? U.u[b][a].re : U.u[a][b].re;
+            u[a][b].im = bwd ? -U.u[b][a].im : U.u[a][b].im;
+        }
+}
+
+template <typename S, int GF, bool DAG, int EPI>
+__global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
+    using C = typename Comp<S>::C;
+    constexpr int SF = DAG ? +1 : -1;  // forward projector I + SF g_mu, backward I - SF g_mu
+    __shared__ Cx<C> prod[8][8][2][3];  // [group][hop][spin][colour]
+    __shared__ double smem[(128 / 32) * MAX_RHS];
+    __shared__ double gsum[8];
+    if (EPI == SPL_NORM || EPI == SPL_CG) {
+        bool any = false;
+        for (unsigned q = 0; q < a.k; q++) any = any || a.st[q].active;
+        if (!any) return;
+    }
+    const int t = threadIdx.x, grp = t >> 4, l = t & 15;
+    const int hop = l >> 1, sp = l & 1, mu = hop >> 1;
+    const bool bwd = hop & 1;
+    const unsigned total = a.V << a.kshift, step = gridDim.x * (blockDim.x >> 4);
+    const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2;
+    // this lane's projection h = a_sp + ph B: partner spin of the lower pair, factor +-1 or +-i
+    const int part = mu <= 1 ? 1 - sp : sp;
+    const bool img = mu == 0 || mu == 2;
+    const bool neg = ((mu == 1 && sp == 0) || (mu == 2 && sp == 1)) != ((bwd ? -SF : SF) < 0);
+    const C sre = (neg != img) ? (C)-1 : (C)1, sim = neg ? (C)-1 : (C)1;
+    double nrm = 0.0;
+    const unsigned niter = (total + step - 1) / step;
+    for (unsigned it = 0; it < niter; it++) {
+        const unsigned g = it * step + blockIdx.x * (blockDim.x >> 4) + grp;
+        const bool live = g < total;  // uniform over a group, not over a warp
+        const unsigned s = live ? g >> a.kshift : 0u, r = g & (a.k - 1);
+        unsigned x, y, z, tt, sl;
+        if (a.eo >= 0) {
+            const unsigned rest = a.lh > 1 ? fastdiv(s, a.dh) : s, q2 = fastdiv(rest, a.d1);
+            tt = fastdiv(q2, a.d2);
+            y = rest - q2 * a.L1;
+            z = q2 - tt * a.L2;
+            x = 2 * (s - rest * a.lh) + ((a.eo + y + z + tt) & 1);
+            sl = x + rest * a.L0;
+        } else {
+            const unsigned q1 = fastdiv(s, a.d0), q2 = fastdiv(q1, a.d1);
+            tt = fastdiv(q2, a.d2);
+            x = s - q1 * a.L0;
+            y = q1 - q2 * a.L1;
+            z = q2 - tt * a.L2;
+            sl = s;
+        }
+        const unsigned cm = mu == 0 ? x : (mu == 1 ? y : (mu == 2 ? z : tt));
+        const unsigned Lm = mu == 0 ? a.L0 : (mu == 1 ? a.L1 : (mu == 2 ? a.L2 : a.L3));
+        const unsigned sm = mu == 0 ? 1u : (mu == 1 ? s1 : (mu == 2 ? s2 : s3));
+        const unsigned nl = bwd ? (cm == 0 ? sl + (Lm - 1) * sm : sl - sm)
+                                : (cm == Lm - 1 ? sl - (Lm - 1) * sm : sl + sm);
+        const unsigned nf = a.eo >= 0 ? nl >> 1 : nl;  // field index of the neighbour
+        const unsigned oin = nf * a.in_x + r * a.in_r;
+        const unsigned oc = s * a.in_x + r * a.in_r, oo = s * a.out_x + r * a.out_r;
+        Cx<C> c0 = cmk<C>(0, 0), e0 = cmk<C>(0, 0);
+        if (live) {
+            Cx<C> h[3], u[3][3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) h[c] = Comp<S>::load(a.in, a.in_s, a.in_c, oin, sp * 3 + c);
+            Cx<C> q[3];
+#pragma unroll
+            for (int c = 0; c < 3; c++) q[c] = Comp<S>::load(a.in, a.in_s, a.in_c, oin, 6 + part * 3 + c);
+            load_link_for<GF>(a.g, a.Vg, mu, bwd ? nl : sl, bwd, u);
+            if (l < 12) {  // the centre and the epilogue's operand, in flight with the hops
+                if (a.cen) c0 = Comp<S>::load(a.cen, a.cen_s, a.in_c, oc, l);
+                if (EPI == SPL_CG) e0 = Comp<S>::load(a.r, a.r_s, a.out_c, oo, l);
+                if (EPI == SPL_RESID) e0 = Comp<S>::load(a.b, nullptr, a.out_c, oo, l);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                h[c].re = fma(sre, img ? q[c].im : q[c].re, h[c].re);
+                h[c].im = fma(sim, img ? q[c].re : q[c].im, h[c].im);
+            }
+#pragma unroll
+            for (int i = 0; i < 3; i++) {
+                Cx<C> v = cmul(u[i][0], h[0]);
+                v = cfma(u[i][1], h[1], v);
+                v = cfma(u[i][2], h[2], v);
+                prod[grp][hop][sp][i] = v;
+            }
+        }
+        __syncwarp();
+        Cx<C> o = cmk<C>(0, 0);
+        if (l < 12 && live) {
+            const int so = l / 3, c = l - 3 * so, lo = so & 1;
+            Cx<C> acc = cmk<C>(0, 0);
+#pragma unroll
+            for (int hh = 0; hh < 8; hh++) {
+                constexpr int SFc = SF;
+                const int m = hh >> 1, sg = (hh & 1) ? -SFc : SFc;
+                // upper spins take the product, lower spins sg B_mu^H of it
+                const int from = so < 2 ? lo : (m <= 1 ? 1 - lo : lo);
+                const Cx<C> w = prod[grp][hh][from][c];
+                const bool im = so >= 2 && (m == 0 || m == 2);
+                bool ng = false;
+                if (so >= 2) ng = ((m == 0) || (m == 1 && lo == 1) || (m == 2 && lo == 0)) != (sg < 0);
+                // factor (-1)^ng, times i where im
+                const C fr = (ng != im) ? (C)-1 : (C)1, fi = ng ? (C)-1 : (C)1;
+                acc.re = fma(fr, im ? w.im : w.re, acc.re);
+                acc.im = fma(fi, im ? w.re : w.im, acc.im);
+            }
+            const C d = (C)a.diag, hc = (C)a.hcoef;
+            o = cmk<C>(d * c0.re + hc * acc.re, d * c0.im + hc * acc.im);
+            if (EPI == SPL_RESID) o = e0 - o;
+        }
+        __syncwarp();
+        if (EPI == SPL_CG) {
+            const CGScalars &st = a.st[r];
+            const C al = st.active ? (C)st.alpha : (C)0;
+            const Cx<C> tv = o;
+            o = cmk<C>(e0.re - al * tv.re, e0.im - al * tv.im);
+            if (live && l < 12 && a.save_t) {  // single RHS, window precision
+                using W = typename Comp<S>::C;
+                Comp<W>::store(a.tsave, a.V, s, l, tv);
+            }
+        }
+        // the store of half-precision fields is collective over the warp: every lane takes part
+        if constexpr (sizeof(S) == 2) {
+            void *dst = EPI == SPL_CG ? a.r : a.out;
+            float *dsc = EPI == SPL_CG ? a.r_s : a.out_s;
+            float mx = (live && l < 12) ? fmaxf(fabsf(o.re), fabsf(o.im)) : 0.f;
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+            const float inv = mx > 0.f ? 1.0f / mx : 0.f;
+            if (live && l < 12)
+                static_cast<__half2 *>(dst)[((unsigned)(l >> 2) * a.out_c + oo) * 4 + (l & 3)] =
+                    __floats2half2_rn(o.re * inv, o.im * inv);
+            if (live && l == 0) dsc[oo] = mx;
+        } else {
+            if (live && l < 12) Comp<S>::store(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
+        }
+        if (EPI != SPL_PLAIN) {
+            C n = (live && l < 12) ? o.re * o.re + o.im * o.im : (C)0;
+#pragma unroll
+            for (int off = 8; off > 0; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
+            nrm += (double)n;  // the same in the 16 lanes; a group's RHS is the same in every pass
+        }
+    }
+    if (EPI == SPL_PLAIN) return;
+    const int ngrp = blockDim.x >> 4, k = (int)a.k;
+    if (l == 0) gsum[grp] = nrm;
+    __syncthreads();
+    if (t < k) {
+        double v = 0.0;
+        for (int q = 0; q < ngrp; q++)
+            if (((blockIdx.x * ngrp + q) & (k - 1)) == t) v += gsum[q];
+        a.partials[(long)blockIdx.x * k + t] = v;
+    }
+    CGScalars *const sts = a.st;
+    double *const h_alpha = a.h_alpha, *const h_beta = a.h_beta, *const h_rho = a.h_rho;
+    const int iter = a.iter + (a.jbase ? *a.jbase : 0), set_rho = a.set_rho;
+    grid_finish_rhs(k, a.partials, a.counter, smem, [=](int rr, double tot) {
+        finish_scalars<EPI>(sts, h_alpha, h_beta, h_rho, iter, k, set_rho, rr, tot);
+    });
+}
+
+inline void split_args(SplitArgs &a, const DslashCall &c) {
+    memset(&a, 0, sizeof(a));
+    a.in = c.in.v.data;
+    a.in_s = c.in.v.scale;
+    a.out = c.out.v.data;
+    a.out_s = c.out.v.scale;
+    a.g = c.gauge.data;
+    a.L0 = c.L[0];
+    a.L1 = c.L[1];
+    a.L2 = c.L[2];
+    a.L3 = c.L[3];
+    a.d0 = fastdiv_make(a.L0);
+    a.d1 = fastdiv_make(a.L1);
+    a.d2 = fastdiv_make(a.L2);
+    a.lh = a.L0 / 2;
+    if (a.lh >= 2) a.dh = fastdiv_make(a.lh);
+    a.Vg = (unsigned)c.V;
+    a.eo = c.eo_parity;
+    a.V = (unsigned)(c.eo_parity >= 0 ? c.V / 2 : c.V);
+    a.k = (unsigned)c.k;
+    while ((1u << a.kshift) < a.k) a.kshift++;
+    a.in_c = a.out_c = a.V * a.k;
+    a.in_x = a.out_x = a.k;
+    a.in_r = a.out_r = 1;
+    if (c.nat_in) {  // [rhs][site][component]
+        a.in_c = 1;
+        a.in_x = 12;
+        a.in_r = 12 * a.V;
+    }
+    if (c.nat_out) {
+        a.out_c = 1;
+        a.out_x = 12;
+        a.out_r = 12 * a.V;
+    }
+    a.cen = c.in.v.data;
+    a.cen_s = c.in.v.scale;
+    if (c.eo_parity >= 0) {
+        a.cen = c.cen.v.data;
+        a.cen_s = c.cen.v.scale;
+    }
+    a.diag = c.diag;
+    a.hcoef = c.hcoef;
+}
+
+inline void split_reduction(SplitArgs &a, CGScalars *st, const History &h, int iter, const RedScratch &red) {
+    a.st = st;
+    a.h_alpha = h.alpha;
+    a.h_beta = h.beta;
+    a.h_rho = h.rho;
+    a.iter = iter;
+    a.jbase = h.jbase;
+    a.partials = red.partials;
+    a.counter = red.counter;
+}
+
+// Blocks of one warp while there are fewer warps than SMs (each then has an SM's FP64 units
+// or L1 to itself), of four otherwise; 16 resident warps per SM at most, and a multiple of 16
+// blocks when a block makes several passes, so that a group keeps its RHS from pass to pass.
+template <typename S, int GF, int EPI>
+cudaError_t split_launch(bool dag, const SplitArgs &a, int cap, cudaStream_t s) {
+    const long groups = (long)a.V << a.kshift, warps = (groups + 1) / 2;
+    if (groups > SPLIT_MAX || a.k > (unsigned)MAX_RHS) return cudaErrorInvalidValue;
+    const int sms = device_sm_count();
+    const int tpb = warps <= sms ? 32 : (warps <= 2L * sms ? 64 : 128);
+    const long need = (groups + tpb / 16 - 1) / (tpb / 16);
+    long most = (long)sms * (2048 / tpb) / 4;
+    if (cap > 0 && most > cap) most = cap;
+    long grid = need;
+    if (grid > most) grid = most / 16 * 16;
+    if (grid < 1) grid = need < 16 ? need : 16;
+    if (dag) k_dslash_split<S, GF, true, EPI><<<(int)grid, tpb, 0, s>>>(a);
+    else k_dslash_split<S, GF, false, EPI><<<(int)grid, tpb, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace eig

@@ -445,6 +445,31 @@ static void store_natural(eig_op_s *op, Field src, double *nat, cudaStream_t s) 
     }
 }
 
+// out = M in, M^H in or A in (which 0..2) for natural-layout device vectors where the FP64
+// stencil reads and writes that layout itself (small lattices): no packing launches.  False
+// if the call does not qualify (host vectors; for one product, overlapping vectors).
+static bool apply_natural(eig_op_s *op, int which, const double *in, double *out, int k, cudaStream_t s) {
+    Field src = op->p.view(k), mid = op->r.view(k), dst = op->u.view(k);
+    src.v.data = const_cast<double *>(in);
+    dst.v.data = out;
+    DslashCall c = op->call(src, dst, which == 1, true);
+    c.nat_in = c.nat_out = true;
+    if (!dslash_takes_natural(c) || !is_device_ptr(in) || !is_device_ptr(out)) return false;
+    if (((uintptr_t)in | (uintptr_t)out) & 15) return false;
+    const char *a = (const char *)in, *b = (const char *)out;
+    const size_t n = (size_t)op->Vf * 12 * 16 * k;
+    if (which <= 1) {
+        if (a < b + n && b < a + n) return false;  // neighbours are read while others are written
+        CUDA_CK(launch_dslash(c, s));
+        return true;
+    }
+    DslashCall c1 = op->call(src, mid, false, true), c2 = op->call(mid, dst, true, true);
+    c1.nat_in = c2.nat_out = true;
+    CUDA_CK(launch_dslash(c1, s));
+    CUDA_CK(launch_dslash(c2, s));
+    return true;
+}
+
 // Loads b and the initial guess x (k RHS) of a solve.  Full-lattice operators: into
 // b64 / x64.  Odd-even operators: b and x are full-lattice vectors of M x = b; b64
 // receives M_hat^H b_hat with b_hat = b_o - (1/d) H_oe b_e, the right-hand side of the
@@ -1504,8 +1529,12 @@ eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int
     // the vectors go straight between the natural layout and the op's storage precision (the
     // same roundings as through an FP64 field, without its passes over memory)
     Field a = op->p.view(k), b = op->u.view(k), c = op->r.view(k);
-    load_natural(op, in, a, s);
     const bool f64 = op->prec == P64;
+    if (f64 && !op->eo && apply_natural(op, which, in, out, k, s)) {
+        sync(s);
+        return EIG_OK;
+    }
+    load_natural(op, in, a, s);
     if (which == 0) apply_M(op, a, b, false, f64, s);
     else if (which == 1) apply_M(op, a, b, true, f64, s);
     else {

@@ -88,7 +88,13 @@ struct DslashCall {
     int eo_parity = -1;
     Field cen;
     double hcoef = -0.5;
+    // in / out in the natural layout [rhs][site][12] of the API instead of the internal one:
+    // only for calls dslash_takes_natural() accepts, with in and out disjoint
+    bool nat_in = false, nat_out = false;
 };
+// True if launch_dslash reads and writes the natural layout for this FP64 call (small
+// lattices, where the stencil spreads a site's hops over lanes).
+bool dslash_takes_natural(const DslashCall &c);
 
 // ---------------------------- dslash.cu ----------------------------------------------
 // out = M in (dagger: M^H in)
