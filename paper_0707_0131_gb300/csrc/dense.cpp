@@ -77,69 +77,84 @@ void herm_tridiag(int n, cd *A, double *d, double *e, cd *Q) {
         for (int j = 0; j < n; j++) Q[r * n + j] *= phi[j];
 }
 
-// number of eigenvalues of (d, e) smaller than x
-static int sturm_count(int n, const double *d, const double *e2, double x, double pivmin) {
-    int cnt = 0;
-    double q = d[0] - x;
-    if (std::fabs(q) < pivmin) q = -pivmin;
-    if (q < 0) cnt++;
-    for (int i = 1; i < n; i++) {
-        q = d[i] - x - e2[i - 1] / q;
-        if (std::fabs(q) < pivmin) q = -pivmin;
-        if (q < 0) cnt++;
+// Numbers of eigenvalues of (d, e) smaller than each of LANES shifts x.  A Sturm sequence is
+// one serial chain of divisions; LANES chains run side by side, so that their latencies
+// overlap and the compiler vectorises across them (the counts of each are those of a chain
+// run alone).
+static const int LANES = 8;
+static void sturm_counts(int n, const double *d, const double *e2, const double *x, double pivmin, long *cnt) {
+    double q[LANES];
+    for (int c = 0; c < LANES; c++) {
+        const double t = d[0] - x[c];
+        q[c] = std::fabs(t) < pivmin ? -pivmin : t;
+        cnt[c] = q[c] < 0 ? 1 : 0;
     }
-    return cnt;
+    for (int i = 1; i < n; i++) {
+        const double di = d[i], ei = e2[i - 1];
+        for (int c = 0; c < LANES; c++) {
+            const double t = di - x[c] - ei / q[c];
+            q[c] = std::fabs(t) < pivmin ? -pivmin : t;
+            cnt[c] += q[c] < 0 ? 1 : 0;
+        }
+    }
 }
 
-// Solves (T - lambda I) y = y in place with a partially pivoted LU of the tridiagonal.
-// Pivots smaller than pivmin (eps * ||T||) are replaced by +-pivmin: the shift is an
-// eigenvalue to rounding, so exact singularity is expected and harmless.
-static void tridiag_shift_solve(int n, const double *d, const double *e, double lambda, double pivmin,
-                                std::vector<double> &y) {
-    std::vector<double> a(n), b(n > 1 ? n - 1 : 1), c(n > 1 ? n - 1 : 1), u2(n > 2 ? n - 2 : 1);
-    std::vector<int> swp(n > 1 ? n - 1 : 1);
-    for (int i = 0; i < n; i++) a[i] = d[i] - lambda;
-    for (int i = 0; i + 1 < n; i++) b[i] = c[i] = e[i];
-    for (int i = 0; i + 1 < n; i++) {
-        if (std::fabs(a[i]) >= std::fabs(c[i])) {
-            if (std::fabs(a[i]) < pivmin) a[i] = a[i] < 0 ? -pivmin : pivmin;
-            const double mult = c[i] / a[i];
-            c[i] = mult;
-            a[i + 1] -= mult * b[i];
-            if (i + 2 < n) u2[i] = 0.0;
-            swp[i] = 0;
-        } else {
-            const double mult = a[i] / c[i];
-            a[i] = c[i];
-            const double tmp = a[i + 1];
-            a[i + 1] = b[i] - mult * tmp;
-            if (i + 2 < n) {
-                u2[i] = b[i + 1];
-                b[i + 1] = -mult * b[i + 1];
+// Partially pivoted LU of the tridiagonal T - lambda I, and its solves.  Pivots smaller than
+// pivmin (eps * ||T||) are replaced by +-pivmin: the shift is an eigenvalue to rounding, so
+// exact singularity is expected and harmless.
+struct TridiagLU {
+    int n;
+    std::vector<double> a, b, c, u2;  // diagonal, super diagonal, multipliers, second super
+    std::vector<char> swp;
+    explicit TridiagLU(int n_) : n(n_), a(n_), b(n_), c(n_), u2(n_), swp(n_) {}
+
+    void factor(const double *d, const double *e, double lambda, double pivmin) {
+        for (int i = 0; i < n; i++) a[i] = d[i] - lambda;
+        for (int i = 0; i + 1 < n; i++) b[i] = c[i] = e[i];
+        for (int i = 0; i + 1 < n; i++) {
+            if (std::fabs(a[i]) >= std::fabs(c[i])) {
+                if (std::fabs(a[i]) < pivmin) a[i] = a[i] < 0 ? -pivmin : pivmin;
+                const double mult = c[i] / a[i];
+                c[i] = mult;
+                a[i + 1] -= mult * b[i];
+                if (i + 2 < n) u2[i] = 0.0;
+                swp[i] = 0;
+            } else {
+                const double mult = a[i] / c[i];
+                a[i] = c[i];
+                const double tmp = a[i + 1];
+                a[i + 1] = b[i] - mult * tmp;
+                if (i + 2 < n) {
+                    u2[i] = b[i + 1];
+                    b[i + 1] = -mult * b[i + 1];
+                }
+                b[i] = tmp;
+                c[i] = mult;
+                swp[i] = 1;
             }
-            b[i] = tmp;
-            c[i] = mult;
-            swp[i] = 1;
         }
+        if (a[n - 1] == 0.0) a[n - 1] = pivmin;
+        for (int i = 0; i < n; i++)
+            if (std::fabs(a[i]) < pivmin) a[i] = a[i] < 0 ? -pivmin : pivmin;
     }
-    if (a[n - 1] == 0.0) a[n - 1] = pivmin;
-    for (int i = 0; i < n; i++)
-        if (std::fabs(a[i]) < pivmin) a[i] = a[i] < 0 ? -pivmin : pivmin;
-    // forward: L
-    for (int i = 0; i + 1 < n; i++) {
-        if (!swp[i]) {
-            y[i + 1] -= c[i] * y[i];
-        } else {
-            const double t = y[i];
-            y[i] = y[i + 1];
-            y[i + 1] = t - c[i] * y[i];
+
+    void solve(std::vector<double> &y) const {
+        // forward: L
+        for (int i = 0; i + 1 < n; i++) {
+            if (!swp[i]) {
+                y[i + 1] -= c[i] * y[i];
+            } else {
+                const double t = y[i];
+                y[i] = y[i + 1];
+                y[i + 1] = t - c[i] * y[i];
+            }
         }
+        // backward: U
+        y[n - 1] /= a[n - 1];
+        if (n > 1) y[n - 2] = (y[n - 2] - b[n - 2] * y[n - 1]) / a[n - 2];
+        for (int i = n - 3; i >= 0; i--) y[i] = (y[i] - b[i] * y[i + 1] - u2[i] * y[i + 2]) / a[i];
     }
-    // backward: U (diagonal a, super b, second super u2)
-    y[n - 1] /= a[n - 1];
-    if (n > 1) y[n - 2] = (y[n - 2] - b[n - 2] * y[n - 1]) / a[n - 2];
-    for (int i = n - 3; i >= 0; i--) y[i] = (y[i] - b[i] * y[i + 1] - u2[i] * y[i + 2]) / a[i];
-}
+};
 
 void tridiag_eig(int n, const double *d, const double *e, int lo, int hi, double *w, double *Z) {
     if (hi <= lo) return;
@@ -164,24 +179,41 @@ void tridiag_eig(int n, const double *d, const double *e, int lo, int hi, double
     const double pivmin = std::max(std::numeric_limits<double>::min(), tnorm * 1e-300 + std::numeric_limits<double>::min() * emax);
     gl -= 2.0 * EPS * tnorm * n + pivmin;
     gu += 2.0 * EPS * tnorm * n + pivmin;
-    // eigenvalues by bisection
-    for (int idx = lo; idx < hi; idx++) {
-        double a = gl, b = gu;
-        for (int it = 0; it < 200; it++) {
-            const double mid = 0.5 * (a + b);
-            if (b - a <= 2.0 * EPS * std::max(std::fabs(a), std::fabs(b)) + 4.0 * pivmin) break;
-            if (mid <= a || mid >= b) break;
-            if (sturm_count(n, d, e2.data(), mid, pivmin) > idx)
-                b = mid;
-            else
-                a = mid;
+    // eigenvalues by bisection, LANES of them in step
+    for (int i0 = lo; i0 < hi; i0 += LANES) {
+        const int nl = std::min(LANES, hi - i0);
+        double a[LANES], b[LANES], mid[LANES];
+        bool run[LANES];
+        long cnt[LANES];
+        for (int c = 0; c < LANES; c++) {
+            a[c] = gl;
+            b[c] = gu;
+            run[c] = c < nl;
         }
-        w[idx - lo] = 0.5 * (a + b);
+        for (int it = 0; it < 200; it++) {
+            bool any = false;
+            for (int c = 0; c < LANES; c++) {
+                mid[c] = 0.5 * (a[c] + b[c]);
+                if (run[c] && (b[c] - a[c] <= 2.0 * EPS * std::max(std::fabs(a[c]), std::fabs(b[c])) + 4.0 * pivmin ||
+                               mid[c] <= a[c] || mid[c] >= b[c]))
+                    run[c] = false;
+                any = any || run[c];
+            }
+            if (!any) break;
+            sturm_counts(n, d, e2.data(), mid, pivmin, cnt);
+            for (int c = 0; c < nl; c++) {
+                if (!run[c]) continue;
+                if (cnt[c] > i0 + c) b[c] = mid[c];
+                else a[c] = mid[c];
+            }
+        }
+        for (int c = 0; c < nl; c++) w[i0 + c - lo] = 0.5 * (a[c] + b[c]);
     }
     // eigenvectors by inverse iteration; re-orthogonalise within clusters
     const double ortol = 1e-3 * tnorm;
     const double sep = 10.0 * EPS * tnorm;
     std::vector<double> y(n);
+    TridiagLU lu(n);
     int cluster_start = 0;
     double lam_prev = 0.0;
     for (int q = 0; q < hi - lo; q++) {
@@ -192,12 +224,13 @@ void tridiag_eig(int n, const double *d, const double *e, int lo, int hi, double
         }
         lam_prev = lam;
         for (int i = 0; i < n; i++) y[i] = 1.0 + 0.5 * std::sin(0.7 * (i + 1) + 1.3 * (q + 1));
+        lu.factor(d, e, lam, std::max(pivmin, EPS * tnorm));
         for (int it = 0; it < 4; it++) {
             // scale to avoid overflow
             double mx = 0.0;
             for (int i = 0; i < n; i++) mx = std::max(mx, std::fabs(y[i]));
             if (mx > 0) for (int i = 0; i < n; i++) y[i] /= mx;
-            tridiag_shift_solve(n, d, e, lam, std::max(pivmin, EPS * tnorm), y);
+            lu.solve(y);
             for (int p = cluster_start; p < q; p++) {
                 const double *zp = Z + (size_t)p * n;
                 double dot = 0.0;
@@ -328,12 +361,17 @@ int restart_coefficients(int m, const cd *T, int kh, int nev, double drop_tol, c
     const int r = orth_columns(m, 2 * nev, X.data(), drop_tol, nullptr);
     // H = Q^H T Q
     std::vector<cd> TQ((size_t)m * r), H((size_t)r * r);
-    for (int c = 0; c < r; c++)
-        for (int i = 0; i < m; i++) {
+    std::vector<int> nz;  // a row of T has at most kh + 3 entries (diagonal head, arrow, tridiagonal tail)
+    for (int i = 0; i < m; i++) {
+        nz.clear();
+        for (int j = 0; j < m; j++)
+            if (T[(size_t)i * m + j] != 0.0) nz.push_back(j);
+        for (int c = 0; c < r; c++) {
             cd s = 0.0;
-            for (int j = 0; j < m; j++) s += T[(size_t)i * m + j] * X[(size_t)c * m + j];
+            for (int j : nz) s += T[(size_t)i * m + j] * X[(size_t)c * m + j];
             TQ[(size_t)c * m + i] = s;
         }
+    }
     for (int a = 0; a < r; a++)
         for (int b = 0; b < r; b++) {
             cd s = 0.0;
@@ -376,19 +414,53 @@ bool cholesky(int n, cd *L) {
     return true;
 }
 
+// One RHS is a serial chain of complex multiply-subtracts; the RHS are taken CB at a time,
+// their entries side by side, so that CB chains advance together (each in the order it has
+// alone).
 void chol_solve(int n, const cd *L, cd *B, int nrhs) {
-    for (int c = 0; c < nrhs; c++) {
-        cd *b = B + (size_t)c * n;
+    const int CB = 8;
+    std::vector<double> re((size_t)n * CB), im((size_t)n * CB);
+    for (int c0 = 0; c0 < nrhs; c0 += CB) {
+        const int nc = std::min(CB, nrhs - c0);
+        for (int i = 0; i < n; i++)
+            for (int c = 0; c < CB; c++) {
+                const cd v = c < nc ? B[(size_t)(c0 + c) * n + i] : cd(0.0);
+                re[(size_t)i * CB + c] = v.real();
+                im[(size_t)i * CB + c] = v.imag();
+            }
+        double sr[CB], si[CB];
+        auto sub = [&](double lr, double li, int k) {  // s -= l * b_k
+            const double *br = &re[(size_t)k * CB], *bi = &im[(size_t)k * CB];
+            for (int c = 0; c < CB; c++) {
+                sr[c] -= lr * br[c] - li * bi[c];
+                si[c] -= lr * bi[c] + li * br[c];
+            }
+        };
+        auto load = [&](int i) {
+            for (int c = 0; c < CB; c++) {
+                sr[c] = re[(size_t)i * CB + c];
+                si[c] = im[(size_t)i * CB + c];
+            }
+        };
+        auto scale = [&](int i) {
+            const double dd = L[(size_t)i * n + i].real();
+            for (int c = 0; c < CB; c++) {
+                re[(size_t)i * CB + c] = sr[c] / dd;
+                im[(size_t)i * CB + c] = si[c] / dd;
+            }
+        };
         for (int i = 0; i < n; i++) {
-            cd s = b[i];
-            for (int k = 0; k < i; k++) s -= L[(size_t)i * n + k] * b[k];
-            b[i] = s / L[(size_t)i * n + i].real();
+            load(i);
+            for (int k = 0; k < i; k++) sub(L[(size_t)i * n + k].real(), L[(size_t)i * n + k].imag(), k);
+            scale(i);
         }
         for (int i = n - 1; i >= 0; i--) {
-            cd s = b[i];
-            for (int k = i + 1; k < n; k++) s -= std::conj(L[(size_t)k * n + i]) * b[k];
-            b[i] = s / L[(size_t)i * n + i].real();
+            load(i);
+            for (int k = i + 1; k < n; k++) sub(L[(size_t)k * n + i].real(), -L[(size_t)k * n + i].imag(), k);
+            scale(i);
         }
+        for (int i = 0; i < n; i++)
+            for (int c = 0; c < nc; c++) B[(size_t)(c0 + c) * n + i] = cd(re[(size_t)i * CB + c], im[(size_t)i * CB + c]);
     }
 }
 
