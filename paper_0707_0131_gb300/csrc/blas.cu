@@ -445,6 +445,97 @@ cudaError_t launch_norm2(Field f, CGScalars *st, bool as_rho, History h, int ite
 // x += alpha p (pending from the previous iteration), p = r + beta p, window append
 // v = r / sqrt(rho).  x lives in the wide precision (FP64 for FP64 storage, else FP32).
 // ---------------------------------------------------------------------------------------
+// FP64 and FP32 fields (p, r, x and v of one precision): one 16-byte chunk per thread and
+// step, all streams in address order.  The per-RHS coefficients are formed once per block:
+// 1 / sqrt(rho) takes ~50 FP64 instructions of ~64 issue cycles per warp, which cost more
+// than the memory traffic when every thread did it (16^3x32, k = 1, with the append: 16.6 us
+// per launch).  gridDim x blockDim is a multiple of 16, so a thread keeps its RHS.
+constexpr int PU_THREADS = 256;
+
+__device__ __forceinline__ void chunk_axpy(float4 &y, float4 x, float a) {
+    y.x += a * x.x;
+    y.y += a * x.y;
+    y.z += a * x.z;
+    y.w += a * x.w;
+}
+__device__ __forceinline__ void chunk_axpy(double2 &y, double2 x, double a) {
+    y.x += a * x.x;
+    y.y += a * x.y;
+}
+__device__ __forceinline__ float4 chunk_scale(float4 x, float a) { return make_float4(x.x * a, x.y * a, x.z * a, x.w * a); }
+__device__ __forceinline__ double2 chunk_scale(double2 x, double a) { return make_double2(x.x * a, x.y * a); }
+
+template <typename V4, typename C>
+__global__ void __launch_bounds__(PU_THREADS) k_pupdate_flat(const V4 *r, V4 *p, V4 *x, size_t n, int k, int first,
+                                                             const CGScalars *st, V4 *v, int append,
+                                                             unsigned long long *dev_bytes) {
+    __shared__ C s_al[MAX_RHS], s_be[MAX_RHS], s_inv[MAX_RHS];
+    __shared__ int s_mode[MAX_RHS];  // 1: active, 2: x lacks alpha p
+    const int t = threadIdx.x;
+    int act = 0;
+    if (t < k) {
+        const CGScalars &sc = st[t];
+        act = sc.active;
+        s_mode[t] = (sc.active ? 1 : 0) | (sc.x_pending ? 2 : 0);
+        s_al[t] = (C)sc.alpha;
+        s_be[t] = (C)sc.beta;
+        if (append) s_inv[t] = (C)(1.0 / sqrt(sc.rho));
+    }
+    if (!__syncthreads_or(act)) return;
+    const int q = t & (k - 1), mode = s_mode[q];
+    // a RHS that has stopped while others in its batch go on keeps its p (and r, x)
+    // untouched, so that if the final residual check resumes it, it continues exactly as
+    // it would have alone
+    const bool active = mode & 1, pend = !first && (mode & 2), app = append && active;
+    const C al = s_al[q], be = s_be[q], inv = append ? s_inv[q] : (C)0;
+    unsigned chunks = 0;
+    if (first || active || pend) {
+        const size_t step = (size_t)gridDim.x * PU_THREADS;
+        for (size_t i = (size_t)blockIdx.x * PU_THREADS + t; i < n; i += 2 * step) {
+            const size_t j = i + step;
+            const bool two = j < n;
+            V4 pa, pb, ra, rb, xa, xb;
+            const bool need_r = first || active;
+            if (!first) {
+                pa = p[i];
+                if (two) pb = p[j];
+            }
+            if (need_r) {
+                ra = r[i];
+                if (two) rb = r[j];
+            }
+            if (pend) {  // Fig. 1 step 13 of the previous iteration
+                xa = x[i];
+                if (two) xb = x[j];
+                chunk_axpy(xa, pa, al);
+                x[i] = xa;
+                if (two) {
+                    chunk_axpy(xb, pb, al);
+                    x[j] = xb;
+                }
+            }
+            if (need_r) {
+                V4 na = ra, nb = rb;
+                if (!first) {
+                    chunk_axpy(na, pa, be);
+                    if (two) chunk_axpy(nb, pb, be);
+                }
+                p[i] = na;
+                if (two) p[j] = nb;
+                if (app) {
+                    v[i] = chunk_scale(ra, inv);
+                    if (two) v[j] = chunk_scale(rb, inv);
+                }
+            }
+            chunks += (two ? 2u : 1u) * ((first ? 2u : 1u) + (pend ? 2u : 0u) + (!first && need_r ? 2u : 0u) + (app ? 1u : 0u));
+        }
+    }
+    if (dev_bytes) {
+        const unsigned w = __reduce_add_sync(0xffffffffu, chunks * 16u);
+        if ((t & 31) == 0 && w) atomicAdd(dev_bytes, (unsigned long long)w);
+    }
+}
+
 template <typename S, typename SV>
 __global__ void k_pupdate(FieldView r, FieldView p, FieldView x, int first, const CGScalars *st, FieldView v,
                           int append, unsigned long long *dev_bytes) {
@@ -454,6 +545,11 @@ __global__ void k_pupdate(FieldView r, FieldView p, FieldView x, int first, cons
         bool any = false;
         for (int q = 0; q < r.k; q++) any = any || st[q].active;
         if (!any) return;
+    }
+    __shared__ CV s_inv;  // 1 / sqrt(rho) of the appended vector (one RHS), formed once per block
+    if (append) {
+        if (threadIdx.x == 0) s_inv = (CV)(1.0 / sqrt(st[0].rho));
+        __syncthreads();
     }
     constexpr unsigned SB = SpinorStore<S>::BYTES, SBV = SpinorStore<SV>::BYTES;
     unsigned moved = 0;  // bytes this thread read and wrote
@@ -501,7 +597,7 @@ __global__ void k_pupdate(FieldView r, FieldView p, FieldView x, int first, cons
         SpinorStore<S>::store(p, s, q, pp);
         moved += SB;
         if (append && sc.active) {
-            const CV sc_inv = (CV)(1.0 / sqrt(sc.rho));
+            const CV sc_inv = s_inv;
             Spinor<CV> vv;
 #pragma unroll
             for (int i = 0; i < 4; i++)
@@ -529,23 +625,26 @@ cudaError_t launch_pupdate(Field r, Field p, Field x, bool first, CGScalars *st,
                         : (double)r.v.V * r.v.k * ((first ? 2.0 : 3.0) * spb(r.prec) + (first ? 0.0 : 2.0 * spb(x.prec))) +
                               (app ? (double)r.v.V * spb(v_append.prec) : 0.0),
                    s);
-    const int B = 128;
-    const int G = stream_grid(r.v.V * r.v.k, B);
     if (app && v_append.prec != x.prec) return cudaErrorInvalidValue;
-    switch (r.prec) {
-        case P64:
-            if (x.prec != P64) return cudaErrorInvalidValue;
-            k_pupdate<double, double><<<G, B, 0, s>>>(r.v, p.v, x.v, first, st, v_append.v, app, devb);
-            break;
-        case P32:
-            if (x.prec != P32) return cudaErrorInvalidValue;
-            k_pupdate<float, float><<<G, B, 0, s>>>(r.v, p.v, x.v, first, st, v_append.v, app, devb);
-            break;
-        case P16:
-            if (x.prec != P32) return cudaErrorInvalidValue;
-            k_pupdate<__half, float><<<G, B, 0, s>>>(r.v, p.v, x.v, first, st, v_append.v, app, devb);
-            break;
+    if (r.prec == P16) {
+        if (x.prec != P32) return cudaErrorInvalidValue;
+        const int B = 128;
+        k_pupdate<__half, float><<<stream_grid(r.v.V * r.v.k, B), B, 0, s>>>(r.v, p.v, x.v, first, st, v_append.v, app,
+                                                                             devb);
+        return cudaGetLastError();
     }
+    if (x.prec != r.prec || (r.v.k & (r.v.k - 1)) != 0 || (app && r.v.k != 1)) return cudaErrorInvalidValue;
+    const size_t n = (size_t)r.v.V * r.v.k * (r.prec == P64 ? 12 : 6);
+    const size_t need = (n + PU_THREADS - 1) / PU_THREADS, cap = (size_t)device_sm_count() * 8;
+    const int G = (int)(need < cap ? need : cap);
+    if (r.prec == P64)
+        k_pupdate_flat<double2, double><<<G, PU_THREADS, 0, s>>>(
+            static_cast<const double2 *>(r.v.data), static_cast<double2 *>(p.v.data), static_cast<double2 *>(x.v.data), n,
+            r.v.k, first, st, static_cast<double2 *>(v_append.v.data), app, devb);
+    else
+        k_pupdate_flat<float4, float><<<G, PU_THREADS, 0, s>>>(
+            static_cast<const float4 *>(r.v.data), static_cast<float4 *>(p.v.data), static_cast<float4 *>(x.v.data), n,
+            r.v.k, first, st, static_cast<float4 *>(v_append.v.data), app, devb);
     return cudaGetLastError();
 }
 
