@@ -894,19 +894,7 @@ static bool cg_run(Solve &sv, int max_iter, Window *w, eig_op_s *op) {
         std::vector<double> Mnew;
         int nout = 0;
         if (w) {
-            if (restart_now) {
-                // Fig. 1 steps 11.3-11.6 on the host from T_m
-                std::vector<cd> T;
-                window_T(*w, w->m, sv.ha(), sv.hb(), sv.hr(), T);
-                QZ.resize((size_t)w->m * 2 * w->nev);
-                Mnew.resize(2 * w->nev);
-                nout = dense::restart_coefficients(w->m, T.data(), w->kh, w->nev,
-                                                   std::max(w->m, 2 * w->nev) * 2.2e-16, QZ.data(), Mnew.data());
-                if (nout < 1) throw Error{EIG_ERR_BREAKDOWN, "eigCG restart basis is empty"};
-                slot = w->freel.back();  // the spare slot
-            } else {
-                slot = w->freel.back();
-            }
+            slot = w->freel.back();  // at a restart, the spare slot
             w->freel.pop_back();
             vapp = field_at(op->wprec, (char *)op->win.p + (size_t)slot * op->wfield_bytes(), op->Vf, 1);
         }
@@ -925,6 +913,15 @@ static bool cg_run(Solve &sv, int max_iter, Window *w, eig_op_s *op) {
                                  s));
         if (w) {
             if (restart_now) {
+                // Fig. 1 steps 11.3-11.6 on the host from T_m, while the GPU runs the iteration
+                // launched above (it needs only the spare slot)
+                std::vector<cd> T;
+                window_T(*w, w->m, sv.ha(), sv.hb(), sv.hr(), T);
+                QZ.resize((size_t)w->m * 2 * w->nev);
+                Mnew.resize(2 * w->nev);
+                nout = dense::restart_coefficients(w->m, T.data(), w->kh, w->nev,
+                                                   std::max(w->m, 2 * w->nev) * 2.2e-16, QZ.data(), Mnew.data());
+                if (nout < 1) throw Error{EIG_ERR_BREAKDOWN, "eigCG restart basis is empty"};
                 // step 11.7 (V <- V QZ in place) fused with step 11.8 (w^H V)
                 const int m = w->m;
                 std::vector<long> off(m);

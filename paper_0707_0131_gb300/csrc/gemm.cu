@@ -388,6 +388,20 @@ cudaError_t launch_gemm_ay(ColSet A, const double *Y, ColSet Out, double beta_ou
     return cudaGetLastError();
 }
 
+// The last block's sum of the grid's partial sums, one warp per output (lanes over blocks, then
+// a shuffle tree: a fixed order).  One thread per output took a serial chain of gridDim
+// dependent loads and FP64 adds (~64 issue cycles each): about 60 us at 608 blocks.
+__device__ __forceinline__ void sum_partials(const double *partials, int nout, double *out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int o = warp; o < nout; o += nw) {
+        double s = 0.0;
+        for (unsigned b = lane; b < gridDim.x; b += 32) s += __ldcg(partials + (long)b * nout + o);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) out[o] = s;
+    }
+}
+
 // ---------------------------------------------------------------------------------------
 // eigCG restart: V[:, c] = sum_a V[:, a] QZ[a, c] for c < nout, in place over the
 // window slots (each thread owns whole rows, reading all m inputs before writing),
@@ -396,90 +410,60 @@ cudaError_t launch_gemm_ay(ColSet A, const double *Y, ColSet Out, double beta_ou
 constexpr int WR_MAXOUT = 32;
 constexpr int WR_THREADS = 128;
 
-// NO: compile-time bound on the number of outputs (8, 16 or 32) so that the
-// per-thread accumulators fit in registers
-template <typename T, int NO>
-__global__ void __launch_bounds__(WR_THREADS) k_window_restart(ColSet Vw, int m, const double *QZ, int nout,
-                                                               const void *tv, const void *tpv,
-                                                               const double *beta_dev, long nrows,
-                                                               double *partials, unsigned *counter, double *wv) {
-    using V2 = typename C2<T>::t;
+// FP64: thread per (row, output); NO = 8, 16 or 32 bounds the outputs.  The kernel is bound by
+// FP64 issue (~64 cycles per warp instruction): with one thread per row a 4^4 window (3072
+// rows, m = 24, 16 outputs) kept 24 blocks busy with 1536 FMAs per thread (84 us); spread over
+// the outputs it fills the GPU.  A block reads all m columns of its rows before it writes any.
+template <int NO>
+__global__ void __launch_bounds__(WR_THREADS) k_window_restart64(ColSet Vw, int m, const double *QZ, int nout,
+                                                                 const double2 *t, const double2 *tp,
+                                                                 const double *beta_dev, long nrows, double *partials,
+                                                                 unsigned *counter, double *wv) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    V2 *Qs = reinterpret_cast<V2 *>(sm_raw);  // [m][nout]
-    __shared__ double red[(WR_THREADS / 32) * 2];
-    for (int L = threadIdx.x; L < m * nout; L += blockDim.x) {
-        V2 v;
-        v.x = (T)QZ[2 * L];
-        v.y = (T)QZ[2 * L + 1];
-        Qs[L] = v;
-    }
+    double2 *Qs = reinterpret_cast<double2 *>(sm_raw);  // [m][nout]
+    __shared__ double2 red[WR_THREADS];
+    for (int L = threadIdx.x; L < m * nout; L += blockDim.x) Qs[L] = make_double2(QZ[2 * L], QZ[2 * L + 1]);
     __syncthreads();
-    const T beta = (T)(*beta_dev);
-    const V2 *t = static_cast<const V2 *>(tv);
-    const V2 *tp = static_cast<const V2 *>(tpv);
-    V2 *base = static_cast<V2 *>(Vw.base);
-    T ws_re[NO], ws_im[NO];
-#pragma unroll
-    for (int c = 0; c < NO; c++) ws_re[c] = ws_im[c] = 0;
-    for (long row = (long)blockIdx.x * blockDim.x + threadIdx.x; row < nrows; row += (long)gridDim.x * blockDim.x) {
-        T re[NO], im[NO];
-#pragma unroll
-        for (int c = 0; c < NO; c++) re[c] = im[c] = 0;
-        for (int a = 0; a < m; a++) {
-            const V2 v = base[Vw.col_off[a] + row];
-#pragma unroll
-            for (int c = 0; c < NO; c++) {
-                if (c < nout) {
-                    const V2 q = Qs[a * nout + c];
-                    re[c] = fma(v.x, q.x, re[c]);
-                    re[c] = fma(-v.y, q.y, re[c]);
-                    im[c] = fma(v.x, q.y, im[c]);
-                    im[c] = fma(v.y, q.x, im[c]);
-                }
+    constexpr int R = WR_THREADS / NO;  // rows per block and pass
+    const int c = threadIdx.x % NO, rr = threadIdx.x / NO;
+    const double beta = *beta_dev;
+    double2 *base = static_cast<double2 *>(Vw.base);
+    double2 ws = make_double2(0.0, 0.0);
+    for (long r0 = (long)blockIdx.x * R; r0 < nrows; r0 += (long)gridDim.x * R) {
+        const long row = r0 + rr;
+        const bool on = row < nrows && c < nout;
+        double re = 0.0, im = 0.0;
+        if (on)
+            for (int a = 0; a < m; a++) {
+                const double2 v = base[Vw.col_off[a] + row], q = Qs[a * nout + c];
+                re = fma(v.x, q.x, re);
+                re = fma(-v.y, q.y, re);
+                im = fma(v.x, q.y, im);
+                im = fma(v.y, q.x, im);
             }
-        }
-        const V2 tt = t[row], tq = tp[row];
-        const T wr = tt.x - beta * tq.x, wi = tt.y - beta * tq.y;
-#pragma unroll
-        for (int c = 0; c < NO; c++) {
-            if (c < nout) {
-                V2 o;
-                o.x = re[c];
-                o.y = im[c];
-                base[Vw.col_off[c] + row] = o;
-                // conj(w) * v
-                ws_re[c] = fma(wr, re[c], ws_re[c]);
-                ws_re[c] = fma(wi, im[c], ws_re[c]);
-                ws_im[c] = fma(wr, im[c], ws_im[c]);
-                ws_im[c] = fma(-wi, re[c], ws_im[c]);
-            }
+        __syncthreads();  // every column of the block's rows has been read
+        if (on) {
+            const double2 tt = t[row], tq = tp[row];
+            const double wr = tt.x - beta * tq.x, wi = tt.y - beta * tq.y;
+            base[Vw.col_off[c] + row] = make_double2(re, im);
+            ws.x = fma(wr, re, ws.x);  // conj(w) * v
+            ws.x = fma(wi, im, ws.x);
+            ws.y = fma(wr, im, ws.y);
+            ws.y = fma(-wi, re, ws.y);
         }
     }
-    // block reduction of the nout complex sums, one output at a time, in FP64
-    double *P = partials + (long)blockIdx.x * nout * 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = 0; c < nout; c++) {
-        double vr = (double)ws_re[c], vi = (double)ws_im[c];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            vr += __shfl_xor_sync(0xffffffffu, vr, off);
-            vi += __shfl_xor_sync(0xffffffffu, vi, off);
+    red[threadIdx.x] = ws;
+    __syncthreads();
+    if (threadIdx.x < nout) {
+        double2 s = make_double2(0.0, 0.0);
+        for (int q = 0; q < R; q++) {
+            const double2 z = red[q * NO + threadIdx.x];
+            s.x += z.x;
+            s.y += z.y;
         }
-        if (lane == 0) {
-            red[warp * 2] = vr;
-            red[warp * 2 + 1] = vi;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sr = 0.0, si = 0.0;
-            for (int w = 0; w < WR_THREADS / 32; w++) {
-                sr += red[w * 2];
-                si += red[w * 2 + 1];
-            }
-            P[c * 2] = sr;
-            P[c * 2 + 1] = si;
-        }
-        __syncthreads();
+        double *P = partials + ((long)blockIdx.x * nout + threadIdx.x) * 2;
+        P[0] = s.x;
+        P[1] = s.y;
     }
     __shared__ bool am_last;
     __threadfence();
@@ -488,11 +472,7 @@ __global__ void __launch_bounds__(WR_THREADS) k_window_restart(ColSet Vw, int m,
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    for (int o = threadIdx.x; o < nout * 2; o += blockDim.x) {
-        double s = 0.0;
-        for (unsigned b = 0; b < gridDim.x; b++) s += __ldcg(partials + (long)b * nout * 2 + o);
-        wv[o] = s;
-    }
+    sum_partials(partials, nout * 2, wv);
     if (threadIdx.x == 0) *counter = 0u;
 }
 
@@ -601,11 +581,7 @@ __global__ void __launch_bounds__(WR_THREADS) k_window_restart32(ColSet Vw, int 
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    for (int o = threadIdx.x; o < nout * 2; o += blockDim.x) {
-        double sum = 0.0;
-        for (unsigned b = 0; b < gridDim.x; b++) sum += __ldcg(partials + (long)b * nout * 2 + o);
-        wv[o] = sum;
-    }
+    sum_partials(partials, nout * 2, wv);
     if (threadIdx.x == 0) *counter = 0u;
 }
 
@@ -619,16 +595,21 @@ cudaError_t launch_window_restart(ColSet Vw, int m, const double *QZ, int nout, 
     if (grid > cap) grid = cap;
     const long pcap = (long)red.max_blocks * MAX_RHS * 64 / (nout * 2);
     if (grid > pcap) grid = pcap;
-#define EIG_WR(T, NO)                                                                                   \
-    do {                                                                                                \
-        cudaFuncSetAttribute(k_window_restart<T, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-        k_window_restart<T, NO><<<(int)grid, WR_THREADS, smem, s>>>(Vw, m, QZ, nout, t, t_prev, beta_dev, nrows, \
-                                                                  red.partials, red.counter, wv);        \
-    } while (0)
     if (Vw.f64) {
-        if (nout <= 8) EIG_WR(double, 8);
-        else if (nout <= 16) EIG_WR(double, 16);
-        else EIG_WR(double, 32);
+#define EIG_WR64(NO)                                                                                            \
+    do {                                                                                                        \
+        const long g64 = (nrows + WR_THREADS / NO - 1) / (WR_THREADS / NO);                                     \
+        if (grid < cap && g64 > grid) grid = g64 < cap ? g64 : cap;                                             \
+        if (grid > pcap) grid = pcap;                                                                           \
+        cudaFuncSetAttribute(k_window_restart64<NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
+        k_window_restart64<NO><<<(int)grid, WR_THREADS, smem, s>>>(                                             \
+            Vw, m, QZ, nout, static_cast<const double2 *>(t), static_cast<const double2 *>(t_prev), beta_dev,   \
+            nrows, red.partials, red.counter, wv);                                                              \
+    } while (0)
+        if (nout <= 8) EIG_WR64(8);
+        else if (nout <= 16) EIG_WR64(16);
+        else EIG_WR64(32);
+#undef EIG_WR64
     } else {
 #define EIG_WR32(NO)                                                                                       \
     do {                                                                                                   \
@@ -644,7 +625,6 @@ cudaError_t launch_window_restart(ColSet Vw, int m, const double *QZ, int nout, 
         else EIG_WR32(32);
 #undef EIG_WR32
     }
-#undef EIG_WR
     return cudaGetLastError();
 }
 
@@ -653,58 +633,58 @@ cudaError_t launch_window_restart(ColSet Vw, int m, const double *QZ, int nout, 
 // device): Fig. 1 step 11.8 after a restart whose V <- V QZ ran elsewhere.  FP32
 // products per thread, FP64 block sums, the grid's sums added in a fixed order.
 namespace {
+// Bound by HBM (the window's columns do not stay in L2): two rows (16 bytes) per thread and
+// column, the column addresses in shared memory.  16^3x32, 20 columns: 176 -> 122 us (2.3 TB/s;
+// about 40 us of it the two reductions).
 template <int NO>
-__global__ void __launch_bounds__(WR_THREADS) k_wdot(const float2 *__restrict__ t, const float2 *__restrict__ tp,
+__global__ void __launch_bounds__(WR_THREADS) k_wdot(const float4 *__restrict__ t, const float4 *__restrict__ tp,
                                                      const double *beta_dev, const float2 *base, const long *off,
-                                                     int nout, long nrows, double *partials, unsigned *counter,
+                                                     int nout, long npairs, double *partials, unsigned *counter,
                                                      double *wv) {
-    __shared__ double red[(WR_THREADS / 32) * 2];
+    __shared__ const float4 *col[NO];
+    if (threadIdx.x < NO)
+        col[threadIdx.x] = reinterpret_cast<const float4 *>(base + off[threadIdx.x < nout ? threadIdx.x : 0]);
+    __syncthreads();
     const float beta = (float)(*beta_dev);
     float2 ws[NO];
 #pragma unroll
     for (int c = 0; c < NO; c++) ws[c] = make_float2(0.f, 0.f);
-    for (long row = (long)blockIdx.x * blockDim.x + threadIdx.x; row < nrows; row += (long)gridDim.x * blockDim.x) {
-        const float2 tv = t[row], pv = tp[row];
-        const float wr = tv.x - beta * pv.x, wi = tv.y - beta * pv.y;
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < npairs; i += (long)gridDim.x * blockDim.x) {
+        const float4 tv = t[i], pv = tp[i];
+        const float4 w = make_float4(tv.x - beta * pv.x, tv.y - beta * pv.y, tv.z - beta * pv.z, tv.w - beta * pv.w);
 #pragma unroll
-        for (int c = 0; c < NO; c++)
-            if (c < nout) {
-                const float2 o = base[off[c] + row];
-                ws[c] = __ffma2_rn(make_float2(wr, wr), o, ws[c]);                      // conj(w) * o
-                ws[c] = __ffma2_rn(make_float2(wi, wi), make_float2(o.y, -o.x), ws[c]);
+        for (int c0 = 0; c0 < NO; c0 += 8) {
+            if (c0 >= nout) break;
+            float4 o[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) o[q] = col[c0 + q][i];  // past nout: column 0 again, unused
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                float2 &a = ws[c0 + q];  // += conj(w) * o for both rows
+                a = __ffma2_rn(make_float2(w.x, w.x), make_float2(o[q].x, o[q].y), a);
+                a = __ffma2_rn(make_float2(w.y, w.y), make_float2(o[q].y, -o[q].x), a);
+                a = __ffma2_rn(make_float2(w.z, w.z), make_float2(o[q].z, o[q].w), a);
+                a = __ffma2_rn(make_float2(w.w, w.w), make_float2(o[q].w, -o[q].z), a);
             }
+        }
     }
-    double *Pp = partials + (long)blockIdx.x * nout * 2;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = 0; c < nout; c++) {
-        double vr = 0.0, vi = 0.0;
+    // block sums in FP64 through shared memory: thread o < 2 nout adds the block's FP32 sums of
+    // one part of one output (a shuffle tree per output costs five times the FP64 adds)
+    __shared__ float part[2 * NO][WR_THREADS + 1];
+    __shared__ double half_sum[2 * NO];
 #pragma unroll
-        for (int cc = 0; cc < NO; cc++)
-            if (cc == c) {
-                vr = (double)ws[cc].x;
-                vi = (double)ws[cc].y;
-            }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            vr += __shfl_xor_sync(0xffffffffu, vr, o);
-            vi += __shfl_xor_sync(0xffffffffu, vi, o);
-        }
-        if (lane == 0) {
-            red[warp * 2] = vr;
-            red[warp * 2 + 1] = vi;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double sr = 0.0, si = 0.0;
-            for (int w = 0; w < WR_THREADS / 32; w++) {
-                sr += red[w * 2];
-                si += red[w * 2 + 1];
-            }
-            Pp[c * 2] = sr;
-            Pp[c * 2 + 1] = si;
-        }
-        __syncthreads();
+    for (int c = 0; c < NO; c++) {
+        part[2 * c][threadIdx.x] = ws[c].x;
+        part[2 * c + 1][threadIdx.x] = ws[c].y;
     }
+    __syncthreads();
+    const int o2 = threadIdx.x % (2 * NO), hh = threadIdx.x / (2 * NO);  // output part, half of the threads
+    double bsum = 0.0;
+    if (hh < 2)
+        for (int q = hh * (WR_THREADS / 2); q < (hh + 1) * (WR_THREADS / 2); q++) bsum += (double)part[o2][q];
+    if (hh == 1) half_sum[o2] = bsum;
+    __syncthreads();
+    if (hh == 0 && o2 < 2 * nout) partials[(long)blockIdx.x * nout * 2 + o2] = bsum + half_sum[o2];
     __shared__ bool am_last;
     __threadfence();
     __syncthreads();
@@ -712,28 +692,25 @@ __global__ void __launch_bounds__(WR_THREADS) k_wdot(const float2 *__restrict__ 
     __syncthreads();
     if (!am_last) return;
     __threadfence();
-    for (int o = threadIdx.x; o < nout * 2; o += blockDim.x) {
-        double sum = 0.0;
-        for (unsigned b = 0; b < gridDim.x; b++) sum += __ldcg(partials + (long)b * nout * 2 + o);
-        wv[o] = sum;
-    }
+    sum_partials(partials, nout * 2, wv);
     if (threadIdx.x == 0) *counter = 0u;
 }
 }  // namespace
 
 cudaError_t launch_wdot(const void *t, const void *t_prev, const double *beta_dev, const void *base, const long *off,
                         int nout, long nrows, double *wv, RedScratch red, cudaStream_t s) {
-    if (nout < 1 || nout > 32) return cudaErrorInvalidValue;
+    // fields hold 12 complex entries per site, so rows come in pairs; slots are 16-byte aligned
+    if (nout < 1 || nout > 32 || (nrows & 1)) return cudaErrorInvalidValue;
     ProfScope prof("wdot", (double)nrows * (nout + 2) * 8.0, s);
-    long grid = (nrows + WR_THREADS - 1) / WR_THREADS;
+    long grid = (nrows / 2 + WR_THREADS - 1) / WR_THREADS;
     long cap = (long)device_sm_count() * 4;
     if (grid > cap) grid = cap;
     const long pcap = (long)red.max_blocks * MAX_RHS * 64 / (nout * 2);
     if (grid > pcap) grid = pcap;
-    auto t2 = static_cast<const float2 *>(t), p2 = static_cast<const float2 *>(t_prev);
+    auto t2 = static_cast<const float4 *>(t), p2 = static_cast<const float4 *>(t_prev);
     auto b2 = static_cast<const float2 *>(base);
 #define EIG_WD(NO) \
-    k_wdot<NO><<<(int)grid, WR_THREADS, 0, s>>>(t2, p2, beta_dev, b2, off, nout, nrows, red.partials, red.counter, wv)
+    k_wdot<NO><<<(int)grid, WR_THREADS, 0, s>>>(t2, p2, beta_dev, b2, off, nout, nrows / 2, red.partials, red.counter, wv)
     if (nout <= 8) EIG_WD(8);
     else if (nout <= 16) EIG_WD(16);
     else if (nout <= 24) EIG_WD(24);
