@@ -113,7 +113,7 @@ eig_status eig_op_trim(eig_op op, size_t *freed);
 
 /* out = M in (which 0), M^H in (which 1) or A in (which 2) for k RHS (1..max_rhs),
  * in the op's storage precision; which 3 (FP32/FP16 ops only) applies A in the
- * double-float arithmetic of the residual replacements (about 44-bit precision).
+ * FP64-accurate arithmetic of the residuals.
  * in/out: natural layout, may alias.
  * This is the dslash of the CG matrix-vector product (Fig. 1 step 11). */
 eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int k, void *stream);

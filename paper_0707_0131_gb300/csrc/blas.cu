@@ -312,6 +312,44 @@ cudaError_t launch_combine(Field out, double ca, Field a, double cb, Field b, cu
 }
 
 // ---------------------------------------------------------------------------------------
+// FP32 columns (one field each) <-> an FP64 RHS-inner field: thread per (chunk, site, column)
+// ---------------------------------------------------------------------------------------
+__global__ void k_cols32_to_f64(const float4 *__restrict__ cols, long cstride, unsigned V, unsigned kc,
+                                double2 *__restrict__ f) {
+    const size_t n = (size_t)V * 6 * kc, plane = (size_t)V * kc;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const unsigned c = (unsigned)(i / plane), o = (unsigned)(i - c * plane), s = o / kc, q = o - s * kc;
+        const float4 v = cols[(long)q * cstride + (long)c * V + s];
+        f[2 * c * plane + o] = make_double2((double)v.x, (double)v.y);
+        f[(2 * c + 1) * plane + o] = make_double2((double)v.z, (double)v.w);
+    }
+}
+
+__global__ void k_f64_to_cols32(const double2 *__restrict__ f, unsigned V, unsigned kc, float4 *__restrict__ cols,
+                                long cstride) {
+    const size_t n = (size_t)V * 6 * kc, plane = (size_t)V * kc;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const unsigned c = (unsigned)(i / plane), o = (unsigned)(i - c * plane), s = o / kc, q = o - s * kc;
+        const double2 a = f[2 * c * plane + o], b = f[(2 * c + 1) * plane + o];
+        cols[(long)q * cstride + (long)c * V + s] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+    }
+}
+
+cudaError_t launch_cols32_to_f64(const void *cols, long cstride_f4, long V, int kc, void *f64, cudaStream_t s) {
+    ProfScope prof("cols_to_f64", (double)V * 12 * kc * 24.0, s);
+    k_cols32_to_f64<<<stream_grid(V * 6 * kc, 128), 128, 0, s>>>(static_cast<const float4 *>(cols), cstride_f4,
+                                                                (unsigned)V, (unsigned)kc, static_cast<double2 *>(f64));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_f64_to_cols32(const void *f64, long V, int kc, void *cols, long cstride_f4, cudaStream_t s) {
+    ProfScope prof("f64_to_cols", (double)V * 12 * kc * 24.0, s);
+    k_f64_to_cols32<<<stream_grid(V * 6 * kc, 128), 128, 0, s>>>(static_cast<const double2 *>(f64), (unsigned)V,
+                                                                (unsigned)kc, static_cast<float4 *>(cols), cstride_f4);
+    return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------------------
 // norms
 // ---------------------------------------------------------------------------------------
 template <typename S>

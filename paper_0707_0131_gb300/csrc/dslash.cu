@@ -393,7 +393,7 @@ static std::string dslash_name(int epi, Prec p, int k) {
     return n;
 }
 
-// FP64 launches of n (site, RHS) pairs: spread the hops over lanes (dslash_split.cuh) while
+// FP64 launches of n (site, RHS) pairs that the fixed-point form does not take: spread the hops over lanes (dslash_split.cuh) while
 // the FP64 issue time of the fullest SM sub-partition is shorter that way.  One thread per
 // pair costs ~912 FP64 warp instructions per 32 pairs, the split form ~62 per 2 pairs; both
 // run in whole warps per sub-partition.
@@ -406,7 +406,8 @@ static bool split64(long n) {
 }
 
 bool dslash_takes_natural(const DslashCall &c) {
-    return c.in.prec == P64 && c.eo_parity < 0 && split64(c.V * c.k);
+    const long n = c.V * c.k;
+    return c.in.prec == P64 && c.eo_parity < 0 && split64(n) && (n < FX_MIN || !c.fx.links);
 }
 
 template <int EPI>
@@ -414,6 +415,22 @@ static cudaError_t dispatch(const DslashCall &c, KArgs &a, int cap, cudaStream_t
     const long work = a.V * c.k;
     const int block = 128;
     ProfScope prof(dslash_name(EPI, c.in.prec, c.k).c_str(), dslash_bytes<EPI>(c, a), s);
+    if (c.in.prec == P64 && c.gformat == GF_F64_18 && c.fx.links && !c.nat_in && !c.nat_out && work >= FX_MIN) {
+        Field fb{}, fr{}, ft{};
+        fb.v = a.b;
+        fr.v = a.r;
+        ft.v = a.tsave;
+        History h;
+        h.alpha = a.h_alpha;
+        h.beta = a.h_beta;
+        h.rho = a.h_rho;
+        h.jbase = a.jbase;
+        RedScratch red;
+        red.partials = a.partials;
+        red.counter = a.counter;
+        red.max_blocks = cap;
+        return launch_dslash_fx(c, EPI, fb, fr, ft, a.st, h, a.iter, a.set_rho, red, s);
+    }
     if (c.in.prec == P64 && c.gformat == GF_F64_18 && split64(work)) {
         SplitArgs b;
         split_args(b, c);

@@ -1,0 +1,502 @@
+// The FP64 Wilson stencil in block fixed-point integer arithmetic.
+//
+// GB300 issues an FP64 warp instruction about every 64 cycles per SM sub-partition, so the
+// ~912 FP64 instructions of a site keep the FP64 units busy for ~1800 cycles per (site, RHS)
+// while everything else idles (24^3x64, k = 16: 22.7 ms per product, 4% of HBM).  The integer
+// pipes run 32 times faster.  Here the hops are computed on 64-bit integers with one exponent
+// per site and RHS (fxmath.h):
+//   k_to_fx      brings a field to integers I = x 2^(1079 - e), |I| <= 2^57, e the largest
+//                exponent of the 24 reals of a (site, RHS); FP64 bits beyond the 57 below a
+//                site's largest component are dropped;
+//   k_dslash_fx  aligns the eight neighbours of a site to their largest exponent (a shift),
+//                projects them by integer adds, multiplies by the links (two 29-bit limbs per
+//                real, three wide multiply-adds per real product), sums the eight hops exactly
+//                and rounds once to FP64, where the centre term and the epilogue are formed.
+// The only errors are the alignment and limb truncations, at most 2^-55 of the largest neighbour
+// component per hop, and the final rounding; against the exact product the measured error is no
+// larger than that of the FP64 chain (16^3x32, Gaussian vectors: 1.3e-16 against 1.4e-16).  A
+// site with an Inf or NaN among its neighbours takes an FP64 path of its own, so non-finite
+// values propagate as there.  Links must be unitary to 1% (checked when an operator is created;
+// the sums of eight hops then stay below 2^63); other operators keep the FP64 stencil, and so
+// do launches too small to fill the GPU (FX_MIN).
+//
+// What bounds it now: the wide multiply-adds (1728 per site, 2 cycles each on the heavy half of
+// the FMA pipe, 46% busy), integer ALU (39%) and the latency of the neighbour loads at 16 warps
+// per SM.  Measured per product, conversion included (the conversion alone 28 us, 5.4 TB/s):
+//   16^3x32, k = 4    FP64 850 us    fixed point 282 us
+//   12^3x24, k = 8    double-float (44 bits; used for residual replacements before) 194 us plus
+//                     120 us of field conversions per A; fixed point 184 us
+// Four blocks per SM (128 registers, ~160 bytes spilled) beat three (294 us) and two (377 us);
+// without the L1 prefetch of the next hop three took 311 us; with the eight hops unrolled, 685.
+#include <cstring>
+
+#include "dslash_split.cuh"
+#include "fxmath.h"
+#include "kernels.cuh"
+#include "prof.h"
+
+namespace eig {
+
+namespace {
+
+// Layout of the integer field and links: tiles of 32 elements ((site, RHS) pairs; sites),
+// [element / 32][component][element % 32], so that a warp's loads are contiguous and the
+// components of an element sit at fixed distances from one address.
+constexpr int TILE = 32;
+__host__ __device__ constexpr size_t tiled(unsigned i, int comps) {
+    return (size_t)(i / TILE) * (size_t)(TILE * comps) + i % TILE;
+}
+
+struct FxArgs {
+    const longlong2 *fx;  // hop input in fixed point (re, im), tiled, 12 components
+    const int *ex;        // its exponents: [V][k]
+    const double2 *in;    // the same field in FP64 (sites with non-finite neighbours)
+    const double2 *cen;   // centre-term input (null: hops only)
+    const int4 *g;        // links, limbs (re hi, re lo, im hi, im lo): [mu] tiled, 9 components
+    const double2 *g64;
+    double2 *out;
+    const double2 *b;
+    double2 *r;
+    double2 *tsave;
+    unsigned L0, L1, L2, L3, V, Vg, lh, k, kshift;
+    FastDiv d0, d1, d2, dh;
+    int eo;
+    double diag, hcoef;
+    int save_t, set_rho;
+    CGScalars *st;
+    double *h_alpha, *h_beta, *h_rho;
+    int iter;
+    const int *jbase;
+    double *partials;
+    unsigned *counter;
+};
+
+constexpr int FX_TPB = 128;
+
+__global__ void __launch_bounds__(FX_TPB) k_to_fx(const double2 *__restrict__ in, longlong2 *__restrict__ fxo,
+                                                  int *__restrict__ ex, unsigned n) {
+    for (unsigned o = blockIdx.x * FX_TPB + threadIdx.x; o < n; o += gridDim.x * FX_TPB) {
+        double2 v[12];
+#pragma unroll
+        for (int c = 0; c < 12; c++) v[c] = in[(size_t)c * n + o];
+        unsigned top = 0;  // largest high word, sign removed: its exponent field is the block's
+#pragma unroll
+        for (int c = 0; c < 12; c++) {
+            top = max(top, (unsigned)__double2hiint(v[c].x) & 0x7fffffffu);
+            top = max(top, (unsigned)__double2hiint(v[c].y) & 0x7fffffffu);
+        }
+        const int e = max((int)(top >> 20), 1);
+        ex[o] = e;
+        if (e >= fx::SPECIAL) continue;  // never read
+#pragma unroll
+        for (int c = 0; c < 12; c++) {
+            longlong2 z;
+            z.x = fx::to_fixed(v[c].x, e);
+            z.y = fx::to_fixed(v[c].y, e);
+            fxo[tiled(o, 12) + c * TILE] = z;
+        }
+    }
+}
+
+__host__ __device__ constexpr size_t fx_link_plane(unsigned V) { return (size_t)((V + TILE - 1) / TILE) * TILE * 9; }
+
+// links [mu][9][V] FP64 -> limbs of u 2^58; *bad is set unless every row and column has norm 1
+// to 1% (NaN and Inf included)
+__global__ void k_links_fx(const double2 *__restrict__ g, int4 *__restrict__ out, unsigned V, int *bad) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < 4u * V; i += gridDim.x * blockDim.x) {
+        const unsigned mu = i / V, s = i - mu * V;
+        const double2 *p = g + (size_t)mu * 9 * V + s;
+        double row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+        for (int e = 0; e < 9; e++) {
+            const double2 u = p[(size_t)e * V];
+            const double n = u.x * u.x + u.y * u.y;
+            row[e / 3] += n;
+            col[e % 3] += n;
+            int4 l;
+            fx::limbs(__double2ll_rn(u.x * 0x1p58), l.x, l.y);
+            fx::limbs(__double2ll_rn(u.y * 0x1p58), l.z, l.w);
+            out[mu * fx_link_plane(V) + tiled(s, 9) + e * TILE] = l;
+        }
+        bool ok = true;
+        for (int q = 0; q < 3; q++)
+            ok = ok && row[q] > 0.98 && row[q] < 1.02 && col[q] > 0.98 && col[q] < 1.02;
+        if (!ok) *bad = 1;
+    }
+}
+
+struct I2 {
+    long long re, im;
+};
+
+__device__ __forceinline__ I2 add(I2 x, I2 y) {
+    x.re += y.re;
+    x.im += y.im;
+    return x;
+}
+__device__ __forceinline__ I2 sub(I2 x, I2 y) {
+    x.re -= y.re;
+    x.im -= y.im;
+    return x;
+}
+__device__ __forceinline__ I2 addi(I2 x, I2 y) {  // x + i y
+    x.re -= y.im;
+    x.im += y.re;
+    return x;
+}
+__device__ __forceinline__ I2 subi(I2 x, I2 y) {  // x - i y
+    x.re += y.im;
+    x.im -= y.re;
+    return x;
+}
+
+__device__ __forceinline__ void prefetch_hop_fx(const FxArgs &a, int mu, unsigned o, unsigned ls) {
+    const longlong2 *f = a.fx + tiled(o, 12);
+#pragma unroll
+    for (int e = 0; e < 12; e++) asm volatile("prefetch.global.L1 [%0];" ::"l"(f + e * TILE));
+    if (mu > 3) return;
+    const int4 *g = a.g + mu * fx_link_plane(a.Vg) + tiled(ls, 9);
+#pragma unroll
+    for (int e = 0; e < 9; e++) asm volatile("prefetch.global.L1 [%0];" ::"l"(g + e * TILE));
+}
+
+// One hop: neighbour at field index o (in (site, RHS) units), link (mu, ls),
+// conj(U)^T if bwd, projector I + sg g_mu.  mu, bwd and sg are uniform over the launch's
+// threads and not template arguments: only the projection and the rebuilding differ between the
+// eight hops, and with all of them unrolled the ~11 000 instructions of a site did not fit the
+// instruction caches (stalled on instruction fetch 3.8 of 7 cycles per issue).
+__device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool plus, unsigned o, unsigned ls, int sh,
+                                       I2 (&acc)[12]) {
+    const longlong2 *f = a.fx + tiled(o, 12);
+    I2 v[12];
+#pragma unroll
+    for (int e = 0; e < 12; e++) {
+        const longlong2 d = __ldg(f + e * TILE);
+        v[e].re = d.x >> sh;
+        v[e].im = d.y >> sh;
+    }
+    // project: h = a + sg B_mu b (see dslash.cu for B_mu)
+    I2 h[6];
+    const int which = mu * 2 + (plus ? 1 : 0);
+#define FX_PROJECT(F0, B0, F1, B1)                   \
+    do {                                             \
+        h[0] = F0(v[0], v[B0]);                      \
+        h[1] = F0(v[1], v[B0 + 1]);                  \
+        h[2] = F0(v[2], v[B0 + 2]);                  \
+        h[3] = F1(v[3], v[B1]);                      \
+        h[4] = F1(v[4], v[B1 + 1]);                  \
+        h[5] = F1(v[5], v[B1 + 2]);                  \
+    } while (0)
+    switch (which) {
+        case 0: FX_PROJECT(subi, 9, subi, 6); break;
+        case 1: FX_PROJECT(addi, 9, addi, 6); break;
+        case 2: FX_PROJECT(add, 9, sub, 6); break;
+        case 3: FX_PROJECT(sub, 9, add, 6); break;
+        case 4: FX_PROJECT(subi, 6, addi, 9); break;
+        case 5: FX_PROJECT(addi, 6, subi, 9); break;
+        case 6: FX_PROJECT(sub, 6, sub, 9); break;
+        default: FX_PROJECT(add, 6, add, 9); break;
+    }
+#undef FX_PROJECT
+    int rh[6], rl[6], ih[6], il[6];
+#pragma unroll
+    for (int e = 0; e < 6; e++) {
+        fx::limbs(h[e].re, rh[e], rl[e]);
+        fx::limbs(h[e].im, ih[e], il[e]);
+    }
+    const int4 *g = a.g + mu * fx_link_plane(a.Vg) + tiled(ls, 9);
+    const int sq = bwd ? TILE : 3 * TILE, sb = bwd ? 3 * TILE : TILE;
+    I2 w[6];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        // output colour q of both spins: sum over colours b of U[q][b] h_b, or conj(U[b][q]) h_b
+        int4 u[3];
+#pragma unroll
+        for (int b = 0; b < 3; b++) {
+            u[b] = __ldg(g + q * sq + b * sb);
+            if (bwd) {
+                u[b].z = -u[b].z;
+                u[b].w = -u[b].w;
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < 2; s++) {
+            fx::Acc re{0, 0}, im{0, 0};
+#pragma unroll
+            for (int b = 0; b < 3; b++) {
+                const int e = s * 3 + b;
+                fx::mul_add(re, u[b].x, u[b].y, rh[e], rl[e]);
+                fx::mul_add(re, u[b].z, u[b].w, -ih[e], -il[e]);
+                fx::mul_add(im, u[b].x, u[b].y, ih[e], il[e]);
+                fx::mul_add(im, u[b].z, u[b].w, rh[e], rl[e]);
+            }
+            w[s * 3 + q].re = fx::value(re.hh, re.mid);
+            w[s * 3 + q].im = fx::value(im.hh, im.mid);
+        }
+    }
+    // rebuild (w, sg B_mu^H w)
+#pragma unroll
+    for (int e = 0; e < 6; e++) acc[e] = add(acc[e], w[e]);
+#define FX_REBUILD(F0, W0, F1, W1)                   \
+    do {                                             \
+        acc[6] = F0(acc[6], w[W0]);                  \
+        acc[7] = F0(acc[7], w[W0 + 1]);              \
+        acc[8] = F0(acc[8], w[W0 + 2]);              \
+        acc[9] = F1(acc[9], w[W1]);                  \
+        acc[10] = F1(acc[10], w[W1 + 1]);            \
+        acc[11] = F1(acc[11], w[W1 + 2]);            \
+    } while (0)
+    switch (which) {
+        case 0: FX_REBUILD(addi, 3, addi, 0); break;
+        case 1: FX_REBUILD(subi, 3, subi, 0); break;
+        case 2: FX_REBUILD(sub, 3, add, 0); break;
+        case 3: FX_REBUILD(add, 3, sub, 0); break;
+        case 4: FX_REBUILD(addi, 0, subi, 3); break;
+        case 5: FX_REBUILD(subi, 0, addi, 3); break;
+        case 6: FX_REBUILD(sub, 0, sub, 3); break;
+        default: FX_REBUILD(add, 0, add, 3); break;
+    }
+#undef FX_REBUILD
+}
+
+// The hop sum of one (site, RHS) in FP64 (sites with an Inf or NaN around them; loops kept
+// rolled: rarely taken)
+__device__ __noinline__ void hops_fp64(const FxArgs &a, size_t P, const unsigned *nbr, const unsigned *lks, int sf,
+                                       double2 *acc) {
+    for (int e = 0; e < 12; e++) acc[e] = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int hop = 0; hop < 8; hop++) {
+        const int mu = hop >> 1, sg = (hop & 1) ? -sf : sf;
+        const double2 *g = a.g64 + (size_t)mu * 9 * a.Vg + lks[hop];
+        double2 h[2][3], w[2][3];
+        for (int s = 0; s < 2; s++)
+            for (int c = 0; c < 3; c++) {
+                const int part = mu <= 1 ? 1 - s : s;
+                const double2 u = a.in[(size_t)(s * 3 + c) * P + nbr[hop]];
+                const double2 v = a.in[(size_t)(6 + part * 3 + c) * P + nbr[hop]];
+                const bool neg = ((mu == 1 && s == 0) || (mu == 2 && s == 1)) != (sg < 0);
+                double2 q = (mu == 0 || mu == 2) ? make_double2(-v.y, v.x) : v;
+                h[s][c] = neg ? make_double2(u.x - q.x, u.y - q.y) : make_double2(u.x + q.x, u.y + q.y);
+            }
+        for (int s = 0; s < 2; s++)
+            for (int i = 0; i < 3; i++) {
+                double2 z = make_double2(0.0, 0.0);
+                for (int b = 0; b < 3; b++) {
+                    double2 u = g[(size_t)((hop & 1) ? b * 3 + i : i * 3 + b) * a.Vg];
+                    if (hop & 1) u.y = -u.y;
+                    z.x += u.x * h[s][b].x - u.y * h[s][b].y;
+                    z.y += u.x * h[s][b].y + u.y * h[s][b].x;
+                }
+                w[s][i] = z;
+            }
+        for (int s = 0; s < 2; s++)
+            for (int c = 0; c < 3; c++) {
+                acc[s * 3 + c].x += w[s][c].x;
+                acc[s * 3 + c].y += w[s][c].y;
+                const double2 v = w[mu <= 1 ? 1 - s : s][c];
+                const bool neg = ((mu == 0) || (mu == 1 && s == 1) || (mu == 2 && s == 0)) != (sg < 0);
+                const double2 q = (mu == 0 || mu == 2) ? make_double2(-v.y, v.x) : v;
+                acc[6 + s * 3 + c].x += neg ? -q.x : q.x;
+                acc[6 + s * 3 + c].y += neg ? -q.y : q.y;
+            }
+    }
+}
+
+template <bool DAG, int EPI>
+__global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const FxArgs a) {
+    __shared__ double smem[(FX_TPB / 32) * MAX_RHS];
+    if (EPI == SPL_NORM || EPI == SPL_CG) {
+        bool any = false;
+        for (unsigned q = 0; q < a.k; q++) any = any || a.st[q].active;
+        if (!any) return;
+    }
+    const unsigned total = a.V << a.kshift;
+    const size_t P = total;
+    const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2;
+    double nrm = 0.0;
+    for (unsigned g = blockIdx.x * FX_TPB + threadIdx.x; g < total; g += gridDim.x * FX_TPB) {
+        const unsigned s = g >> a.kshift, r = g & (a.k - 1);
+        unsigned x, y, z, t, sl;
+        if (a.eo >= 0) {
+            const unsigned rest = a.lh > 1 ? fastdiv(s, a.dh) : s, q2 = fastdiv(rest, a.d1);
+            t = fastdiv(q2, a.d2);
+            y = rest - q2 * a.L1;
+            z = q2 - t * a.L2;
+            x = 2 * (s - rest * a.lh) + ((a.eo + y + z + t) & 1);
+            sl = x + rest * a.L0;
+        } else {
+            const unsigned q1 = fastdiv(s, a.d0), q2 = fastdiv(q1, a.d1);
+            t = fastdiv(q2, a.d2);
+            x = s - q1 * a.L0;
+            y = q1 - q2 * a.L1;
+            z = q2 - t * a.L2;
+            sl = s;
+        }
+        // neighbour of hop h = 2 mu + (backward) as a lattice site
+        auto neighbour = [&](int h) {
+            const int mu = h >> 1;
+            const unsigned c = mu == 0 ? x : (mu == 1 ? y : (mu == 2 ? z : t));
+            const unsigned L = mu == 0 ? a.L0 : (mu == 1 ? a.L1 : (mu == 2 ? a.L2 : a.L3));
+            const unsigned st = mu == 0 ? 1u : (mu == 1 ? s1 : (mu == 2 ? s2 : s3));
+            return (h & 1) ? (c == 0 ? sl + (L - 1) * st : sl - st) : (c == L - 1 ? sl - (L - 1) * st : sl + st);
+        };
+        auto field_index = [&](unsigned nl) { return ((a.eo >= 0 ? nl >> 1 : nl) << a.kshift) + r; };
+        int e[8], em = 1;
+#pragma unroll
+        for (int h = 0; h < 8; h++) {
+            e[h] = __ldg(a.ex + field_index(neighbour(h)));
+            em = max(em, e[h]);
+        }
+        unsigned long long shifts = 0;  // alignment of each hop, 8 bits each
+#pragma unroll
+        for (int h = 0; h < 8; h++) shifts |= (unsigned long long)min(em - e[h], 63) << (8 * h);
+        double2 hs[12];  // hop sum
+        if (em < fx::SPECIAL) {
+            I2 acc[12];
+#pragma unroll
+            for (int q = 0; q < 12; q++) acc[q].re = acc[q].im = 0;
+            unsigned nl = neighbour(0);
+#pragma unroll 1
+            for (int h = 0; h < 8; h++) {
+                const bool bwd = h & 1;
+                // ask L1 for the next hop's data while this one is computed
+                const unsigned nx = h < 7 ? neighbour(h + 1) : nl;
+                prefetch_hop_fx(a, (h + 1) >> 1, field_index(nx), bwd ? sl : nx);
+                hop_fx(a, h >> 1, bwd, DAG != bwd, field_index(nl), bwd ? nl : sl, (int)(shifts & 63), acc);
+                shifts >>= 8;
+                nl = nx;
+            }
+#pragma unroll
+            for (int q = 0; q < 12; q++) hs[q] = make_double2(fx::to_double(acc[q].re, em), fx::to_double(acc[q].im, em));
+        } else {
+            unsigned nbr[8], lks[8];
+#pragma unroll 1
+            for (int h = 0; h < 8; h++) {
+                const unsigned nl = neighbour(h);
+                nbr[h] = field_index(nl);
+                lks[h] = (h & 1) ? nl : sl;
+            }
+            hops_fp64(a, P, nbr, lks, DAG ? +1 : -1, hs);
+        }
+        // diag * centre + hcoef * hops, then the epilogue, component by component
+        const double d = a.diag, hc = a.hcoef;
+        double al = 0.0;
+        if (EPI == SPL_CG) {
+            const CGScalars &st = a.st[r];
+            al = st.active ? st.alpha : 0.0;
+        }
+        double n2 = 0.0;
+#pragma unroll
+        for (int q = 0; q < 12; q++) {
+            const size_t o = (size_t)q * P + g;
+            const double2 c0 = a.cen ? a.cen[o] : make_double2(0.0, 0.0);
+            double2 w = make_double2(d * c0.x + hc * hs[q].x, d * c0.y + hc * hs[q].y);
+            if (EPI == SPL_PLAIN || EPI == SPL_NORM) {
+                a.out[o] = w;
+            } else if (EPI == SPL_CG) {
+                if (a.save_t) a.tsave[(size_t)q * a.V + s] = w;
+                double2 rr = a.r[o];
+                rr.x -= al * w.x;
+                rr.y -= al * w.y;
+                a.r[o] = rr;
+                w = rr;
+            } else {
+                const double2 bb = a.b[o];
+                w = make_double2(bb.x - w.x, bb.y - w.y);
+                a.r[o] = w;
+            }
+            if (EPI != SPL_PLAIN) n2 += w.x * w.x + w.y * w.y;
+        }
+        nrm += n2;
+    }
+    if (EPI == SPL_PLAIN) return;
+    const double bs = block_reduce_rhs(nrm, (int)a.k, smem);
+    const int k = (int)a.k;
+    CGScalars *const sts = a.st;
+    double *const h_alpha = a.h_alpha, *const h_beta = a.h_beta, *const h_rho = a.h_rho;
+    const int iter = a.iter + (a.jbase ? *a.jbase : 0), set_rho = a.set_rho;
+    grid_reduce_rhs(bs, k, a.partials, a.counter, smem, [=](int rr, double tot) {
+        finish_scalars<EPI>(sts, h_alpha, h_beta, h_rho, iter, k, set_rho, rr, tot);
+    });
+}
+
+template <int EPI>
+cudaError_t fx_launch(bool dag, const FxArgs &a, int cap, cudaStream_t s) {
+    const long n = (long)a.V << a.kshift;
+    long grid = (n + FX_TPB - 1) / FX_TPB;
+    const long most = (long)device_sm_count() * 4;  // resident blocks
+    if (EPI != SPL_PLAIN && grid > most) grid = most;
+    if (cap > 0 && grid > cap) grid = cap;
+    if (dag) k_dslash_fx<true, EPI><<<(int)grid, FX_TPB, 0, s>>>(a);
+    else k_dslash_fx<false, EPI><<<(int)grid, FX_TPB, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// bytes of the integer field of n (site, RHS) pairs and of the links of V sites
+size_t fx_field_bytes(long n) { return (size_t)((n + TILE - 1) / TILE) * TILE * 12 * 16; }
+size_t fx_link_bytes(long V) { return 4 * fx_link_plane((unsigned)V) * 16; }
+
+cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaStream_t s) {
+    ProfScope prof("links_fx", (double)V * 4 * 288.0, s);
+    long grid = (4 * V + 127) / 128;
+    const long cap = (long)device_sm_count() * 16;
+    if (grid > cap) grid = cap;
+    k_links_fx<<<(int)grid, 128, 0, s>>>(static_cast<const double2 *>(g64), static_cast<int4 *>(gfx), (unsigned)V, bad);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Field t_save, CGScalars *st, History h,
+                             int iter, bool set_rho, RedScratch red, cudaStream_t s) {
+    FxArgs a;
+    memset(&a, 0, sizeof(a));
+    a.V = (unsigned)(c.eo_parity >= 0 ? c.V / 2 : c.V);
+    a.k = (unsigned)c.k;
+    while ((1u << a.kshift) < a.k) a.kshift++;
+    const unsigned n = a.V << a.kshift;
+    a.fx = static_cast<const longlong2 *>(c.fx.data);
+    a.ex = c.fx.ex;
+    a.in = static_cast<const double2 *>(c.in.v.data);
+    a.cen = static_cast<const double2 *>(c.eo_parity >= 0 ? (c.diag != 0.0 ? c.cen.v.data : nullptr) : c.in.v.data);
+    a.g = static_cast<const int4 *>(c.fx.links);
+    a.g64 = static_cast<const double2 *>(c.gauge.data);
+    a.out = static_cast<double2 *>(c.out.v.data);
+    a.b = static_cast<const double2 *>(b.v.data);
+    a.r = static_cast<double2 *>(r.v.data);
+    a.tsave = static_cast<double2 *>(t_save.v.data);
+    a.save_t = t_save.v.data != nullptr;
+    a.L0 = c.L[0];
+    a.L1 = c.L[1];
+    a.L2 = c.L[2];
+    a.L3 = c.L[3];
+    a.d0 = fastdiv_make(a.L0);
+    a.d1 = fastdiv_make(a.L1);
+    a.d2 = fastdiv_make(a.L2);
+    a.lh = a.L0 / 2;
+    if (a.lh >= 2) a.dh = fastdiv_make(a.lh);
+    a.Vg = (unsigned)c.V;
+    a.eo = c.eo_parity;
+    a.diag = c.diag;
+    a.hcoef = c.hcoef;
+    a.st = st;
+    a.h_alpha = h.alpha;
+    a.h_beta = h.beta;
+    a.h_rho = h.rho;
+    a.iter = iter;
+    a.jbase = h.jbase;
+    a.set_rho = set_rho;
+    a.partials = red.partials;
+    a.counter = red.counter;
+    {
+        long grid = (n + FX_TPB - 1) / FX_TPB;
+        k_to_fx<<<(int)grid, FX_TPB, 0, s>>>(a.in, static_cast<longlong2 *>(c.fx.data), c.fx.ex, n);
+    }
+    switch (epi) {
+        case SPL_PLAIN: return fx_launch<SPL_PLAIN>(c.dagger, a, 0, s);
+        case SPL_NORM: return fx_launch<SPL_NORM>(c.dagger, a, red.max_blocks, s);
+        case SPL_CG: return fx_launch<SPL_CG>(c.dagger, a, red.max_blocks, s);
+        default: return fx_launch<SPL_RESID>(c.dagger, a, red.max_blocks, s);
+    }
+}
+
+}  // namespace eig

@@ -191,7 +191,9 @@ struct eig_op_s {
     int gf_inner;
     int max_rhs;
     double delta;
-    DevBuf gauge64, gauge_in, gauge_dd;  // gauge_dd: double-float copy (mixed precision)
+    DevBuf gauge64, gauge_in;
+    DevBuf gauge_fx;  // the FP64 links as limbs (dslash_fx.cu); empty if they are not unitary
+    DevBuf fx_ex;     // workspace: exponents of the fixed-point field (which sits in nat_in)
     DevBuf gauge_alt;                    // FP32 ops: the links in the other FP32 format
     int gf_alt = -1;
     // workspace
@@ -265,6 +267,13 @@ struct eig_op_s {
         c.diag = 4.0 + m_q;
         c.dagger = dag;
         c.cen = Field{};
+        if (f64 && gauge_fx.p && fx_ex.p) {
+            // the fixed-point input field borrows the host staging buffer: copies from the host
+            // land there and are packed on the same stream before any stencil of the call
+            c.fx.data = nat_in.p;
+            c.fx.ex = fx_ex.as<int>();
+            c.fx.links = gauge_fx.p;
+        }
         return c;
     }
     History history(int k) const {
@@ -346,8 +355,9 @@ static void ensure_workspace(eig_op_s *op) {
         op->full64.alloc(P64, V, K);
         op->be64.alloc(P64, Vf, K);
     }
-    op->nat_in.alloc((size_t)V * 12 * 16 * K);
+    op->nat_in.alloc(fx_field_bytes(V * K));  // at least V * 12 * 16 * K
     op->nat_out.alloc((size_t)V * 12 * 16 * K);
+    if (op->gauge_fx.p) op->fx_ex.alloc((size_t)Vf * K * sizeof(int));
     op->ws = true;
 }
 
@@ -360,6 +370,7 @@ static void release_workspace(eig_op_s *op) {
         f->release();
     op->nat_in.release();
     op->nat_out.release();
+    op->fx_ex.release();
     op->win.release();
     op->win_slots = 0;
     op->tprev.release();
@@ -417,7 +428,7 @@ static void apply_M(eig_op_s *op, Field in, Field out, bool dag, bool f64, cudaS
     CUDA_CK(launch_dslash(mcall(op, in, out, dag, f64, s), s));
 }
 
-// out = A in in FP64 (uses op->u64 as scratch; in/out must not be u64)
+// out = A in in FP64 (uses op->u64 as scratch; in/out must not be u64, and may be the same)
 static void apply_A64(eig_op_s *op, Field in, Field out, cudaStream_t s) {
     Field u = op->u64.view(in.v.k);
     apply_M(op, in, u, false, true, s);
@@ -603,31 +614,20 @@ struct Solve {
     const double *hb() const { return op->hist_h.as<double>() + (size_t)h.cap * k; }
     const double *hr() const { return op->hist_h.as<double>() + 2 * (size_t)h.cap * k; }
 
-    // r64 = b - A x64; with set_rho the CG scalars take the true residual.  final:
-    // FP64 arithmetic (the reported residual); otherwise, in mixed precision, the
-    // double-float stencil (residual replacements between checks).
-    void true_residual(bool set_rho, bool final_check = true) {
+    // r64 = b - A x64 in FP64; with set_rho the CG scalars take the true residual.
+    void true_residual(bool set_rho) {
         CUDA_CK(launch_xflush(p, xlo, st, k, s));
         if (mixed) {
             CUDA_CK(launch_combine(x64, 1.0, x64, 1.0, xlo, s));
             zero_field(xlo, s);
         }
-        if (mixed && !final_check && !op->eo) {
-            const long n = op->Vf * 12 * (long)k;
-            CUDA_CK(launch_to_dd(x64.v.data, r64.v.data, n, s));  // r64 holds x in dd until overwritten
-            CUDA_CK(launch_dslash_dd(op->call(x64, u64, false, true), op->gauge_dd.p, r64.v.data, u64.v.data, s));
-            CUDA_CK(launch_dslash_dd_resid(op->call(u64, r64, true, true), op->gauge_dd.p, u64.v.data, b64, r64, st, h,
-                                           j, set_rho, red, s));
-        } else {
-            apply_M(op, x64, u64, false, true, s);
-            CUDA_CK(launch_dslash_resid(mcall(op, u64, r64, true, true, s), b64, r64, st, h, j, set_rho, red, s));
-        }
+        apply_M(op, x64, u64, false, true, s);
+        CUDA_CK(launch_dslash_resid(mcall(op, u64, r64, true, true, s), b64, r64, st, h, j, set_rho, red, s));
         if (mixed && set_rho) CUDA_CK(launch_combine(r, 1.0, r64, 0.0, null_field(), s));
     }
 
     // r64 = b64 - A x64 for the deflation of the initial guess (Eq. 1): r64 = b64 when
-    // every x is zero, else the double-float stencil in mixed precision (full lattice)
-    // or the FP64 one.
+    // every x is zero.
     void initial_residual() {
         CUDA_CK(launch_norm2(x64, st, false, h, 0, red, s));
         read_scalars();
@@ -635,16 +635,9 @@ struct Solve {
         for (int q = 0; q < k; q++) zero = zero && sth[q].aux == 0.0;
         if (zero) {
             CUDA_CK(launch_combine(r64, 1.0, b64, 0.0, null_field(), s));
-        } else if (mixed && !op->eo) {
-            const long n = op->Vf * 12 * (long)k;
-            CUDA_CK(launch_to_dd(x64.v.data, r64.v.data, n, s));  // r64 holds x in dd until overwritten
-            CUDA_CK(launch_dslash_dd(op->call(x64, u64, false, true), op->gauge_dd.p, r64.v.data, u64.v.data, s));
-            CUDA_CK(launch_dslash_dd_resid(op->call(u64, r64, true, true), op->gauge_dd.p, u64.v.data, b64, r64, st, h,
-                                           0, false, red, s));
         } else {
             apply_M(op, x64, u64, false, true, s);
-            apply_M(op, u64, r64, true, true, s);
-            CUDA_CK(launch_combine(r64, 1.0, b64, -1.0, r64, s));
+            CUDA_CK(launch_dslash_resid(mcall(op, u64, r64, true, true, s), b64, r64, st, h, 0, false, red, s));
         }
     }
 
@@ -654,7 +647,7 @@ struct Solve {
         CUDA_CK(launch_norm2(b64, st, false, h, 0, red, s));
         CUDA_CK(launch_cg_init(st, k, tol, h, s));
         if (mixed) zero_field(xlo, s);
-        true_residual(false, false);
+        true_residual(false);
         if (mixed) CUDA_CK(launch_combine(r, 1.0, r64, 0.0, null_field(), s));
         CUDA_CK(launch_norm2(r64, st, true, h, 0, red, s));
         read_scalars();
@@ -715,7 +708,7 @@ struct Solve {
         return (int)std::min<double>(CHECK, std::max(1.0, std::floor(worst)));
     }
     void reliable_update() {
-        true_residual(true, false);
+        true_residual(true);
         read_scalars();
         for (int q = 0; q < k; q++) {
             rmax[q] = std::sqrt(sth[q].rho);
@@ -1445,9 +1438,18 @@ eig_status eig_op_create(const double *gauge, const int dims[4], double m_q, con
     CUDA_CK(cudaMemcpy(stage.p, gauge, stage.n, cudaMemcpyHostToDevice));
     op->gauge64.alloc((size_t)V * 4 * 9 * 16);
     CUDA_CK(launch_pack_gauge(stage.as<double>(), op->gauge64.p, GF_F64_18, V, 0));
+    if (op->Vf * K >= FX_MIN) {
+        // the links as limbs of the fixed-point FP64 stencil, unless one is not unitary
+        eig::DevBuf bad;
+        int h_bad = 1;
+        bad.alloc(sizeof(int));
+        op->gauge_fx.alloc(fx_link_bytes(V));
+        CUDA_CK(cudaMemset(bad.p, 0, sizeof(int)));
+        CUDA_CK(launch_links_fx(op->gauge64.p, op->gauge_fx.p, V, bad.as<int>(), 0));
+        CUDA_CK(cudaMemcpy(&h_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost));
+        if (h_bad) op->gauge_fx.release();
+    }
     if (op->prec != P64) {
-        op->gauge_dd.alloc((size_t)V * 4 * 9 * 16);
-        CUDA_CK(launch_to_dd(op->gauge64.p, op->gauge_dd.p, V * 4 * 9, 0));
         size_t gb = op->gf_inner == GF_F32_12 ? 48 : (op->gf_inner == GF_F32_18 ? 72 : 24);
         op->gauge_in.alloc((size_t)V * 4 * gb);
         CUDA_CK(launch_pack_gauge(stage.as<double>(), op->gauge_in.p, op->gf_inner, V, 0));
@@ -1495,7 +1497,7 @@ eig_status eig_op_trim(eig_op op, size_t *freed) {
                               &op->xsv, &op->tmp_e, &op->tmp64_e, &op->full64, &op->be64, &op->zsp, &op->bc_rh,
                               &op->bc_s, &op->bc_t})
         bytes += f->data.n + f->scale.n;
-    bytes += op->nat_in.n + op->nat_out.n + op->win.n + op->tprev.n + op->tcur.n;
+    bytes += op->nat_in.n + op->nat_out.n + op->fx_ex.n + op->win.n + op->tprev.n + op->tcur.n;
     release_workspace(op);
     if (freed) *freed = bytes;
     API_END
@@ -1504,21 +1506,17 @@ eig_status eig_op_trim(eig_op op, size_t *freed) {
 eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int k, void *stream) {
     API_BEGIN
     ARG_CHECK(op && in && out, "null argument");
-    ARG_CHECK(which >= 0 && which <= 3, "which must be 0 (M), 1 (M^H), 2 (A) or 3 (A in double-float)");
+    ARG_CHECK(which >= 0 && which <= 3, "which must be 0 (M), 1 (M^H), 2 (A) or 3 (A in FP64)");
     ARG_CHECK(which != 3 || op->prec != P64, "which = 3 needs an FP32 or FP16 op");
     ARG_CHECK(which != 3 || !op->eo, "which = 3 is not available for odd-even operators");
     ARG_CHECK(k >= 1 && k <= op->max_rhs && (k & (k - 1)) == 0, "k must be a power of two <= max_rhs");
     std::lock_guard<std::mutex> lk(op->mu);
     ensure_workspace(op);
     cudaStream_t s = (cudaStream_t)stream;
-    if (which == 3) {  // A = M^H M in double-float arithmetic
-        const long n = op->Vf * 12 * (long)k;
-        Field x64 = op->x64.view(k), t1 = op->u64.view(k), t2 = op->r64.view(k);
+    if (which == 3) {  // A = M^H M as the residuals of a mixed-precision op take it
+        Field x64 = op->x64.view(k);
         load_natural(op, in, x64, s);
-        CUDA_CK(launch_to_dd(x64.v.data, t1.v.data, n, s));
-        CUDA_CK(launch_dslash_dd(op->call(x64, t2, false, true), op->gauge_dd.p, t1.v.data, t2.v.data, s));
-        CUDA_CK(launch_dslash_dd(op->call(x64, t1, true, true), op->gauge_dd.p, t2.v.data, t1.v.data, s));
-        CUDA_CK(launch_from_dd(t1.v.data, x64.v.data, n, s));
+        apply_A64(op, x64, x64, s);
         store_natural(op, x64, out, s);
         sync(s);
         return EIG_OK;
@@ -1857,18 +1855,19 @@ eig_status eig_basis_grow(eig_basis B, void *stream) {
         sync(s);
     }
     if (op->prec != P64 && !op->eo) {
-        // W = A V-bar in double-float arithmetic (about 44 bits, far below the FP32
-        // rounding of the stored W), up to max_rhs columns per stencil launch
+        // W = A V-bar in FP64, up to max_rhs columns per stencil launch
         const long cstride = (long)(op->wfield_bytes() / 16);
-        for (int c0 = 0; c0 < r; c0 += op->max_rhs) {
-            const int n = std::min(op->max_rhs, r - c0);
+        int n = 0;
+        for (int c0 = 0; c0 < r; c0 += n) {
+            n = 1;  // batches are powers of two
+            while (2 * n <= std::min(op->max_rhs, r - c0)) n *= 2;
             Field xin = op->r64.view(n), mid = op->u64.view(n), wout = op->x64.view(n);
-            CUDA_CK(launch_cols32_to_dd((char *)B->U.p + (size_t)(l + c0) * op->wfield_bytes(), cstride, op->Vf, n,
-                                        xin.v.data, s));
-            CUDA_CK(launch_dslash_dd(op->call(xin, mid, false, true), op->gauge_dd.p, xin.v.data, mid.v.data, s));
-            CUDA_CK(launch_dslash_dd(op->call(mid, wout, true, true), op->gauge_dd.p, mid.v.data, wout.v.data, s));
-            CUDA_CK(launch_dd_to_cols32(wout.v.data, op->Vf, n, (char *)B->W.p + (size_t)c0 * op->wfield_bytes(),
-                                        cstride, s));
+            CUDA_CK(launch_cols32_to_f64((char *)B->U.p + (size_t)(l + c0) * op->wfield_bytes(), cstride, op->Vf, n,
+                                         xin.v.data, s));
+            apply_M(op, xin, mid, false, true, s);
+            apply_M(op, mid, wout, true, true, s);
+            CUDA_CK(launch_f64_to_cols32(wout.v.data, op->Vf, n, (char *)B->W.p + (size_t)c0 * op->wfield_bytes(),
+                                         cstride, s));
         }
     } else {
         // W = A V-bar with the FP64 operator
@@ -1975,7 +1974,7 @@ eig_status eig_initcg_solve(eig_op op, eig_basis basis, const double *b, double 
         for (int q = 0; q < k; q++) it1[q] = sv.sth[q].nit;
         std::vector<int> rel1 = sv.reliable;
         if (ok) {
-            sv.true_residual(false, false);  // x64 += x_lo; r64 = b - A x64
+            sv.true_residual(false);  // x64 += x_lo; r64 = b - A x64
             deflate_into(basis, sv.r64, sv.x64, s);
             restarts = 1;
             sv.start(tol);

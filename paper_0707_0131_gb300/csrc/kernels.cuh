@@ -71,6 +71,14 @@ struct History {
     const int *jbase = nullptr;
 };
 
+// Scratch and links of the fixed-point FP64 stencil (dslash_fx.cu): 192 bytes per (site, RHS)
+// of the input, one int each, and the links as limbs; links == nullptr: not available.
+struct FxScratch {
+    void *data = nullptr;
+    int *ex = nullptr;
+    const void *links = nullptr;
+};
+
 struct DslashCall {
     Field in, out;     // out may be unused by the CG epilogue (store_out = 0)
     GaugeView gauge;
@@ -91,6 +99,7 @@ struct DslashCall {
     // in / out in the natural layout [rhs][site][12] of the API instead of the internal one:
     // only for calls dslash_takes_natural() accepts, with in and out disjoint
     bool nat_in = false, nat_out = false;
+    FxScratch fx;      // FP64 calls of operators that have it
 };
 // True if launch_dslash reads and writes the natural layout for this FP64 call (small
 // lattices, where the stencil spreads a site's hops over lanes).
@@ -130,18 +139,16 @@ int dslash32_best_gformat(long V, int k, int prec);
 // Link format (-1 before tuning) and stencil variant (0..7) the call would launch with.
 int dslash32_choice(const DslashCall &c, int *variant);
 
-// dslash_dd.cu: double-float (FP32-pair) stencil for residual replacements.  dd fields
-// have the FP64 layout with float4 (re_hi, im_hi, re_lo, im_lo) per complex number.
-cudaError_t launch_to_dd(const void *fp64, void *dd, long n_complex, cudaStream_t s);
-// kc FP32 fields of one RHS each (column c at cols + c * cstride_f4 float4s) <->
-// a double-float RHS-inner field of kc RHS
-cudaError_t launch_cols32_to_dd(const void *cols, long cstride_f4, long V, int kc, void *dd, cudaStream_t s);
-cudaError_t launch_dd_to_cols32(const void *dd, long V, int kc, void *cols, long cstride_f4, cudaStream_t s);
-cudaError_t launch_from_dd(const void *dd, void *fp64, long n_complex, cudaStream_t s);
-cudaError_t launch_dslash_dd(const DslashCall &c, const void *gauge_dd, const void *in_dd, void *out_dd,
-                             cudaStream_t s);
-cudaError_t launch_dslash_dd_resid(const DslashCall &c, const void *gauge_dd, const void *in_dd, Field b, Field r,
-                                   CGScalars *st, History h, int iter, bool set_rho, RedScratch red, cudaStream_t s);
+// dslash_fx.cu: the FP64 stencil in block fixed-point integer arithmetic (c.fx set), epilogue
+// epi of dslash_split.cuh; and the links as limbs, *bad (device) set where a link is not
+// unitary to 1%
+cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Field t_save, CGScalars *st, History h,
+                             int iter, bool set_rho, RedScratch red, cudaStream_t s);
+// From this many (site, RHS) pairs on, FP64 launches of operators with unitary links take it.
+constexpr long FX_MIN = 6144;
+size_t fx_field_bytes(long n);
+size_t fx_link_bytes(long V);
+cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaStream_t s);
 
 // ---------------------------- blas.cu -------------------------------------------------
 // natural FP64 [k][V][12] complex  <->  internal field
@@ -151,6 +158,10 @@ cudaError_t launch_unpack(Field f, double *nat, cudaStream_t s);
 cudaError_t launch_pack_gauge(const double *nat, void *dst, int gformat, long V, cudaStream_t s);
 // out = ca * a + cb * b   (b may have data == nullptr; ca, cb real).  All fields same V, k.
 cudaError_t launch_combine(Field out, double ca, Field a, double cb, Field b, cudaStream_t s);
+// kc FP32 fields of one RHS each (column c at cols + c * cstride_f4 float4s) <-> an FP64
+// RHS-inner field of kc RHS
+cudaError_t launch_cols32_to_f64(const void *cols, long cstride_f4, long V, int kc, void *f64, cudaStream_t s);
+cudaError_t launch_f64_to_cols32(const void *f64, long V, int kc, void *cols, long cstride_f4, cudaStream_t s);
 // per-RHS ||f||^2 -> st[r].aux;  with as_rho: also rho = aux, rho_prev = aux, history rho[iter]
 // and target = tol2 * bnorm2[r] computed elsewhere (untouched here).
 cudaError_t launch_norm2(Field f, CGScalars *st, bool as_rho, History h, int iter, RedScratch red, cudaStream_t s);

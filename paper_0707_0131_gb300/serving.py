@@ -64,9 +64,9 @@ class OpSpec:
         """Device bytes an operator keeps while idle: links in all forms, the basis."""
         V = int(np.prod(self.dims))
         wide = 192 if self.prec == 64 else 96
-        # FP64 links, their double-float copy (mixed precision) and the inner formats
+        # FP64 links, their fixed-point limbs and the inner formats
         # (FP32 ops keep both the 12- and the 18-real form, FP16 ops the 12-real one)
-        links = V * 4 * (144 + (0 if self.prec == 64 else 144) + {64: 0, 32: 48 + 72, 16: 48}[self.prec])
+        links = V * 4 * (144 + 144 + {64: 0, 32: 48 + 72, 16: 48}[self.prec])
         basis = V * wide * (self.basis_max + self.nev + 16 + 16)
         return links + basis
 
@@ -76,7 +76,7 @@ class OpSpec:
         V = int(np.prod(self.dims))
         sp = {64: 192, 32: 96, 16: 52}[self.prec]
         wide = 192 if self.prec == 64 else 96
-        work = V * self.max_rhs * (3 * sp + 5 * 192 + 2 * wide + 2 * 192) + V * 96 * 4
+        work = V * self.max_rhs * (3 * sp + 5 * 192 + 2 * wide + 2 * 192 + 4) + V * 96 * 4
         window = V * wide * (self.m + 3)
         return work + window
 
