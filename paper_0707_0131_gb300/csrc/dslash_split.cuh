@@ -107,14 +107,17 @@ __device__ __forceinline__ void finish_scalars(CGScalars *sts, double *h_alpha, 
 }
 
 // one complex component e of the spinor at (site, RHS) offset o = site stride * site + RHS
-// stride * RHS (in chunks), chunk stride cs
+// stride * RHS (in chunks), chunk stride cs; COH: read from L2 (data that other SMs write
+// during the launch)
 template <typename S>
 struct Comp;
 template <>
 struct Comp<double> {
     using C = double;
+    template <bool COH = false>
     __device__ static __forceinline__ Cx<double> load(const void *p, const float *, unsigned cs, unsigned o, int e) {
-        const double2 d = static_cast<const double2 *>(p)[(unsigned)e * cs + o];
+        const double2 *q = static_cast<const double2 *>(p) + ((unsigned)e * cs + o);
+        const double2 d = COH ? __ldcg(q) : *q;
         return cmk<double>(d.x, d.y);
     }
     __device__ static __forceinline__ void store(void *p, unsigned cs, unsigned o, int e, Cx<double> z) {
@@ -124,24 +127,16 @@ struct Comp<double> {
 template <>
 struct Comp<float> {
     using C = float;
+    template <bool COH = false>
     __device__ static __forceinline__ Cx<float> load(const void *p, const float *, unsigned cs, unsigned o, int e) {
-        const float2 d = static_cast<const float2 *>(p)[((unsigned)(e >> 1) * cs + o) * 2 + (e & 1)];
+        const float2 *q = static_cast<const float2 *>(p) + (((unsigned)(e >> 1) * cs + o) * 2 + (e & 1));
+        const float2 d = COH ? __ldcg(q) : *q;
         return cmk<float>(d.x, d.y);
     }
     __device__ static __forceinline__ void store(void *p, unsigned cs, unsigned o, int e, Cx<float> z) {
         static_cast<float2 *>(p)[((unsigned)(e >> 1) * cs + o) * 2 + (e & 1)] = make_float2(z.re, z.im);
     }
 };
-template <>
-struct Comp<__half> {
-    using C = float;
-    __device__ static __forceinline__ Cx<float> load(const void *p, const float *sc, unsigned cs, unsigned o, int e) {
-        const float2 d = __half22float2(static_cast<const __half2 *>(p)[((unsigned)(e >> 2) * cs + o) * 4 + (e & 3)]);
-        const float s = sc[o];
-        return cmk<float>(d.x * s, d.y * s);
-    }
-};
-
 // the rows of the link this lane multiplies by: u[a][b] = U[a][b] (bwd = false) or
 // conj(U[b][a]) (bwd = true)
 template <int GF, typename C>
@@ -160,10 +155,123 @@ __device__ __forceinline__ void load_link_for(const void *g, unsigned Vg, int mu
         }
 }
 
+// What lane l = 2 hop + spin of a 16-lane group does in every site: the projection
+// h = a_spin + ph (lower partner), partner spin part, factor +-1 or +-i
+template <typename C>
+struct LaneRole {
+    int l, mu, sp, part;
+    bool bwd, img;
+    C sre, sim;
+};
+template <bool DAG, typename C>
+__device__ __forceinline__ LaneRole<C> lane_role(int l) {
+    constexpr int SF = DAG ? +1 : -1;  // forward projector I + SF g_mu, backward I - SF g_mu
+    LaneRole<C> q;
+    q.l = l;
+    q.mu = l >> 2;
+    q.sp = l & 1;
+    q.bwd = (l >> 1) & 1;
+    q.part = q.mu <= 1 ? 1 - q.sp : q.sp;
+    q.img = q.mu == 0 || q.mu == 2;
+    const bool neg = ((q.mu == 1 && q.sp == 0) || (q.mu == 2 && q.sp == 1)) != ((q.bwd ? -SF : SF) < 0);
+    q.sre = (neg != q.img) ? (C)-1 : (C)1;
+    q.sim = neg ? (C)-1 : (C)1;
+    return q;
+}
+
+// Component l (lanes 0..11) of diag * centre + hcoef * (hop sum) at output site s, RHS r, from
+// the field in / in_s of a (cen: its centre term).  Collective over the warp; live is uniform
+// over a 16-lane group.  prod: the group's [8][2][3] products.
+template <typename S, int GF, bool DAG, bool COH>
+__device__ __forceinline__ Cx<typename Comp<S>::C> split_component(const SplitArgs &a, const LaneRole<typename Comp<S>::C> &q,
+                                                                   const void *in, const void *cen, bool live, unsigned s,
+                                                                   unsigned r, Cx<typename Comp<S>::C> (*prod)[2][3]) {
+    using C = typename Comp<S>::C;
+    constexpr int SF = DAG ? +1 : -1;
+    const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2;
+    unsigned x, y, z, tt, sl;
+    if (a.eo >= 0) {
+        const unsigned rest = a.lh > 1 ? fastdiv(s, a.dh) : s, q2 = fastdiv(rest, a.d1);
+        tt = fastdiv(q2, a.d2);
+        y = rest - q2 * a.L1;
+        z = q2 - tt * a.L2;
+        x = 2 * (s - rest * a.lh) + ((a.eo + y + z + tt) & 1);
+        sl = x + rest * a.L0;
+    } else {
+        const unsigned q1 = fastdiv(s, a.d0), q2 = fastdiv(q1, a.d1);
+        tt = fastdiv(q2, a.d2);
+        x = s - q1 * a.L0;
+        y = q1 - q2 * a.L1;
+        z = q2 - tt * a.L2;
+        sl = s;
+    }
+    const int l = q.l, mu = q.mu;
+    const unsigned cm = mu == 0 ? x : (mu == 1 ? y : (mu == 2 ? z : tt));
+    const unsigned Lm = mu == 0 ? a.L0 : (mu == 1 ? a.L1 : (mu == 2 ? a.L2 : a.L3));
+    const unsigned sm = mu == 0 ? 1u : (mu == 1 ? s1 : (mu == 2 ? s2 : s3));
+    const unsigned nl = q.bwd ? (cm == 0 ? sl + (Lm - 1) * sm : sl - sm) : (cm == Lm - 1 ? sl - (Lm - 1) * sm : sl + sm);
+    const unsigned nf = a.eo >= 0 ? nl >> 1 : nl;  // field index of the neighbour
+    const unsigned oin = nf * a.in_x + r * a.in_r, oc = s * a.in_x + r * a.in_r;
+    Cx<C> c0 = cmk<C>(0, 0);
+    if (live) {
+        Cx<C> h[3], u[3][3], v[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++) h[c] = Comp<S>::template load<COH>(in, nullptr, a.in_c, oin, q.sp * 3 + c);
+#pragma unroll
+        for (int c = 0; c < 3; c++) v[c] = Comp<S>::template load<COH>(in, nullptr, a.in_c, oin, 6 + q.part * 3 + c);
+        load_link_for<GF>(a.g, a.Vg, mu, q.bwd ? nl : sl, q.bwd, u);
+        if (l < 12 && cen) c0 = Comp<S>::template load<COH>(cen, nullptr, a.in_c, oc, l);  // in flight with the hops
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            h[c].re = fma(q.sre, q.img ? v[c].im : v[c].re, h[c].re);
+            h[c].im = fma(q.sim, q.img ? v[c].re : v[c].im, h[c].im);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            Cx<C> w = cmul(u[i][0], h[0]);
+            w = cfma(u[i][1], h[1], w);
+            w = cfma(u[i][2], h[2], w);
+            prod[l >> 1][q.sp][i] = w;
+        }
+    }
+    __syncwarp();
+    Cx<C> o = cmk<C>(0, 0);
+    if (l < 12 && live) {
+        const int so = l / 3, c = l - 3 * so, lo = so & 1;
+        Cx<C> acc = cmk<C>(0, 0);
+#pragma unroll
+        for (int hh = 0; hh < 8; hh++) {
+            const int m = hh >> 1, sg = (hh & 1) ? -SF : SF;
+            // upper spins take the product, lower spins sg B_mu^H of it
+            const int from = so < 2 ? lo : (m <= 1 ? 1 - lo : lo);
+            const Cx<C> w = prod[hh][from][c];
+            const bool im = so >= 2 && (m == 0 || m == 2);
+            bool ng = false;
+            if (so >= 2) ng = ((m == 0) || (m == 1 && lo == 1) || (m == 2 && lo == 0)) != (sg < 0);
+            // factor (-1)^ng, times i where im
+            const C fr = (ng != im) ? (C)-1 : (C)1, fi = ng ? (C)-1 : (C)1;
+            acc.re = fma(fr, im ? w.im : w.re, acc.re);
+            acc.im = fma(fi, im ? w.re : w.im, acc.im);
+        }
+        const C d = (C)a.diag, hc = (C)a.hcoef;
+        o = cmk<C>(d * c0.re + hc * acc.re, d * c0.im + hc * acc.im);
+    }
+    __syncwarp();
+    return o;
+}
+
+// |component|^2 summed over a 16-lane group (the same in its lanes)
+template <typename C>
+__device__ __forceinline__ double group_norm2(bool mine, Cx<C> o) {
+    C n = mine ? o.re * o.re + o.im * o.im : (C)0;
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
+    return (double)n;
+}
+
 template <typename S, int GF, bool DAG, int EPI>
 __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
     using C = typename Comp<S>::C;
-    constexpr int SF = DAG ? +1 : -1;  // forward projector I + SF g_mu, backward I - SF g_mu
     __shared__ Cx<C> prod[8][8][2][3];  // [group][hop][spin][colour]
     __shared__ double smem[(128 / 32) * MAX_RHS];
     __shared__ double gsum[8];
@@ -173,128 +281,29 @@ __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
         if (!any) return;
     }
     const int t = threadIdx.x, grp = t >> 4, l = t & 15;
-    const int hop = l >> 1, sp = l & 1, mu = hop >> 1;
-    const bool bwd = hop & 1;
+    const LaneRole<C> role = lane_role<DAG, C>(l);
     const unsigned total = a.V << a.kshift, step = gridDim.x * (blockDim.x >> 4);
-    const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2;
-    // this lane's projection h = a_sp + ph B: partner spin of the lower pair, factor +-1 or +-i
-    const int part = mu <= 1 ? 1 - sp : sp;
-    const bool img = mu == 0 || mu == 2;
-    const bool neg = ((mu == 1 && sp == 0) || (mu == 2 && sp == 1)) != ((bwd ? -SF : SF) < 0);
-    const C sre = (neg != img) ? (C)-1 : (C)1, sim = neg ? (C)-1 : (C)1;
     double nrm = 0.0;
     const unsigned niter = (total + step - 1) / step;
     for (unsigned it = 0; it < niter; it++) {
         const unsigned g = it * step + blockIdx.x * (blockDim.x >> 4) + grp;
         const bool live = g < total;  // uniform over a group, not over a warp
         const unsigned s = live ? g >> a.kshift : 0u, r = g & (a.k - 1);
-        unsigned x, y, z, tt, sl;
-        if (a.eo >= 0) {
-            const unsigned rest = a.lh > 1 ? fastdiv(s, a.dh) : s, q2 = fastdiv(rest, a.d1);
-            tt = fastdiv(q2, a.d2);
-            y = rest - q2 * a.L1;
-            z = q2 - tt * a.L2;
-            x = 2 * (s - rest * a.lh) + ((a.eo + y + z + tt) & 1);
-            sl = x + rest * a.L0;
-        } else {
-            const unsigned q1 = fastdiv(s, a.d0), q2 = fastdiv(q1, a.d1);
-            tt = fastdiv(q2, a.d2);
-            x = s - q1 * a.L0;
-            y = q1 - q2 * a.L1;
-            z = q2 - tt * a.L2;
-            sl = s;
-        }
-        const unsigned cm = mu == 0 ? x : (mu == 1 ? y : (mu == 2 ? z : tt));
-        const unsigned Lm = mu == 0 ? a.L0 : (mu == 1 ? a.L1 : (mu == 2 ? a.L2 : a.L3));
-        const unsigned sm = mu == 0 ? 1u : (mu == 1 ? s1 : (mu == 2 ? s2 : s3));
-        const unsigned nl = bwd ? (cm == 0 ? sl + (Lm - 1) * sm : sl - sm)
-                                : (cm == Lm - 1 ? sl - (Lm - 1) * sm : sl + sm);
-        const unsigned nf = a.eo >= 0 ? nl >> 1 : nl;  // field index of the neighbour
-        const unsigned oin = nf * a.in_x + r * a.in_r;
-        const unsigned oc = s * a.in_x + r * a.in_r, oo = s * a.out_x + r * a.out_r;
-        Cx<C> c0 = cmk<C>(0, 0), e0 = cmk<C>(0, 0);
-        if (live) {
-            Cx<C> h[3], u[3][3];
-#pragma unroll
-            for (int c = 0; c < 3; c++) h[c] = Comp<S>::load(a.in, a.in_s, a.in_c, oin, sp * 3 + c);
-            Cx<C> q[3];
-#pragma unroll
-            for (int c = 0; c < 3; c++) q[c] = Comp<S>::load(a.in, a.in_s, a.in_c, oin, 6 + part * 3 + c);
-            load_link_for<GF>(a.g, a.Vg, mu, bwd ? nl : sl, bwd, u);
-            if (l < 12) {  // the centre and the epilogue's operand, in flight with the hops
-                if (a.cen) c0 = Comp<S>::load(a.cen, a.cen_s, a.in_c, oc, l);
-                if (EPI == SPL_CG) e0 = Comp<S>::load(a.r, a.r_s, a.out_c, oo, l);
-                if (EPI == SPL_RESID) e0 = Comp<S>::load(a.b, nullptr, a.out_c, oo, l);
-            }
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                h[c].re = fma(sre, img ? q[c].im : q[c].re, h[c].re);
-                h[c].im = fma(sim, img ? q[c].re : q[c].im, h[c].im);
-            }
-#pragma unroll
-            for (int i = 0; i < 3; i++) {
-                Cx<C> v = cmul(u[i][0], h[0]);
-                v = cfma(u[i][1], h[1], v);
-                v = cfma(u[i][2], h[2], v);
-                prod[grp][hop][sp][i] = v;
-            }
-        }
-        __syncwarp();
-        Cx<C> o = cmk<C>(0, 0);
-        if (l < 12 && live) {
-            const int so = l / 3, c = l - 3 * so, lo = so & 1;
-            Cx<C> acc = cmk<C>(0, 0);
-#pragma unroll
-            for (int hh = 0; hh < 8; hh++) {
-                constexpr int SFc = SF;
-                const int m = hh >> 1, sg = (hh & 1) ? -SFc : SFc;
-                // upper spins take the product, lower spins sg B_mu^H of it
-                const int from = so < 2 ? lo : (m <= 1 ? 1 - lo : lo);
-                const Cx<C> w = prod[grp][hh][from][c];
-                const bool im = so >= 2 && (m == 0 || m == 2);
-                bool ng = false;
-                if (so >= 2) ng = ((m == 0) || (m == 1 && lo == 1) || (m == 2 && lo == 0)) != (sg < 0);
-                // factor (-1)^ng, times i where im
-                const C fr = (ng != im) ? (C)-1 : (C)1, fi = ng ? (C)-1 : (C)1;
-                acc.re = fma(fr, im ? w.im : w.re, acc.re);
-                acc.im = fma(fi, im ? w.re : w.im, acc.im);
-            }
-            const C d = (C)a.diag, hc = (C)a.hcoef;
-            o = cmk<C>(d * c0.re + hc * acc.re, d * c0.im + hc * acc.im);
-            if (EPI == SPL_RESID) o = e0 - o;
-        }
-        __syncwarp();
+        const unsigned oo = s * a.out_x + r * a.out_r;
+        const bool mine = live && l < 12;
+        Cx<C> e0 = cmk<C>(0, 0);
+        if (EPI == SPL_CG && mine) e0 = Comp<S>::load(a.r, nullptr, a.out_c, oo, l);
+        if (EPI == SPL_RESID && mine) e0 = Comp<S>::load(a.b, nullptr, a.out_c, oo, l);
+        Cx<C> o = split_component<S, GF, DAG, false>(a, role, a.in, a.cen, live, s, r, prod[grp]);
+        if (EPI == SPL_RESID) o = e0 - o;
         if (EPI == SPL_CG) {
             const CGScalars &st = a.st[r];
             const C al = st.active ? (C)st.alpha : (C)0;
-            const Cx<C> tv = o;
-            o = cmk<C>(e0.re - al * tv.re, e0.im - al * tv.im);
-            if (live && l < 12 && a.save_t) {  // single RHS, window precision
-                using W = typename Comp<S>::C;
-                Comp<W>::store(a.tsave, a.V, s, l, tv);
-            }
+            if (mine && a.save_t) Comp<S>::store(a.tsave, a.V, s, l, o);  // single RHS
+            o = cmk<C>(e0.re - al * o.re, e0.im - al * o.im);
         }
-        // the store of half-precision fields is collective over the warp: every lane takes part
-        if constexpr (sizeof(S) == 2) {
-            void *dst = EPI == SPL_CG ? a.r : a.out;
-            float *dsc = EPI == SPL_CG ? a.r_s : a.out_s;
-            float mx = (live && l < 12) ? fmaxf(fabsf(o.re), fabsf(o.im)) : 0.f;
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-            const float inv = mx > 0.f ? 1.0f / mx : 0.f;
-            if (live && l < 12)
-                static_cast<__half2 *>(dst)[((unsigned)(l >> 2) * a.out_c + oo) * 4 + (l & 3)] =
-                    __floats2half2_rn(o.re * inv, o.im * inv);
-            if (live && l == 0) dsc[oo] = mx;
-        } else {
-            if (live && l < 12) Comp<S>::store(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
-        }
-        if (EPI != SPL_PLAIN) {
-            C n = (live && l < 12) ? o.re * o.re + o.im * o.im : (C)0;
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
-            nrm += (double)n;  // the same in the 16 lanes; a group's RHS is the same in every pass
-        }
+        if (mine) Comp<S>::store(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
+        if (EPI != SPL_PLAIN) nrm += group_norm2<C>(mine, o);  // a group's RHS is the same in every pass
     }
     if (EPI == SPL_PLAIN) return;
     const int ngrp = blockDim.x >> 4, k = (int)a.k;

@@ -866,6 +866,36 @@ static bool cg_run(Solve &sv, int max_iter, Window *w, eig_op_s *op) {
                 fprintf(stderr, "\n");
             }
         }
+        if (!restart_now && !sv.sp && sv.j + 1 <= max_iter) {
+            // small lattices: the iterations up to the next check (or a full window) as one launch
+            const DslashCall c = op->call(sv.p, sv.u, false, op->prec == P64);
+            if (!op->eo && cg_cluster_takes(c)) {
+                CgCluster q;
+                q.p = sv.p;
+                q.r = sv.r;
+                q.x = sv.xlo;
+                q.j0 = sv.j;
+                q.n = std::min(std::min(CG_CLUSTER_ITERS, std::max(1, next_check - since)), max_iter - sv.j);
+                if (w) q.n = std::min(q.n, w->m - w->i);
+                q.first = sv.j == 0;
+                q.win = w ? op->win.p : nullptr;
+                q.slot_bytes = op->wfield_bytes();
+                q.tsave = nullptr;
+                for (int t = 0; t < q.n && w; t++) {
+                    q.slot[t] = w->freel.back();
+                    w->freel.pop_back();
+                    w->slots.push_back(q.slot[t]);
+                }
+                if (w) {
+                    w->i += q.n;
+                    if (w->i == w->m) q.tsave = w->tprev_is_a ? op->tprev.p : op->tcur.p;
+                }
+                CUDA_CK(launch_cg_cluster(c, q, sv.st, sv.h, s));
+                sv.j += q.n;
+                since += q.n;
+                continue;
+            }
+        }
         if (!w && !sv.sp && since == 0 && next_check == CHECK && sv.j >= 1 && sv.j + CHECK <= max_iter &&
             cg_graphs_enabled()) {
             // CHECK plain iterations as one replayed CUDA graph

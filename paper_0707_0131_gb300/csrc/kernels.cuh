@@ -122,6 +122,24 @@ cudaError_t launch_dslash_cg(const DslashCall &c, Field r, Field t_save, CGScala
 cudaError_t launch_dslash_resid(const DslashCall &c, Field b, Field r, CGScalars *st, History h, int iter,
                                 bool set_rho, RedScratch red, cudaStream_t s);
 
+// cg_cluster.cu: iterations j0 + 1 .. j0 + n of CG on a small FP32 lattice inside one thread-block
+// cluster (c: the call of u = M p; r, p and x are updated, u is not written).  With win (one
+// RHS): iteration j0 + 1 + q appends r / sqrt(rho) to slot[q], and the last one's t goes to
+// tsave if given.
+constexpr int CG_CLUSTER_ITERS = 16;
+constexpr long CG_CLUSTER_MAX = 4096;  // (site, RHS) pairs: 16 CTAs of 256 threads
+struct CgCluster {
+    Field p, r, x;
+    int j0, n;
+    bool first;        // the first iteration takes p = r
+    void *win;
+    size_t slot_bytes;
+    int slot[CG_CLUSTER_ITERS];
+    void *tsave;
+};
+bool cg_cluster_takes(const DslashCall &c);
+cudaError_t launch_cg_cluster(const DslashCall &c, const CgCluster &q, CGScalars *st, History h, cudaStream_t s);
+
 // dslash32.cu: FP32-arithmetic versions (FP32 / FP16 storage) of the three launches above
 cudaError_t launch_dslash32(const DslashCall &c, cudaStream_t s);
 cudaError_t launch_dslash32_norm(const DslashCall &c, CGScalars *st, History h, int iter, RedScratch red,
