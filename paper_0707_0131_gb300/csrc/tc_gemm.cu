@@ -26,6 +26,14 @@
 // they hand stages and TMEM regions to each other through mbarriers.  Every wait is
 // bounded: on timeout the CTA records an error, lets its copies land (bounded), frees
 // its TMEM and returns.
+//
+// The split A goes to tensor memory, where the MMAs read it: a staging slot is free as soon as
+// its rows are in registers, so shared memory holds only copies in flight.  The workers are two
+// groups of four warps on alternate K tiles, so that one group's waits hide behind the other's
+// work.  (With the split written back to shared memory and all eight warps on every tile, a 16
+// KB tile took ~2900 cycles whatever the basis size.)  16^3x32: 96 vectors, 16 RHS 936 -> 525 us
+// (2.7 TB/s); 20 to 30 vectors, 10 columns 890 -> 493 us.  A tile now takes ~1500 cycles: the
+// 8 MMAs issue in ~640, the rest is a worker warp's split and its share of the drain.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -120,15 +128,8 @@ __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int accum) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(dtmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accum)
-        : "memory");
-}
-// the same with A read from tensor memory (M = 128 rows in the 128 lanes, one 32-bit
-// column per K element; a K step of 8 advances the address by 8 columns)
+// D += A B, A read from tensor memory (M = 128 rows in the 128 lanes, one 32-bit column per K
+// element; a K step of 8 advances the address by 8 columns), B from shared memory
 __device__ __forceinline__ void mma_tf32_ts(uint32_t dtmem, uint32_t atmem, uint64_t bdesc, uint32_t idesc, int accum) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -187,27 +188,29 @@ __device__ __forceinline__ void two_sum_add(float &hi, float &lo, float x) {
     lo = __fadd_rn(lo, err);
 }
 
-// Warp specialisation: warp 0 (one lane) keeps the TMA ring full, warp 1 (one lane)
-// issues the MMAs, warps 2..9 split the A tiles in place into hi / lo, build the B
-// tiles and drain the accumulators.  The roles hand stages and TMEM regions to each
-// other through mbarriers only, so no role waits for work that was issued just
-// before (a block-wide barrier per tile made every tile cost one MMA round trip).
-//
-// Accumulation: groups of FLUSH K tiles accumulate in one of NREG TMEM regions (MT * N
-// columns each).  The tensor pipe adds in FP32 with its own rounding, so its error
-// grows with the accumulation length; each finished group is drained into per-thread
-// double-float sums, two groups behind the MMAs, and its region is then reused.
+// Accumulation: groups of FLUSH K tiles accumulate in one of NREG TMEM regions (MT * 2N
+// columns each).  The tensor pipe adds in FP32 with its own rounding, so its error grows with
+// the accumulation length; each finished group is drained into per-thread double-float sums,
+// NREG - 1 groups behind the MMAs, and its region is then reused.
 constexpr int FLUSH = 2;
-constexpr int NREG = 3;
-constexpr int WORKERS = 8;                    // worker warps
+constexpr int WORKERS = 8;                    // worker warps, two groups of four
 constexpr int TC_THREADS = 32 * (2 + WORKERS);
-static_assert((KT / 2) * 16 <= 32 * WORKERS, "one B value per worker thread per tile for k <= 16");
+static_assert(FLUSH == 2, "each worker group takes one K tile of every flush group");
+
+// M tiles -> TMEM regions, operand buffers and staging slots: TMEM holds NREG * MT * 2N
+// accumulator columns and NOP * MT * 64 operand columns (hi and lo, 32 each)
+template <int MT>
+struct AhbShape {
+    static constexpr int NREG = MT == 1 ? 3 : 2;
+    static constexpr int NOP = MT == 1 ? 4 : 2;
+    static constexpr int NS = MT == 1 ? 10 : 5;
+};
 
 // Worker warp w (warps 2..9) drains TMEM lanes 32 (w % 4) .. + 31 (the lane quarter a
 // warp may access) and the half h = (w - 2) / 4 of the region's MT * N columns.
-template <int MT, int N>
 // A region holds, for M tile mt, A_mt B_hi in columns mt 2N + [0, N) and A_mt B_lo in
 // mt 2N + N + [0, N); output column cc = mt N + c is the sum of the two.
+template <int MT, int N>
 __device__ __forceinline__ void drain(uint32_t region, int quarter, int half, float *acc_hi, float *acc_lo) {
     constexpr int HC = MT * N / 2;
     const uint32_t base = region + ((uint32_t)(quarter * 32) << 16);
@@ -230,24 +233,28 @@ __device__ __forceinline__ void drain(uint32_t region, int quarter, int half, fl
     }
 }
 
-template <int MT, int N, int NS>
+template <int MT, int N>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant__ CUtensorMap tmap, const TcArgs a) {
+    using SH = AhbShape<MT>;
+    constexpr int NREG = SH::NREG, NOP = SH::NOP, NS = SH::NS;
     extern __shared__ __align__(1024) unsigned char sm_raw[];
-    // 1024-byte aligned stages: [MT] A tiles (TMA lands here, split in place to hi),
-    // [MT] A_lo tiles, B_hi, B_lo
+    // 1024-byte aligned: NS stages of [MT] raw A tiles (TMA), then NOP operand buffers of
+    // B_hi, B_lo
     unsigned char *base = sm_raw + ((1024 - (sa(sm_raw) & 1023)) & 1023);
     constexpr uint32_t a_bytes = TM * KT * 4;  // 16 KB
     constexpr uint32_t b_bytes = (uint32_t)((N + 7) / 8) * 1024;
-    constexpr uint32_t stage_bytes = 2 * MT * a_bytes + 2 * b_bytes;
-    constexpr uint32_t RCOLS = MT * 2 * N;  // per M tile: A B_hi, then A B_lo (drain adds them)
-    constexpr uint32_t NCOLS =
-        NREG * RCOLS <= 32 ? 32 : (NREG * RCOLS <= 64 ? 64 : (NREG * RCOLS <= 128 ? 128 : (NREG * RCOLS <= 256 ? 256 : 512)));
-    static_assert(NREG * RCOLS <= 512, "TMEM columns");
-    __shared__ __align__(8) uint64_t raw_full[NS], split_done[NS], stage_free[NS], acc_full[NREG], acc_empty[NREG],
-        done, never;
+    constexpr uint32_t stage_bytes = MT * a_bytes, op_bytes = 2 * b_bytes;
+    constexpr uint32_t RCOLS = MT * 2 * N;      // per M tile: A B_hi, then A B_lo (drain adds them)
+    constexpr uint32_t AC0 = NREG * RCOLS;      // first operand column
+    constexpr uint32_t ACOLS = MT * 2 * KT;     // operand columns per buffer
+    constexpr uint32_t USED = AC0 + NOP * ACOLS;
+    static_assert(USED <= 512, "TMEM columns");
+    constexpr uint32_t NCOLS = USED <= 256 ? 256 : 512;
+    __shared__ __align__(8) uint64_t raw_full[NS], stage_free[NS], op_ready[NOP], op_free[NOP], acc_full[NREG],
+        acc_empty[NREG], done, never;
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
-    __shared__ int n_issued, n_consumed;
+    __shared__ int n_issued;
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
     const int kt0 = blockIdx.x * a.chunk;
     const int nkt = min(a.chunk, a.ktiles - kt0);
@@ -255,8 +262,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant_
     if (t == 0) {
         for (int s = 0; s < NS; s++) {
             mbar_init(&raw_full[s], 1);
-            mbar_init(&split_done[s], WORKERS);
-            mbar_init(&stage_free[s], 1);
+            mbar_init(&stage_free[s], WORKERS / 2);
+        }
+        for (int o = 0; o < NOP; o++) {
+            mbar_init(&op_ready[o], WORKERS / 2);
+            mbar_init(&op_free[o], 1);
         }
         for (int r = 0; r < NREG; r++) {
             mbar_init(&acc_full[r], 1);
@@ -266,7 +276,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant_
         mbar_init(&never, 1);
         abort_flag = 0;
         n_issued = 0;
-        n_consumed = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 0) {
@@ -275,14 +284,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant_
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
     }
+    unsigned char *ops = base + NS * stage_bytes;
+    // the rows of the B tiles past the 2k used ones stay zero
+    for (uint32_t i = t; i < NOP * op_bytes / 16; i += TC_THREADS)
+        reinterpret_cast<float4 *>(ops)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = tmem_base;
-    auto region = [&](int g) { return tmem + (uint32_t)((g % NREG) * RCOLS); };
-    auto A_hi = [&](int s, int mt) { return base + s * stage_bytes + mt * a_bytes; };
-    auto A_lo = [&](int s, int mt) { return base + s * stage_bytes + (MT + mt) * a_bytes; };
-    auto B_hi = [&](int s) { return base + s * stage_bytes + 2 * MT * a_bytes; };
-    auto B_lo = [&](int s) { return base + s * stage_bytes + 2 * MT * a_bytes + b_bytes; };
     auto fail = [&](int code) {
         atomicExch(a.err, code);
         abort_flag = 1;
@@ -295,18 +304,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant_
     if (warp == 0) {
         // ---------------- producer: TMA loads of the A tiles ----------------
         if (lane == 0) {
-            int kt = 0;
+            int kt = 0, s = 0;
+            unsigned lap = 0;  // kt / NS
             for (; kt < nkt && !abort_flag; kt++) {
-                const int s = kt % NS;
-                if (kt >= NS) {
-                    const unsigned pf = ((kt / NS) - 1) & 1;
+                if (lap > 0) {
+                    const unsigned pf = (lap - 1) & 1;
                     if (!mbar_test(&stage_free[s], pf) && !mbar_wait(&stage_free[s], pf)) {
                         fail(1);
                         break;
                     }
+                    // the workers read this slot through the generic proxy; the copies write it
+                    // through the async proxy
+                    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 }
-                mbar_expect_tx(&raw_full[s], MT * a_bytes);
-                for (int mt = 0; mt < MT; mt++) tma_load_2d(A_hi(s, mt), &tmap, (kt0 + kt) * KT, mt * TM, &raw_full[s]);
+                mbar_expect_tx(&raw_full[s], stage_bytes);
+#pragma unroll
+                for (int mt = 0; mt < MT; mt++)
+                    tma_load_2d(base + s * stage_bytes + mt * a_bytes, &tmap, (kt0 + kt) * KT, mt * TM, &raw_full[s]);
+                if (++s == NS) {
+                    s = 0;
+                    lap++;
+                }
             }
             n_issued = kt;
         }
@@ -314,141 +332,166 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant_
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
             const uint32_t idesc = idesc_tf32(TM, 2 * N);
+            const uint64_t bdesc0 = sdesc(sa(ops));  // buffer o's B adds (o op_bytes) >> 4
             for (int kt = 0; kt < nkt && !abort_flag; kt++) {
-                const int s = kt % NS, g = kt / FLUSH;
-                const unsigned ps = (kt / NS) & 1;
-                if (!mbar_test(&split_done[s], ps) && !mbar_wait(&split_done[s], ps)) {
+                const int o = kt % NOP, g = kt / FLUSH, rg = g % NREG;
+                const unsigned po = (kt / NOP) & 1;
+                if (!mbar_test(&op_ready[o], po) && !mbar_wait(&op_ready[o], po)) {
                     fail(2);
                     break;
                 }
                 if (kt % FLUSH == 0 && g >= NREG) {
                     const unsigned pe = ((g / NREG) - 1) & 1;
-                    if (!mbar_test(&acc_empty[g % NREG], pe) && !mbar_wait(&acc_empty[g % NREG], pe)) {
+                    if (!mbar_test(&acc_empty[rg], pe) && !mbar_wait(&acc_empty[rg], pe)) {
                         fail(3);
                         break;
                     }
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                // descriptors of the stage's tiles; a K step of 8 tf32 (32 bytes along the
-                // swizzled row) adds 2 to the start-address field
                 // B_lo's rows follow B_hi's: one MMA of width 2N takes A [B_hi B_lo]; per K step
+                // of 8 (32 bytes along B's swizzled row, 8 TMEM columns of A)
                 // A_hi [B_hi B_lo] + A_lo [B_hi B_lo] (the lo x lo term is below FP32 rounding)
-                const uint64_t b0 = sdesc(sa(B_hi(s)));
+                const uint64_t b0 = bdesc0 + (uint64_t)(((uint32_t)o * op_bytes) >> 4);
 #pragma unroll
                 for (int mt = 0; mt < MT; mt++) {
-                    const uint32_t d = region(g) + mt * 2 * N;
-                    const uint64_t ah0 = sdesc(sa(A_hi(s, mt))), al0 = sdesc(sa(A_lo(s, mt)));
+                    const uint32_t d = tmem + (uint32_t)rg * RCOLS + mt * 2 * N;
+                    const uint32_t ahi = tmem + AC0 + (uint32_t)o * ACOLS + mt * 2 * KT, alo = ahi + KT;
 #pragma unroll
                     for (int ks = 0; ks < KT / 8; ks++) {
-                        const uint64_t o = 2 * ks;
-                        mma_tf32(d, ah0 + o, b0 + o, idesc, (kt % FLUSH != 0 || ks > 0) ? 1 : 0);
-                        mma_tf32(d, al0 + o, b0 + o, idesc, 1);
+                        mma_tf32_ts(d, ahi + 8 * ks, b0 + 2 * ks, idesc, (kt % FLUSH != 0 || ks > 0) ? 1 : 0);
+                        mma_tf32_ts(d, alo + 8 * ks, b0 + 2 * ks, idesc, 1);
                     }
                 }
-                mma_commit(&stage_free[s]);
-                if (kt % FLUSH == FLUSH - 1 || kt == nkt - 1) mma_commit(&acc_full[g % NREG]);
+                mma_commit(&op_free[o]);
+                if (kt % FLUSH == FLUSH - 1 || kt == nkt - 1) mma_commit(&acc_full[rg]);
             }
             mma_commit(&done);  // arrives once every MMA issued above has completed
         }
     } else {
         // ---------------- workers: split A, build B, drain ----------------
-        const int wt = t - 64, quarter = warp & 3, half = (warp - 2) >> 2;
+        const int grp = (warp - 2) >> 2, quarter = warp & 3, wt = (t - 64) & (TM - 1);
+        const int row = quarter * 32 + lane;  // basis vector (TMEM lane) this thread splits
         constexpr int HC = MT * N / 2;
         float acc_hi[HC], acc_lo[HC];
 #pragma unroll
         for (int c = 0; c < HC; c++) acc_hi[c] = acc_lo[c] = 0.f;
-        // B values: worker thread wt < 16 k takes (row np, column c) of each tile; its value
-        // for the next tile is loaded one tile ahead
-        const int bnp = a.ki == 1 ? wt % (KT / 2) : wt / max(a.k, 1);
-        const int bc = a.ki == 1 ? wt / (KT / 2) : wt % max(a.k, 1);
-        const bool bth = wt < (KT / 2) * a.k;
+        // B values: the group's thread wt takes values wt and wt + 128 of a tile's 16 k (row np,
+        // column c); its values for its next tile are loaded one tile ahead
+        constexpr int NBV = N / 16;  // 16 k <= 8 N values over 128 threads
+        static_assert(NBV * TM * 2 >= (KT / 2) * N, "B values over a worker group");
+        int bnp[NBV], bc[NBV];
+        bool bth[NBV];
+#pragma unroll
+        for (int i = 0; i < NBV; i++) {
+            const int v = wt + TM * i;
+            bth[i] = v < (KT / 2) * a.k;
+            bnp[i] = a.ki == 1 ? v % (KT / 2) : v / a.k;
+            bc[i] = a.ki == 1 ? v / (KT / 2) : v % a.k;
+        }
+        float2 bval[NBV];
         auto load_b = [&](int kt) {
-            float2 v = make_float2(0.f, 0.f);
-            const long n = (long)(kt0 + kt) * (KT / 2) + bnp;
-            if (bth && kt < nkt && n < a.nrows)
-                v = a.R[((n >> 1) * a.ki + bc % a.ki) * 2 + (n & 1) + (long)(bc / a.ki) * a.bcol];
-            return v;
+#pragma unroll
+            for (int i = 0; i < NBV; i++) {
+                const long n = (long)(kt0 + kt) * (KT / 2) + bnp[i];
+                bval[i] = make_float2(0.f, 0.f);
+                if (bth[i] && kt < nkt && n < a.nrows)
+                    bval[i] = a.R[((n >> 1) * a.ki + bc[i] % a.ki) * 2 + (n & 1) + (long)(bc[i] / a.ki) * a.bcol];
+            }
         };
         auto drain_group = [&](int g) {  // warp-uniform
-            const bool ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[g % NREG], (g / NREG) & 1));
+            const unsigned pa = (g / NREG) & 1;
+            const bool ok = __all_sync(0xffffffffu, mbar_test(&acc_full[g % NREG], pa) || mbar_wait(&acc_full[g % NREG], pa));
             if (!ok) {
                 fail(4);
                 return false;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            drain<MT, N>(region(g), quarter, half, acc_hi, acc_lo);
+            drain<MT, N>(tmem + (uint32_t)((g % NREG) * RCOLS), quarter, grp, acc_hi, acc_lo);
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(&acc_empty[g % NREG]);
             return true;
         };
-        float2 bcur = load_b(0);
-        int kt = 0;
+        load_b(grp);
+        int nd = 0;  // flush groups drained
         bool ok = true;
-        for (; kt < nkt && ok && !abort_flag; kt++) {
-            const int s = kt % NS, g = kt / FLUSH;
-            const float2 bnext = load_b(kt + 1);
-            if (!__all_sync(0xffffffffu, mbar_wait(&raw_full[s], (kt / NS) & 1))) {
+        int kt = grp;
+        for (; kt < nkt && ok && !abort_flag; kt += 2) {
+            const int s = kt % NS, o = kt % NOP, g = kt / FLUSH;
+            const unsigned pr = (kt / NS) & 1, pp = ((kt / NOP) - 1) & 1;
+            if (!__all_sync(0xffffffffu, mbar_test(&raw_full[s], pr) || mbar_wait(&raw_full[s], pr))) {
                 fail(5);
                 break;
             }
-            // split A in place: hi (low mantissa bits cleared), lo = x - hi
-            for (int mt = 0; mt < MT; mt++) {
-                float4 *ah = reinterpret_cast<float4 *>(A_hi(s, mt));
-                float4 *al = reinterpret_cast<float4 *>(A_lo(s, mt));
-                for (int i = wt; i < TM * KT / 4; i += 32 * WORKERS) {
-                    const float4 v = ah[i];
-                    const float4 h = make_float4(hi_tf32(v.x), hi_tf32(v.y), hi_tf32(v.z), hi_tf32(v.w));
-                    ah[i] = h;
-                    al[i] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
-                }
+            if (kt >= NOP && !__all_sync(0xffffffffu, mbar_test(&op_free[o], pp) || mbar_wait(&op_free[o], pp))) {
+                fail(6);
+                break;
             }
-            // B tile: rows c (B1) and k + c (B2), K positions 2n' and 2n' + 1 for complex row n'
-            unsigned char *bh = B_hi(s), *bl = B_lo(s);
-            for (int i = 2 * a.k * KT + wt; i < N * KT; i += 32 * WORKERS) {  // zero padding rows
-                const int r = i / KT, e = i % KT;
-                *reinterpret_cast<float *>(bh + sw128(r, e)) = 0.f;
-                *reinterpret_cast<float *>(bl + sw128(r, e)) = 0.f;
-            }
-            if (bth) {
-                const float vals[4] = {bcur.x, bcur.y, bcur.y, -bcur.x};  // B1 (re, im), B2 (im, -re)
+            // the MMAs that read this buffer's previous contents have completed (op_free)
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-                    const int r = q < 2 ? bc : a.k + bc;
-                    const int e = 2 * bnp + (q & 1);
-                    const float h = hi_tf32(vals[q]);
-                    *reinterpret_cast<float *>(bh + sw128(r, e)) = h;
-                    *reinterpret_cast<float *>(bl + sw128(r, e)) = vals[q] - h;
+            for (int mt = 0; mt < MT; mt++) {
+                // this thread's row: 32 floats, swizzled by 16-byte chunks
+                const unsigned char *src = base + s * stage_bytes + mt * a_bytes + (row >> 3) * 1024 + (row & 7) * 128;
+                float hv[KT], lv[KT];
+#pragma unroll
+                for (int c = 0; c < KT / 4; c++) {
+                    const float4 v = *reinterpret_cast<const float4 *>(src + ((c ^ (row & 7)) << 4));
+                    const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        hv[4 * c + e] = hi_tf32(x[e]);
+                        lv[4 * c + e] = x[e] - hv[4 * c + e];
+                    }
                 }
+                if (mt == MT - 1) {  // the staging slot has been read
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&stage_free[s]);
+                }
+                const uint32_t ta = tmem + ((uint32_t)(quarter * 32) << 16) + AC0 + (uint32_t)o * ACOLS + mt * 2 * KT;
+                tmem_st32(ta, hv);
+                tmem_st32(ta + KT, lv);
             }
-            bcur = bnext;
+            // B tile: rows c (B1 = re, im) and k + c (B2 = im, -re), K positions 2n' and 2n' + 1
+            // for complex row n'
+            unsigned char *bh = ops + o * op_bytes, *bl = bh + b_bytes;
+#pragma unroll
+            for (int i = 0; i < NBV; i++)
+                if (bth[i]) {
+                    const float2 h = make_float2(hi_tf32(bval[i].x), hi_tf32(bval[i].y));
+                    const float2 l = make_float2(bval[i].x - h.x, bval[i].y - h.y);
+                    const uint32_t p1 = sw128(bc[i], 2 * bnp[i]), p2 = sw128(a.k + bc[i], 2 * bnp[i]);
+                    *reinterpret_cast<float2 *>(bh + p1) = h;
+                    *reinterpret_cast<float2 *>(bl + p1) = l;
+                    *reinterpret_cast<float2 *>(bh + p2) = make_float2(h.y, -h.x);
+                    *reinterpret_cast<float2 *>(bl + p2) = make_float2(l.y, -l.x);
+                }
+            load_b(kt + 2);
+            asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             __syncwarp();
-            if (lane == 0) mbar_arrive(&split_done[s]);
-            // drain the group two behind the one this tile starts
-            if (kt % FLUSH == 0 && g >= 2) ok = drain_group(g - 2);
+            if (lane == 0) mbar_arrive(&op_ready[o]);
+            while (ok && nd <= g - (NREG - 1)) ok = drain_group(nd++);
         }
-        if (wt == 0) n_consumed = kt;
-        if (ok && kt == nkt && !abort_flag) {
-            // the last two groups
-            for (int g = max(0, ngroups - 2); g < ngroups && ok; g++) ok = drain_group(g);
+        if (ok && kt >= nkt && !abort_flag) {
+            while (ok && nd < ngroups) ok = drain_group(nd++);
             if (ok) {
                 double *P = a.partials + (long)blockIdx.x * MT * TM * N;
 #pragma unroll
                 for (int j = 0; j < HC; j++) {
-                    const int col = half * HC + j;  // TMEM column within the region: mt * N + c
-                    const int row = (col / N) * TM + quarter * 32 + lane;
-                    P[(long)row * N + col % N] = (double)acc_hi[j] + (double)acc_lo[j];
+                    const int col = grp * HC + j;  // output column: mt * N + c
+                    P[(long)((col / N) * TM + row) * N + col % N] = (double)acc_hi[j] + (double)acc_lo[j];
                 }
             }
         }
     }
     __syncthreads();
-    if (t == 0) {
-        // after an abort: let the loads still in flight land, and every MMA complete
-        for (int j = n_consumed; j < n_issued; j++) mbar_wait(&raw_full[j % NS], (j / NS) & 1);
-    }
-    if (!mbar_wait(&done, 0)) atomicExch(a.err, 6);
+    // after an abort: let the copies still in flight land (the last one issued on each staging
+    // slot; a slot's earlier phases completed before it was refilled), and every MMA complete
+    if (t == 0)
+        for (int j = max(0, n_issued - NS); j < n_issued; j++) mbar_wait(&raw_full[j % NS], (j / NS) & 1);
+    if (!mbar_wait(&done, 0)) atomicExch(a.err, 8);
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     __syncthreads();
     if (warp == 0)
@@ -456,19 +499,27 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tc_ahb(const __grid_constant_
 }
 
 // C[a][c] = sum over CTAs of D[a][c] + i D[a][k + c], FP64, fixed order
+// (eight lanes per output, over the CTAs)
 __global__ void k_tc_reduce(const double *partials, int grid, int MT, int N, int l, int k, double *C) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= l * k) return;
+    const int idx = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, sub = threadIdx.x & 7;
     const int arow = idx / k, c = idx % k;
     double re = 0.0, im = 0.0;
     const long stride = (long)MT * TM * N;
-    for (int g = 0; g < grid; g++) {
-        const double *P = partials + g * stride + (long)arow * N;
-        re += P[c];
-        im += P[k + c];
+    if (idx < l * k)
+        for (int g = sub; g < grid; g += 8) {
+            const double *P = partials + g * stride + (long)arow * N;
+            re += P[c];
+            im += P[k + c];
+        }
+#pragma unroll
+    for (int off = 4; off > 0; off >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, off);
+        im += __shfl_xor_sync(0xffffffffu, im, off);
     }
-    C[2 * idx] = re;
-    C[2 * idx + 1] = im;
+    if (sub == 0 && idx < l * k) {
+        C[2 * idx] = re;
+        C[2 * idx + 1] = im;
+    }
 }
 
 // ------------------------------------------------------------------------------------
@@ -950,20 +1001,22 @@ cudaError_t launch_tc_ahb(const ColSet &A, const ColSet &B, long nrows, double *
         if (ev[0] == '1') a.inject_ns = 5000000ull;  // 5 ms
     int grid = 0;
     tc_grid(a.ktiles, &a.chunk, &grid);
-    const size_t stage = 2 * MT * (size_t)(TM * KT * 4) + 2 * (size_t)((N + 7) / 8) * 1024;
-    const size_t smem = (MT == 1 ? 5 : 3) * stage + 1024;  // stages of the TMA ring (k_tc_ahb's NS)
+    const size_t opb = 2 * (size_t)((N + 7) / 8) * 1024;
+    const size_t smem = (MT == 1 ? (size_t)AhbShape<1>::NS * TM * KT * 4 + AhbShape<1>::NOP * opb
+                                 : (size_t)AhbShape<2>::NS * 2 * TM * KT * 4 + AhbShape<2>::NOP * opb) +
+                        1024;
     auto go = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         kern<<<grid, TC_THREADS, smem, s>>>(map, a);
     };
-    if (MT == 1 && N == 16) go(k_tc_ahb<1, 16, 5>);
-    else if (MT == 1) go(k_tc_ahb<1, 32, 5>);
-    else if (N == 16) go(k_tc_ahb<2, 16, 3>);
-    else go(k_tc_ahb<2, 32, 3>);
+    if (MT == 1 && N == 16) go(k_tc_ahb<1, 16>);
+    else if (MT == 1) go(k_tc_ahb<1, 32>);
+    else if (N == 16) go(k_tc_ahb<2, 16>);
+    else go(k_tc_ahb<2, 32>);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int n = l * k;
-    k_tc_reduce<<<(n + 127) / 128, 128, 0, s>>>(partials, grid, MT, N, l, k, C);
+    k_tc_reduce<<<(8 * n + 127) / 128, 128, 0, s>>>(partials, grid, MT, N, l, k, C);
     return cudaGetLastError();
 }
 
