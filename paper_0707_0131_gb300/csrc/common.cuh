@@ -299,52 +299,51 @@ __device__ __forceinline__ double block_reduce_rhs(double v, int k, double *smem
     return s;
 }
 
-// Last-block completion: every block writes its per-rhs partials, then the block
-// that arrives last sums all partials in block order (deterministic) and runs
-// `finish(rhs, total)` for each rhs.  counter must be zero on entry; it is reset.
+// Last-block completion for kernels whose blocks have written their k per-RHS partial sums to
+// partials[blockIdx.x * k + r], from threads of warp 0: the block that arrives last sums all
+// partials in block order (deterministic) and runs `finish(rhs, total)` for each rhs.  counter
+// must be zero on entry; it is reset.
+//
+// This tail is serial time at the end of every CG kernel, so it is kept short: only warp 0
+// fences (the partials are all that the last block reads; with every thread fencing, each
+// waited for its own field stores), and the partials are loaded eight at a time before they are
+// added (one dependent load per step took most of the tail).
 template <typename F>
-__device__ __forceinline__ void grid_reduce_rhs(double blocksum, int k, double *partials, unsigned *counter,
-                                                double *smem, F finish) {
+__device__ __forceinline__ void grid_finish_rhs(int k, double *partials, unsigned *counter, double *smem, F finish) {
     __shared__ bool am_last;
-    if (threadIdx.x < k) partials[(long)blockIdx.x * k + threadIdx.x] = blocksum;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned prev = atomicAdd(counter, 1u);
-        am_last = (prev == gridDim.x - 1);
+    if (threadIdx.x < 32) {
+        __threadfence();
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            const unsigned prev = atomicAdd(counter, 1u);
+            am_last = (prev == gridDim.x - 1);
+            __threadfence();
+        }
     }
     __syncthreads();
     if (!am_last) return;
-    __threadfence();
     // each thread sums a strided set of blocks for its rhs, in fixed order
-    const int r = threadIdx.x % k;
+    const int r = threadIdx.x % k, step = blockDim.x / k;
     double s = 0.0;
-    for (long b = threadIdx.x / k; b < gridDim.x; b += blockDim.x / k) s += __ldcg(partials + b * k + r);
+    for (long b = threadIdx.x / k; b < gridDim.x; b += 8 * step) {
+        double v[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) v[i] = b + i * step < gridDim.x ? __ldcg(partials + (b + i * step) * k + r) : 0.0;
+#pragma unroll
+        for (int i = 0; i < 8; i++)
+            if (b + i * step < gridDim.x) s += v[i];
+    }
     double tot = block_reduce_rhs(s, k, smem);
     if (threadIdx.x < k) finish(threadIdx.x, tot);
     if (threadIdx.x == 0) *counter = 0u;
 }
 
-// As grid_reduce_rhs, for kernels whose blocks have already written their k
-// per-RHS partial sums to partials[blockIdx.x * k + r].
+// The same, writing the block's partial sums first (blocksum of thread r < k for rhs r).
 template <typename F>
-__device__ __forceinline__ void grid_finish_rhs(int k, double *partials, unsigned *counter, double *smem, F finish) {
-    __shared__ bool am_last;
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned prev = atomicAdd(counter, 1u);
-        am_last = (prev == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!am_last) return;
-    __threadfence();
-    const int r = threadIdx.x % k;
-    double s = 0.0;
-    for (long b = threadIdx.x / k; b < gridDim.x; b += blockDim.x / k) s += __ldcg(partials + b * k + r);
-    double tot = block_reduce_rhs(s, k, smem);
-    if (threadIdx.x < k) finish(threadIdx.x, tot);
-    if (threadIdx.x == 0) *counter = 0u;
+__device__ __forceinline__ void grid_reduce_rhs(double blocksum, int k, double *partials, unsigned *counter,
+                                                double *smem, F finish) {
+    if (threadIdx.x < k) partials[(long)blockIdx.x * k + threadIdx.x] = blocksum;
+    grid_finish_rhs(k, partials, counter, smem, finish);
 }
 
 }  // namespace eig
