@@ -602,12 +602,20 @@ struct Solve {
         sync(s);
     }
     void write_scalars() { CUDA_CK(cudaMemcpyAsync(st, sth, sizeof(CGScalars) * k, cudaMemcpyHostToDevice, s)); }
-    void read_history(int upto) {
+    // rows 0 .. upto + 1 of alpha, beta and rho in one strided copy
+    void copy_history(int upto) {
         double *hh = op->hist_h.as<double>();
-        const size_t n = (size_t)(upto + 2) * k;
-        CUDA_CK(cudaMemcpyAsync(hh, h.alpha, n * sizeof(double), cudaMemcpyDeviceToHost, s));
-        CUDA_CK(cudaMemcpyAsync(hh + (size_t)h.cap * k, h.beta, n * sizeof(double), cudaMemcpyDeviceToHost, s));
-        CUDA_CK(cudaMemcpyAsync(hh + 2 * (size_t)h.cap * k, h.rho, n * sizeof(double), cudaMemcpyDeviceToHost, s));
+        const size_t pitch = (size_t)h.cap * k * sizeof(double), width = (size_t)(upto + 2) * k * sizeof(double);
+        CUDA_CK(cudaMemcpy2DAsync(hh, pitch, h.alpha, pitch, width, 3, cudaMemcpyDeviceToHost, s));
+    }
+    void read_history(int upto) {
+        copy_history(upto);
+        sync(s);
+    }
+    // scalars and history with one synchronisation (a host check)
+    void read_state(int upto) {
+        CUDA_CK(cudaMemcpyAsync(sth, st, sizeof(CGScalars) * k, cudaMemcpyDeviceToHost, s));
+        copy_history(upto);
         sync(s);
     }
     const double *ha() const { return op->hist_h.as<double>(); }
@@ -834,7 +842,7 @@ static bool cg_run(Solve &sv, int max_iter, Window *w, eig_op_s *op) {
     while (true) {
         const bool restart_now = w && w->i == w->m;
         if (since >= next_check || restart_now || sv.j >= max_iter) {
-            sv.read_scalars();
+            sv.read_state(sv.j);
             bool any = false;
             for (int q = 0; q < k; q++) any = any || sv.sth[q].active;
             if (w && !any && sv.sth[0].iters < sv.j) {
@@ -849,7 +857,6 @@ static bool cg_run(Solve &sv, int max_iter, Window *w, eig_op_s *op) {
             }
             if (!any) break;
             if (sv.j >= max_iter) return false;
-            sv.read_history(sv.j);
             const bool rel = sv.needs_reliable();
             if (rel) {
                 sv.reliable_update();
