@@ -546,7 +546,7 @@ def main():
     launches = int(sum(v["launches"] for v in prof.values()))
     # roofline of the dominant kernel: the one with the most device time in the timed
     # region, whatever it is; every kernel of the path is HBM-bound at this size except
-    # the FP64 / double-float stencils (arithmetic), reported against the FMA roofs below
+    # the FP64 stencils (arithmetic), reported against the FMA roof below
     kern = max(prof, key=lambda n: prof[n]["ms"])
     kp = prof[kern]
     peaks_path = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -583,7 +583,8 @@ def main():
         gbs = (v["bytes"] / (v["ms"] / 1e3) / 1e9) if v["ms"] > 0 else None
         e = {"launches": v["launches"], "ms": round(v["ms"], 3), "GBps": gbs,
              "frac_of_hbm": (gbs / peak) if gbs else None}
-        # FP64 stencils: ~1320 flop per site and RHS for one M (spin-projected count)
+        # FP64 stencils: ~1320 flop per site and RHS for one M (spin-projected count); the hops
+        # run on the integer pipes (dslash_fx.cu), so the FP64 FMA roof does not bound them
         if n.startswith("dslash_") and "f64" in n and v["ms"] > 0 and alu.get("fp64_tflops"):
             kk_ = int(n.rsplit("_k", 1)[1]) if "_k" in n else 1
             tf = 1320.0 * V * kk_ * v["launches"] / (v["ms"] / 1e3) / 1e12
@@ -727,7 +728,7 @@ def main():
                                       f"basis {l0} FP32 vectors, tol {a.tol}, restart {a.restart_tol}",
                           "lattice": a.lattice, "k": k, "basis": l0, "storage": ("fp32 spinors, fp32 links (12- and 18-real resident, chosen per k by the autotuner), " if a.prec == 32 else
                                      "fp16 spinors with one fp32 scale per site and RHS, fp32 12-real links, fp32 eigCG window and basis, ") +
-                          f"double-float residual replacements (delta {a.reliable_delta}), fp64 final residual", "l2": "inputs larger than L2 (each field >= 85 MB)",
+                          f"fp64 residual replacements (delta {a.reliable_delta}) and final residual", "l2": "inputs larger than L2 (each field >= 85 MB)",
                           "parallelism": f"replicas{world}"},
                "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": launches,
                "clocks": clk, "p50_ms": serve["p50_ms"] if serve else None,

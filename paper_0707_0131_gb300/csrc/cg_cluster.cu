@@ -13,7 +13,7 @@
 // stopping decisions are the same everywhere.  One launch runs up to 16 iterations; CTA 0 keeps
 // the device scalars.
 //
-// 8^4, one RHS: 13.6 us per iteration (whole solve to 1e-8 at cond 1e4: 5.2 -> 4.2 ms); 4^4: 9.1.
+// 8^4, one RHS: 13.6 us per iteration (whole solve to 1e-8 at cond 1e4: 5.2 -> 4.0 ms); 4^4: 9.1.
 // About 4 us of it are the FP64 sums and divisions of the two reductions, most of the rest the
 // stencils' latency at two warps per sub-partition.  Nothing in the loop touches global memory
 // but the window: the barrier's release waits for global stores, and its acquire drops the links

@@ -16,8 +16,8 @@
 // FP32 accuracy.
 // The tensor pipe's own FP32 accumulation loses accuracy with the length of the
 // sum (measured at 10.6M complex rows: relative error 1e-6 after 2 K tiles per
-// accumulator, 3e-5 after 128), so TMEM holds two accumulators used by alternate
-// groups of two K tiles; each finished group is drained into per-thread
+// accumulator, 3e-5 after 128), so TMEM holds two or three accumulators that take
+// turns on groups of two K tiles; each finished group is drained into per-thread
 // double-float (TwoSum) sums while the next group accumulates.  Each CTA writes
 // its sums as FP64 partials; a second kernel adds the partials in a fixed order.
 //
