@@ -546,7 +546,7 @@ def main():
     launches = int(sum(v["launches"] for v in prof.values()))
     # roofline of the dominant kernel: the one with the most device time in the timed
     # region, whatever it is; every kernel of the path is HBM-bound at this size except
-    # the FP64 stencils (arithmetic), reported against the FMA roof below
+    # the FP64 stencils (integer arithmetic), whose FP64-equivalent rate is given below
     kern = max(prof, key=lambda n: prof[n]["ms"])
     kp = prof[kern]
     peaks_path = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -584,12 +584,11 @@ def main():
         e = {"launches": v["launches"], "ms": round(v["ms"], 3), "GBps": gbs,
              "frac_of_hbm": (gbs / peak) if gbs else None}
         # FP64 stencils: ~1320 flop per site and RHS for one M (spin-projected count); the hops
-        # run on the integer pipes (dslash_fx.cu), so the FP64 FMA roof does not bound them
+        # run on the integer pipes (dslash_fx.cu), so the FP64 FMA roof of alu_peaks is no bound
         if n.startswith("dslash_") and "f64" in n and v["ms"] > 0 and alu.get("fp64_tflops"):
             kk_ = int(n.rsplit("_k", 1)[1]) if "_k" in n else 1
             tf = 1320.0 * V * kk_ * v["launches"] / (v["ms"] / 1e3) / 1e12
             e["fp64_tflops"] = tf
-            e["frac_of_fp64_fma"] = tf / alu["fp64_tflops"]
         kernels[n] = e
 
     # --- end to end: same steps with pinned host buffers -----------------------------

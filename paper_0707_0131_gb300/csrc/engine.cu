@@ -75,6 +75,16 @@ struct DevBuf {
         }
         n = bytes;
     }
+    // false (and empty) where alloc would report EIG_ERR_OOM
+    bool try_alloc(size_t bytes) {
+        try {
+            alloc(bytes);
+        } catch (const Error &e) {
+            if (e.st != EIG_ERR_OOM) throw;
+            return false;
+        }
+        return true;
+    }
     void ensure(size_t bytes) {
         if (bytes > n) alloc(bytes);
     }
@@ -355,9 +365,14 @@ static void ensure_workspace(eig_op_s *op) {
         op->full64.alloc(P64, V, K);
         op->be64.alloc(P64, Vf, K);
     }
-    op->nat_in.alloc(fx_field_bytes(V * K));  // at least V * 12 * 16 * K
+    if (op->gauge_fx.p && !(op->fx_ex.try_alloc((size_t)Vf * K * sizeof(int)) &&
+                            op->nat_in.try_alloc(fx_field_bytes(V * K)))) {  // at least V * 12 * 16 * K
+        // the fixed-point form is optional: without room for it the FP64 stencil does its work
+        op->fx_ex.release();
+        op->gauge_fx.release();
+    }
+    if (!op->nat_in.p) op->nat_in.alloc((size_t)V * 12 * 16 * K);
     op->nat_out.alloc((size_t)V * 12 * 16 * K);
-    if (op->gauge_fx.p) op->fx_ex.alloc((size_t)Vf * K * sizeof(int));
     op->ws = true;
 }
 
@@ -1475,12 +1490,12 @@ eig_status eig_op_create(const double *gauge, const int dims[4], double m_q, con
     CUDA_CK(cudaMemcpy(stage.p, gauge, stage.n, cudaMemcpyHostToDevice));
     op->gauge64.alloc((size_t)V * 4 * 9 * 16);
     CUDA_CK(launch_pack_gauge(stage.as<double>(), op->gauge64.p, GF_F64_18, V, 0));
-    if (op->Vf * K >= FX_MIN) {
-        // the links as limbs of the fixed-point FP64 stencil, unless one is not unitary
+    if (op->Vf * K >= FX_MIN && op->gauge_fx.try_alloc(fx_link_bytes(V))) {
+        // the links as limbs of the fixed-point FP64 stencil, unless one is not unitary (or there
+        // is no room for them)
         eig::DevBuf bad;
         int h_bad = 1;
         bad.alloc(sizeof(int));
-        op->gauge_fx.alloc(fx_link_bytes(V));
         CUDA_CK(cudaMemset(bad.p, 0, sizeof(int)));
         CUDA_CK(launch_links_fx(op->gauge64.p, op->gauge_fx.p, V, bad.as<int>(), 0));
         CUDA_CK(cudaMemcpy(&h_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost));

@@ -163,7 +163,10 @@ int dslash32_choice(const DslashCall &c, int *variant);
 cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Field t_save, CGScalars *st, History h,
                              int iter, bool set_rho, RedScratch red, cudaStream_t s);
 // From this many (site, RHS) pairs on, FP64 launches of operators with unitary links take it.
-constexpr long FX_MIN = 6144;
+// Per product, conversion to fixed point included, against the hops spread over lanes
+// (dslash_split.cuh): 4096 pairs 27 : 17 us, 6144 27 : 21, 8192 27 : 26, 16384 29 : 38, 41472
+// 31 : 78 (one wave of latency on this side, FP64 issue time on the other).
+constexpr long FX_MIN = 8192;
 size_t fx_field_bytes(long n);
 size_t fx_link_bytes(long V);
 cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaStream_t s);

@@ -1,4 +1,4 @@
-"""The fixed-point FP64 stencil (launches of at least 6144 (site, RHS) pairs, unitary links).
+"""The fixed-point FP64 stencil (launches of at least 8192 (site, RHS) pairs, unitary links).
 
 Each neighbour enters with at most 2^-55 of the largest component of the eight (alignment and limb
 truncation), so on Gaussian vectors (largest of ~200 components about 4.5 standard deviations,
@@ -10,6 +10,7 @@ import pytest
 
 import oracle
 from oracle import wilson_eo
+from paper_0707_0131_gb300 import _lib
 from paper_0707_0131_gb300 import fixtures as fx
 
 pytestmark = pytest.mark.gpu
@@ -30,13 +31,13 @@ def _rel(out, ref):
     return np.linalg.norm(out - ref) / np.linalg.norm(ref)
 
 
-@pytest.mark.parametrize("dims,k", [((7, 9, 5, 21), 1), ((2, 3, 64, 16), 1), ((8, 8, 8, 8), 2), ((5, 6, 7, 5), 16)])
+@pytest.mark.parametrize("dims,k", [((7, 9, 7, 21), 1), ((2, 3, 64, 22), 1), ((8, 8, 8, 8), 2), ((5, 6, 7, 5), 16)])
 def test_products(api, dims, k):
     gauge = fx.make_gauge(dims, 71)
     W = oracle.Wilson(dims, -0.1, gauge)
     op = api.Op(gauge, dims, -0.1, prec=64, max_rhs=k)
     psi = fx.make_rhs(dims, 72, k).reshape(k, -1)
-    assert psi.shape[1] // 12 * k >= 6144
+    assert psi.shape[1] // 12 * k >= 8192
     for which, f in [(0, W.M), (1, W.Mdag), (2, W.A)]:
         out = np.empty_like(psi)
         op.apply(which, psi, out, k)
@@ -119,4 +120,29 @@ def test_links_that_are_not_unitary_keep_fp64(api):
     op.apply(0, psi, out, k)
     for r in range(k):
         assert _rel(out[r], np.asarray(W.M(psi[r])).reshape(-1)) < 1e-12
+    op.close()
+
+
+@pytest.mark.parametrize("when", ["links", "workspace"])
+def test_no_room_for_the_fixed_point_form(api, monkeypatch, when):
+    """An allocation limit that fits the FP64 links and fields but not their fixed-point forms
+    (rounded up to 32 elements): the operator works with the FP64 stencil."""
+    dims = (7, 9, 15, 31)  # the links larger than the 16 MB of reduction scratch
+    V = int(np.prod(dims))
+    assert V % 32
+    gauge = fx.make_gauge(dims, 71)
+    W = oracle.Wilson(dims, -0.1, gauge)
+    psi = fx.make_rhs(dims, 72, 1).reshape(-1)
+    op = api.Op(gauge, dims, -0.1, prec=64, max_rhs=1)
+    full = _lib.eig_op_trim(op.h)
+    if when == "links":
+        op.close()
+        monkeypatch.setenv("EIG_TEST_ALLOC_LIMIT", str(V * 576))
+        op = api.Op(gauge, dims, -0.1, prec=64, max_rhs=1)
+    else:
+        monkeypatch.setenv("EIG_TEST_ALLOC_LIMIT", str(V * 192))
+    out = np.empty_like(psi)
+    op.apply(2, psi, out, 1)
+    assert _rel(out, np.asarray(W.A(psi)).reshape(-1)) < 1e-15
+    assert _lib.eig_op_trim(op.h) < full  # no exponents, no rounding of the field
     op.close()
