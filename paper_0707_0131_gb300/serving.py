@@ -38,6 +38,14 @@ from .api import Basis, Op
 from .policy import SwitchPolicy
 
 
+# A basis is the work of the eigCG solves that grew it, milliseconds each on small lattices: an
+# operator keeps it while its requests come less than KEEP_IDLE_S apart, unless the operator that
+# needs the room has waited KEEP_WAIT_S.  Without it, two operators that take turns and each finish
+# before their next request would close each other every time, and no basis would ever be used.
+KEEP_IDLE_S = 0.05
+KEEP_WAIT_S = 0.5
+
+
 @dataclass
 class OpSpec:
     key: str
@@ -244,6 +252,7 @@ class Server:
     # admission by HBM budget: activate the operator; first take workspaces back from idle
     # operators (their bases stay), then close the least recently used idle operator
     def _admit(self, w: _Worker):
+        asked = time.perf_counter()
         with self.cv:
             while not w.active:
                 need = w.spec.workspace_bytes() + (0 if w.resident else w.spec.resident_bytes())
@@ -271,6 +280,11 @@ class Server:
                 resident_idle = [o for o in idle if o.resident and not o.active]
                 if resident_idle:
                     victim = min(resident_idle, key=lambda o: o.last_used)
+                    now = time.perf_counter()
+                    keep = min(victim.last_used + KEEP_IDLE_S, asked + KEEP_WAIT_S) - now
+                    if keep > 0:
+                        self.cv.wait(timeout=min(0.05, keep))
+                        continue
                     victim.close()
                     self.used -= victim.spec.resident_bytes()
                     self.closes += 1
