@@ -27,8 +27,8 @@
 #include <cstring>
 #include <mutex>
 
+#include "cg_scalars.cuh"
 #include "dslash32.cuh"
-#include "dslash_split.cuh"
 #include "prof.h"
 
 namespace eig {

@@ -297,7 +297,7 @@ __global__ void __launch_bounds__(128) k_dslash(const KArgs a) {
 
 static_assert((int)EPI_PLAIN == (int)SPL_PLAIN && (int)EPI_NORM == (int)SPL_NORM && (int)EPI_CG == (int)SPL_CG &&
                   (int)EPI_RESID == (int)SPL_RESID,
-              "epilogue numbers shared with dslash_split.cuh");
+              "epilogue numbers shared with cg_scalars.cuh");
 
 // ------------------------------------------------------------------------------------
 // launch plumbing
@@ -393,9 +393,10 @@ static std::string dslash_name(int epi, Prec p, int k) {
     return n;
 }
 
-// FP64 launches of n (site, RHS) pairs that the fixed-point form does not take: spread the hops over lanes (dslash_split.cuh) while
-// the FP64 issue time of the fullest SM sub-partition is shorter that way.  One thread per
-// pair costs ~912 FP64 warp instructions per 32 pairs, the split form ~62 per 2 pairs; both
+// FP64 launches of n (site, RHS) pairs that the fixed-point form does not take: spread the hops
+// over lanes (dslash_split.cuh) while the FP64 issue time of the fullest SM sub-partition is
+// shorter that way.  One thread per
+// pair costs ~912 FP64 warp instructions per 32 pairs, the split form ~68 per 2 pairs; both
 // run in whole warps per sub-partition.
 static bool split64(long n) {
     if (n > SPLIT_MAX) return false;
@@ -450,7 +451,7 @@ static cudaError_t dispatch(const DslashCall &c, KArgs &a, int cap, cudaStream_t
         b.tsave = a.tsave.data;
         b.save_t = a.save_t;
         b.set_rho = a.set_rho;
-        return split_launch<double, GF_F64_18, EPI>(c.dagger, b, cap, s);
+        return split_launch<EPI>(c.dagger, b, cap, s);
     }
     if (c.nat_in || c.nat_out) return cudaErrorInvalidValue;
 #define EIG_LAUNCH(S, GF)                                                                   \

@@ -1,19 +1,19 @@
-// Internal header: the Wilson stencil with the hops of a site spread over lanes, for
+// Internal header: the FP64 Wilson stencil with the hops of a site spread over lanes, for
 // launches with too few (site, RHS) pairs to fill the GPU one thread each.
 //
-// Same operator, layouts and epilogues as dslash.cu / dslash32.cuh.  There one thread
-// walks the eight hops of a site: on a small lattice that is one long serial chain on a
-// few SMs (4^4: two blocks; GB300 issues an FP64 warp instruction about every 64 cycles,
-// so the ~900 FP64 instructions of a site took 37 us with 150 SMs idle; in FP32 the chain
-// is eight dependent rounds of loads, 5-7 us).  Here 16 lanes share a (site, RHS): lane
+// Same operator, layouts and epilogues as dslash.cu.  There one thread walks the eight hops
+// of a site: on a small lattice that is one long serial chain on a few SMs (4^4: two blocks;
+// GB300 issues an FP64 warp instruction about every 64 cycles, so the ~900 FP64 instructions
+// of a site took 37 us with 150 SMs idle).  Here 16 lanes share a (site, RHS): lane
 // 2 h + s forms spin component s of the half spinor of hop h (three colours), multiplies it
 // by the link and leaves the product in shared memory; lanes 0..11 then each sum one
 // complex component of the output over the eight hops and run the epilogue on it.  The
-// arithmetic per site is the same but for the reduction, about 31 FP64 warp instructions
+// arithmetic per site is the same but for the reduction, about 34 FP64 warp instructions
 // per site against 28.5, so the one-thread form stays for lattices that fill the GPU.
 #pragma once
 #include <cstring>
 
+#include "cg_scalars.cuh"
 #include "fastdiv.h"
 #include "kernels.cuh"
 
@@ -21,18 +21,14 @@ namespace eig {
 
 struct SplitArgs {
     const void *in;
-    const float *in_s;
     void *out;
-    float *out_s;
     const void *cen;  // centre-term input (odd-even form), else in; null: hops only
-    const float *cen_s;
     void *r;
-    float *r_s;
     const void *b;    // residual epilogue
     void *tsave;
     const void *g;
-    // complex-component, site and RHS strides of in and out, in chunks (FP64: one complex
-    // per chunk, so the natural layout of the API can be read and written as it is)
+    // complex-component, site and RHS strides of in and out, so that the natural layout
+    // of the API can be read and written as it is
     unsigned in_c, in_x, in_r, out_c, out_x, out_r;
     unsigned L0, L1, L2, L3, V, Vg, lh;
     FastDiv d0, d1, d2, dh;
@@ -51,101 +47,27 @@ struct SplitArgs {
 // largest number of (site, RHS) pairs the split launchers take (32-bit offsets)
 constexpr long SPLIT_MAX = 1L << 20;
 
-// epilogues: the numbers of dslash.cu's Epi and dslash32.cuh's E_*
-enum { SPL_PLAIN = 0, SPL_NORM = 1, SPL_CG = 2, SPL_RESID = 3 };
-
 namespace {
 
-// the scalar updates of RHS r after a grid reduction gave tot (Fig. 1 steps 12, 4, 8; see
-// kernels.cuh for the launches they belong to)
-template <int EPI>
-__device__ __forceinline__ void finish_scalars(CGScalars *sts, double *h_alpha, double *h_beta, double *h_rho, int iter,
-                                               int k, int set_rho, int r, double tot) {
-    CGScalars &st = sts[r];
-    const long hi = (long)iter * k + r;
-    if (EPI == SPL_NORM) {
-        if (st.active) {
-            st.pAp = tot;
-            if (!(tot > 0.0) || !isfinite(tot)) {
-                st.breakdown = 1;
-                st.active = 0;
-                st.alpha = 0.0;
-            } else {
-                st.alpha = st.rho / tot;
-            }
-            h_alpha[hi] = st.alpha;
-            st.x_pending = st.active;
-        } else {
-            st.alpha = 0.0;
-            st.x_pending = 0;
-        }
-    } else if (EPI == SPL_CG) {
-        if (st.active) {
-            if (!isfinite(tot)) {
-                st.breakdown = 1;
-                st.active = 0;
-                return;
-            }
-            st.iters = iter;
-            st.nit++;
-            st.rho_prev = st.rho;
-            st.rho = tot;
-            st.beta = tot / st.rho_prev;
-            h_rho[hi] = tot;
-            h_beta[hi + k] = st.beta;
-            if (tot <= st.target) st.active = 0;
-        }
-    } else if (EPI == SPL_RESID) {
-        st.aux = tot;
-        if (set_rho) {
-            st.rho = tot;
-            st.beta = tot / st.rho_prev;
-            h_rho[hi] = tot;
-            h_beta[hi + k] = st.beta;
-        }
-    }
+// complex component e of the spinor at offset o = site stride * site + RHS stride * RHS,
+// component stride cs
+__device__ __forceinline__ Cx<double> load_comp(const void *p, unsigned cs, unsigned o, int e) {
+    const double2 d = static_cast<const double2 *>(p)[(unsigned)e * cs + o];
+    return cmk<double>(d.x, d.y);
+}
+__device__ __forceinline__ void store_comp(void *p, unsigned cs, unsigned o, int e, Cx<double> z) {
+    static_cast<double2 *>(p)[(unsigned)e * cs + o] = make_double2(z.re, z.im);
 }
 
-// one complex component e of the spinor at (site, RHS) offset o = site stride * site + RHS
-// stride * RHS (in chunks), chunk stride cs; COH: read from L2 (data that other SMs write
-// during the launch)
-template <typename S>
-struct Comp;
-template <>
-struct Comp<double> {
-    using C = double;
-    template <bool COH = false>
-    __device__ static __forceinline__ Cx<double> load(const void *p, const float *, unsigned cs, unsigned o, int e) {
-        const double2 *q = static_cast<const double2 *>(p) + ((unsigned)e * cs + o);
-        const double2 d = COH ? __ldcg(q) : *q;
-        return cmk<double>(d.x, d.y);
-    }
-    __device__ static __forceinline__ void store(void *p, unsigned cs, unsigned o, int e, Cx<double> z) {
-        static_cast<double2 *>(p)[(unsigned)e * cs + o] = make_double2(z.re, z.im);
-    }
-};
-template <>
-struct Comp<float> {
-    using C = float;
-    template <bool COH = false>
-    __device__ static __forceinline__ Cx<float> load(const void *p, const float *, unsigned cs, unsigned o, int e) {
-        const float2 *q = static_cast<const float2 *>(p) + (((unsigned)(e >> 1) * cs + o) * 2 + (e & 1));
-        const float2 d = COH ? __ldcg(q) : *q;
-        return cmk<float>(d.x, d.y);
-    }
-    __device__ static __forceinline__ void store(void *p, unsigned cs, unsigned o, int e, Cx<float> z) {
-        static_cast<float2 *>(p)[((unsigned)(e >> 1) * cs + o) * 2 + (e & 1)] = make_float2(z.re, z.im);
-    }
-};
 // the rows of the link this lane multiplies by: u[a][b] = U[a][b] (bwd = false) or
 // conj(U[b][a]) (bwd = true)
-template <int GF, typename C>
-__device__ __forceinline__ void load_link_for(const void *g, unsigned Vg, int mu, unsigned s, bool bwd, Cx<C> (&u)[3][3]) {
+__device__ __forceinline__ void load_link_for(const void *g, unsigned Vg, int mu, unsigned s, bool bwd,
+                                              Cx<double> (&u)[3][3]) {
     GaugeView gv;
     gv.data = g;
     gv.V = Vg;
-    Link<C> U;
-    GaugeLoad<GF>::load(gv, mu, s, U);
+    Link<double> U;
+    GaugeLoad<GF_F64_18>::load(gv, mu, s, U);
 #pragma unroll
     for (int a = 0; a < 3; a++)
 #pragma unroll
@@ -157,16 +79,15 @@ __device__ __forceinline__ void load_link_for(const void *g, unsigned Vg, int mu
 
 // What lane l = 2 hop + spin of a 16-lane group does in every site: the projection
 // h = a_spin + ph (lower partner), partner spin part, factor +-1 or +-i
-template <typename C>
 struct LaneRole {
     int l, mu, sp, part;
     bool bwd, img;
-    C sre, sim;
+    double sre, sim;
 };
-template <bool DAG, typename C>
-__device__ __forceinline__ LaneRole<C> lane_role(int l) {
+template <bool DAG>
+__device__ __forceinline__ LaneRole lane_role(int l) {
     constexpr int SF = DAG ? +1 : -1;  // forward projector I + SF g_mu, backward I - SF g_mu
-    LaneRole<C> q;
+    LaneRole q;
     q.l = l;
     q.mu = l >> 2;
     q.sp = l & 1;
@@ -174,19 +95,17 @@ __device__ __forceinline__ LaneRole<C> lane_role(int l) {
     q.part = q.mu <= 1 ? 1 - q.sp : q.sp;
     q.img = q.mu == 0 || q.mu == 2;
     const bool neg = ((q.mu == 1 && q.sp == 0) || (q.mu == 2 && q.sp == 1)) != ((q.bwd ? -SF : SF) < 0);
-    q.sre = (neg != q.img) ? (C)-1 : (C)1;
-    q.sim = neg ? (C)-1 : (C)1;
+    q.sre = (neg != q.img) ? -1.0 : 1.0;
+    q.sim = neg ? -1.0 : 1.0;
     return q;
 }
 
 // Component l (lanes 0..11) of diag * centre + hcoef * (hop sum) at output site s, RHS r, from
-// the field in / in_s of a (cen: its centre term).  Collective over the warp; live is uniform
+// the field a.in (a.cen: its centre term).  Collective over the warp; live is uniform
 // over a 16-lane group.  prod: the group's [8][2][3] products.
-template <typename S, int GF, bool DAG, bool COH>
-__device__ __forceinline__ Cx<typename Comp<S>::C> split_component(const SplitArgs &a, const LaneRole<typename Comp<S>::C> &q,
-                                                                   const void *in, const void *cen, bool live, unsigned s,
-                                                                   unsigned r, Cx<typename Comp<S>::C> (*prod)[2][3]) {
-    using C = typename Comp<S>::C;
+template <bool DAG>
+__device__ __forceinline__ Cx<double> split_component(const SplitArgs &a, const LaneRole &q, bool live, unsigned s, unsigned r,
+                                                      Cx<double> (*prod)[2][3]) {
     constexpr int SF = DAG ? +1 : -1;
     const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2;
     unsigned x, y, z, tt, sl;
@@ -212,15 +131,15 @@ __device__ __forceinline__ Cx<typename Comp<S>::C> split_component(const SplitAr
     const unsigned nl = q.bwd ? (cm == 0 ? sl + (Lm - 1) * sm : sl - sm) : (cm == Lm - 1 ? sl - (Lm - 1) * sm : sl + sm);
     const unsigned nf = a.eo >= 0 ? nl >> 1 : nl;  // field index of the neighbour
     const unsigned oin = nf * a.in_x + r * a.in_r, oc = s * a.in_x + r * a.in_r;
-    Cx<C> c0 = cmk<C>(0, 0);
+    Cx<double> c0 = cmk<double>(0, 0);
     if (live) {
-        Cx<C> h[3], u[3][3], v[3];
+        Cx<double> h[3], u[3][3], v[3];
 #pragma unroll
-        for (int c = 0; c < 3; c++) h[c] = Comp<S>::template load<COH>(in, nullptr, a.in_c, oin, q.sp * 3 + c);
+        for (int c = 0; c < 3; c++) h[c] = load_comp(a.in, a.in_c, oin, q.sp * 3 + c);
 #pragma unroll
-        for (int c = 0; c < 3; c++) v[c] = Comp<S>::template load<COH>(in, nullptr, a.in_c, oin, 6 + q.part * 3 + c);
-        load_link_for<GF>(a.g, a.Vg, mu, q.bwd ? nl : sl, q.bwd, u);
-        if (l < 12 && cen) c0 = Comp<S>::template load<COH>(cen, nullptr, a.in_c, oc, l);  // in flight with the hops
+        for (int c = 0; c < 3; c++) v[c] = load_comp(a.in, a.in_c, oin, 6 + q.part * 3 + c);
+        load_link_for(a.g, a.Vg, mu, q.bwd ? nl : sl, q.bwd, u);
+        if (l < 12 && a.cen) c0 = load_comp(a.cen, a.in_c, oc, l);  // in flight with the hops
 #pragma unroll
         for (int c = 0; c < 3; c++) {
             h[c].re = fma(q.sre, q.img ? v[c].im : v[c].re, h[c].re);
@@ -228,51 +147,49 @@ __device__ __forceinline__ Cx<typename Comp<S>::C> split_component(const SplitAr
         }
 #pragma unroll
         for (int i = 0; i < 3; i++) {
-            Cx<C> w = cmul(u[i][0], h[0]);
+            Cx<double> w = cmul(u[i][0], h[0]);
             w = cfma(u[i][1], h[1], w);
             w = cfma(u[i][2], h[2], w);
             prod[l >> 1][q.sp][i] = w;
         }
     }
     __syncwarp();
-    Cx<C> o = cmk<C>(0, 0);
+    Cx<double> o = cmk<double>(0, 0);
     if (l < 12 && live) {
         const int so = l / 3, c = l - 3 * so, lo = so & 1;
-        Cx<C> acc = cmk<C>(0, 0);
+        Cx<double> acc = cmk<double>(0, 0);
 #pragma unroll
         for (int hh = 0; hh < 8; hh++) {
             const int m = hh >> 1, sg = (hh & 1) ? -SF : SF;
             // upper spins take the product, lower spins sg B_mu^H of it
             const int from = so < 2 ? lo : (m <= 1 ? 1 - lo : lo);
-            const Cx<C> w = prod[hh][from][c];
+            const Cx<double> w = prod[hh][from][c];
             const bool im = so >= 2 && (m == 0 || m == 2);
             bool ng = false;
             if (so >= 2) ng = ((m == 0) || (m == 1 && lo == 1) || (m == 2 && lo == 0)) != (sg < 0);
             // factor (-1)^ng, times i where im
-            const C fr = (ng != im) ? (C)-1 : (C)1, fi = ng ? (C)-1 : (C)1;
+            const double fr = (ng != im) ? -1.0 : 1.0, fi = ng ? -1.0 : 1.0;
             acc.re = fma(fr, im ? w.im : w.re, acc.re);
             acc.im = fma(fi, im ? w.re : w.im, acc.im);
         }
-        const C d = (C)a.diag, hc = (C)a.hcoef;
-        o = cmk<C>(d * c0.re + hc * acc.re, d * c0.im + hc * acc.im);
+        const double d = a.diag, hc = a.hcoef;
+        o = cmk<double>(d * c0.re + hc * acc.re, d * c0.im + hc * acc.im);
     }
     __syncwarp();
     return o;
 }
 
 // |component|^2 summed over a 16-lane group (the same in its lanes)
-template <typename C>
-__device__ __forceinline__ double group_norm2(bool mine, Cx<C> o) {
-    C n = mine ? o.re * o.re + o.im * o.im : (C)0;
+__device__ __forceinline__ double group_norm2(bool mine, Cx<double> o) {
+    double n = mine ? o.re * o.re + o.im * o.im : 0.0;
 #pragma unroll
     for (int off = 8; off > 0; off >>= 1) n += __shfl_xor_sync(0xffffffffu, n, off);
-    return (double)n;
+    return n;
 }
 
-template <typename S, int GF, bool DAG, int EPI>
+template <bool DAG, int EPI>
 __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
-    using C = typename Comp<S>::C;
-    __shared__ Cx<C> prod[8][8][2][3];  // [group][hop][spin][colour]
+    __shared__ Cx<double> prod[8][8][2][3];  // [group][hop][spin][colour]
     __shared__ double smem[(128 / 32) * MAX_RHS];
     __shared__ double gsum[8];
     if (EPI == SPL_NORM || EPI == SPL_CG) {
@@ -281,7 +198,7 @@ __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
         if (!any) return;
     }
     const int t = threadIdx.x, grp = t >> 4, l = t & 15;
-    const LaneRole<C> role = lane_role<DAG, C>(l);
+    const LaneRole role = lane_role<DAG>(l);
     const unsigned total = a.V << a.kshift, step = gridDim.x * (blockDim.x >> 4);
     double nrm = 0.0;
     const unsigned niter = (total + step - 1) / step;
@@ -291,19 +208,19 @@ __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
         const unsigned s = live ? g >> a.kshift : 0u, r = g & (a.k - 1);
         const unsigned oo = s * a.out_x + r * a.out_r;
         const bool mine = live && l < 12;
-        Cx<C> e0 = cmk<C>(0, 0);
-        if (EPI == SPL_CG && mine) e0 = Comp<S>::load(a.r, nullptr, a.out_c, oo, l);
-        if (EPI == SPL_RESID && mine) e0 = Comp<S>::load(a.b, nullptr, a.out_c, oo, l);
-        Cx<C> o = split_component<S, GF, DAG, false>(a, role, a.in, a.cen, live, s, r, prod[grp]);
+        Cx<double> e0 = cmk<double>(0, 0);
+        if (EPI == SPL_CG && mine) e0 = load_comp(a.r, a.out_c, oo, l);
+        if (EPI == SPL_RESID && mine) e0 = load_comp(a.b, a.out_c, oo, l);
+        Cx<double> o = split_component<DAG>(a, role, live, s, r, prod[grp]);
         if (EPI == SPL_RESID) o = e0 - o;
         if (EPI == SPL_CG) {
             const CGScalars &st = a.st[r];
-            const C al = st.active ? (C)st.alpha : (C)0;
-            if (mine && a.save_t) Comp<S>::store(a.tsave, a.V, s, l, o);  // single RHS
-            o = cmk<C>(e0.re - al * o.re, e0.im - al * o.im);
+            const double al = st.active ? st.alpha : 0.0;
+            if (mine && a.save_t) store_comp(a.tsave, a.V, s, l, o);  // single RHS
+            o = cmk<double>(e0.re - al * o.re, e0.im - al * o.im);
         }
-        if (mine) Comp<S>::store(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
-        if (EPI != SPL_PLAIN) nrm += group_norm2<C>(mine, o);  // a group's RHS is the same in every pass
+        if (mine) store_comp(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
+        if (EPI != SPL_PLAIN) nrm += group_norm2(mine, o);  // a group's RHS is the same in every pass
     }
     if (EPI == SPL_PLAIN) return;
     const int ngrp = blockDim.x >> 4, k = (int)a.k;
@@ -326,9 +243,7 @@ __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
 inline void split_args(SplitArgs &a, const DslashCall &c) {
     memset(&a, 0, sizeof(a));
     a.in = c.in.v.data;
-    a.in_s = c.in.v.scale;
     a.out = c.out.v.data;
-    a.out_s = c.out.v.scale;
     a.g = c.gauge.data;
     a.L0 = c.L[0];
     a.L1 = c.L[1];
@@ -358,11 +273,7 @@ inline void split_args(SplitArgs &a, const DslashCall &c) {
         a.out_r = 12 * a.V;
     }
     a.cen = c.in.v.data;
-    a.cen_s = c.in.v.scale;
-    if (c.eo_parity >= 0) {
-        a.cen = c.cen.v.data;
-        a.cen_s = c.cen.v.scale;
-    }
+    if (c.eo_parity >= 0) a.cen = c.cen.v.data;
     a.diag = c.diag;
     a.hcoef = c.hcoef;
 }
@@ -379,9 +290,9 @@ inline void split_reduction(SplitArgs &a, CGScalars *st, const History &h, int i
 }
 
 // Blocks of one warp while there are fewer warps than SMs (each then has an SM's FP64 units
-// or L1 to itself), of four otherwise; 16 resident warps per SM at most, and a multiple of 16
+// to itself), of four otherwise; 16 resident warps per SM at most, and a multiple of 16
 // blocks when a block makes several passes, so that a group keeps its RHS from pass to pass.
-template <typename S, int GF, int EPI>
+template <int EPI>
 cudaError_t split_launch(bool dag, const SplitArgs &a, int cap, cudaStream_t s) {
     const long groups = (long)a.V << a.kshift, warps = (groups + 1) / 2;
     if (groups > SPLIT_MAX || a.k > (unsigned)MAX_RHS) return cudaErrorInvalidValue;
@@ -393,8 +304,8 @@ cudaError_t split_launch(bool dag, const SplitArgs &a, int cap, cudaStream_t s) 
     long grid = need;
     if (grid > most) grid = most / 16 * 16;
     if (grid < 1) grid = need < 16 ? need : 16;
-    if (dag) k_dslash_split<S, GF, true, EPI><<<(int)grid, tpb, 0, s>>>(a);
-    else k_dslash_split<S, GF, false, EPI><<<(int)grid, tpb, 0, s>>>(a);
+    if (dag) k_dslash_split<true, EPI><<<(int)grid, tpb, 0, s>>>(a);
+    else k_dslash_split<false, EPI><<<(int)grid, tpb, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -48,12 +48,6 @@ FX_HD int clz64(uint64_t u) {
 #endif
 }
 
-// biased exponent (1 for zeros and denormals, SPECIAL for Inf and NaN)
-FX_HD int exponent(double x) {
-    const int e = (int)((bits(x) >> 52) & 0x7ff);
-    return e > 1 ? e : 1;
-}
-
 // x 2^(1079 - emax) rounded to the nearest integer (ties away from zero)
 FX_HD long long to_fixed(double x, int emax) {
     const uint64_t u = bits(x);
