@@ -113,7 +113,9 @@ eig_status eig_op_trim(eig_op op, size_t *freed);
 
 /* out = M in (which 0), M^H in (which 1) or A in (which 2) for k RHS (1..max_rhs),
  * in the op's storage precision; which 3 (FP32/FP16 ops only) applies A in the
- * FP64-accurate arithmetic of the residuals.
+ * arithmetic of the residuals, which is that of FP64 ops.  FP64 products hold every component
+ * to FP64 rounding of its own terms (the |u_ab| |psi_b| of its eight hops), whichever kernel
+ * a size takes; their last bits depend on the size.
  * in/out: natural layout, may alias.
  * This is the dslash of the CG matrix-vector product (Fig. 1 step 11). */
 eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int k, void *stream);

@@ -416,7 +416,7 @@ static cudaError_t dispatch(const DslashCall &c, KArgs &a, int cap, cudaStream_t
     const long work = a.V * c.k;
     const int block = 128;
     ProfScope prof(dslash_name(EPI, c.in.prec, c.k).c_str(), dslash_bytes<EPI>(c, a), s);
-    if (c.in.prec == P64 && c.gformat == GF_F64_18 && c.fx.links && !c.nat_in && !c.nat_out && work >= FX_MIN) {
+    if (c.in.prec == P64 && c.gformat == GF_F64_18 && c.fx.links && !c.nat_in && !c.nat_out && work >= FX_MIN && work <= FX_MAX) {
         Field fb{}, fr{}, ft{};
         fb.v = a.b;
         fr.v = a.r;

@@ -12,22 +12,25 @@
 //                projects them by integer adds, multiplies by the links (two 29-bit limbs per
 //                real, three wide multiply-adds per real product), sums the eight hops exactly
 //                and rounds once to FP64, where the centre term and the epilogue are formed.
-// The only errors are the alignment and limb truncations, at most 2^-55 of the largest neighbour
-// component per hop, and the final rounding; against the exact product the measured error is no
-// larger than that of the FP64 chain (16^3x32, Gaussian vectors: 1.3e-16 against 1.4e-16).  A
-// site with an Inf or NaN among its neighbours takes an FP64 path of its own, so non-finite
-// values propagate as there.  Links must be unitary to 1% (checked when an operator is created;
-// the sums of eight hops then stay below 2^63); other operators keep the FP64 stencil, and so
-// do launches too small to fill the GPU (FX_MIN).
+// The errors are at most 2^-50 of the largest neighbour component, so an element whose hop
+// products are all small against that one is not kept (fxmath.h has the bound and the guard): the
+// warp forms it again in FP64, 16 lanes to an element (dslash_split.cuh).  The same path takes
+// elements with an Inf or NaN among their neighbours, and those near the ends of the exponent
+// range.  Links must be unitary to 1% (checked when an operator is created; the sums of eight hops
+// then stay below 2^63); other operators keep the FP64 stencil, and so do launches too small to
+// fill the GPU (FX_MIN).
 //
 // What bounds it now: the wide multiply-adds (1728 per site, 2 cycles each on the heavy half of
 // the FMA pipe, 46% busy), integer ALU (39%) and the latency of the neighbour loads at 16 warps
 // per SM.  Measured per product, conversion included (the conversion alone 28 us, 5.4 TB/s):
-//   16^3x32, k = 4    FP64 850 us    fixed point 282 us
+//   16^3x32, k = 4    FP64 850 us    fixed point 282 us (every element left to FP64: 1135 us)
 //   12^3x24, k = 8    double-float (44 bits; used for residual replacements before) 194 us plus
-//                     120 us of field conversions per A; fixed point 184 us
-// Four blocks per SM (128 registers, ~160 bytes spilled) beat three (294 us) and two (377 us);
-// without the L1 prefetch of the next hop three took 311 us; with the eight hops unrolled, 685.
+//                     120 us of field conversions per A; fixed point 186 us
+// The guard keeps one bit per product; with sums of magnitudes in six registers the same product
+// took 303 us.
+// Four blocks per SM (128 registers, ~170 to 230 bytes spilled) beat three (294 us) and two (377
+// us); without the L1 prefetch of the next hop three took 311 us; with the eight hops unrolled,
+// 685.
 #include <cstring>
 
 #include "dslash_split.cuh"
@@ -49,26 +52,9 @@ __host__ __device__ constexpr size_t tiled(unsigned i, int comps) {
 
 struct FxArgs {
     const longlong2 *fx;  // hop input in fixed point (re, im), tiled, 12 components
-    const int *ex;        // its exponents: [V][k]
-    const double2 *in;    // the same field in FP64 (sites with non-finite neighbours)
-    const double2 *cen;   // centre-term input (null: hops only)
+    const int *ex;        // its exponent words: [V][k]
     const int4 *g;        // links, limbs (re hi, re lo, im hi, im lo): [mu] tiled, 9 components
-    const double2 *g64;
-    double2 *out;
-    const double2 *b;
-    double2 *r;
-    double2 *tsave;
-    unsigned L0, L1, L2, L3, V, Vg, lh, k, kshift;
-    FastDiv d0, d1, d2, dh;
-    int eo;
-    double diag, hcoef;
-    int save_t, set_rho;
-    CGScalars *st;
-    double *h_alpha, *h_beta, *h_rho;
-    int iter;
-    const int *jbase;
-    double *partials;
-    unsigned *counter;
+    SplitArgs s;          // the call in FP64
 };
 
 constexpr int FX_TPB = 128;
@@ -86,7 +72,17 @@ __global__ void __launch_bounds__(FX_TPB) k_to_fx(const double2 *__restrict__ in
             top = max(top, (unsigned)__double2hiint(v[c].y) & 0x7fffffffu);
         }
         const int e = max((int)(top >> 20), 1);
-        ex[o] = e;
+        unsigned spins = 0;
+#pragma unroll
+        for (int sp = 0; sp < 4; sp++) {
+            unsigned any = 0;
+#pragma unroll
+            for (int c = 3 * sp; c < 3 * sp + 3; c++)
+                any |= (unsigned)(__double2loint(v[c].x) | __double2loint(v[c].y)) |
+                       (((unsigned)__double2hiint(v[c].x) | (unsigned)__double2hiint(v[c].y)) & 0x7fffffffu);
+            spins |= any ? 1u << sp : 0u;
+        }
+        ex[o] = e | (int)(spins << fx::NZ);
         if (e >= fx::SPECIAL) continue;  // never read
 #pragma unroll
         for (int c = 0; c < 12; c++) {
@@ -154,7 +150,7 @@ __device__ __forceinline__ void prefetch_hop_fx(const FxArgs &a, int mu, unsigne
 #pragma unroll
     for (int e = 0; e < 12; e++) asm volatile("prefetch.global.L1 [%0];" ::"l"(f + e * TILE));
     if (mu > 3) return;
-    const int4 *g = a.g + mu * fx_link_plane(a.Vg) + tiled(ls, 9);
+    const int4 *g = a.g + mu * fx_link_plane(a.s.Vg) + tiled(ls, 9);
 #pragma unroll
     for (int e = 0; e < 9; e++) asm volatile("prefetch.global.L1 [%0];" ::"l"(g + e * TILE));
 }
@@ -163,16 +159,17 @@ __device__ __forceinline__ void prefetch_hop_fx(const FxArgs &a, int mu, unsigne
 // conj(U)^T if bwd, projector I + sg g_mu.  mu, bwd and sg are uniform over the launch's
 // threads and not template arguments: only the projection and the rebuilding differ between the
 // eight hops, and with all of them unrolled the ~11 000 instructions of a site did not fit the
-// instruction caches (stalled on instruction fetch 3.8 of 7 cycles per issue).
+// instruction caches (stalled on instruction fetch 3.8 of 7 cycles per issue).  large: bit e
+// is set if product e passes guard_large.
 __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool plus, unsigned o, unsigned ls, int sh,
-                                       I2 (&acc)[12]) {
+                                       I2 (&acc)[12], unsigned &large) {
     const longlong2 *f = a.fx + tiled(o, 12);
     I2 v[12];
 #pragma unroll
     for (int e = 0; e < 12; e++) {
         const longlong2 d = __ldg(f + e * TILE);
-        v[e].re = d.x >> sh;
-        v[e].im = d.y >> sh;
+        v[e].re = fx::align(d.x, sh);
+        v[e].im = fx::align(d.y, sh);
     }
     // project: h = a + sg B_mu b (see dslash.cu for B_mu)
     I2 h[6];
@@ -203,7 +200,7 @@ __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool p
         fx::limbs(h[e].re, rh[e], rl[e]);
         fx::limbs(h[e].im, ih[e], il[e]);
     }
-    const int4 *g = a.g + mu * fx_link_plane(a.Vg) + tiled(ls, 9);
+    const int4 *g = a.g + mu * fx_link_plane(a.s.Vg) + tiled(ls, 9);
     const int sq = bwd ? TILE : 3 * TILE, sb = bwd ? 3 * TILE : TILE;
     I2 w[6];
 #pragma unroll
@@ -231,6 +228,7 @@ __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool p
             }
             w[s * 3 + q].re = fx::value(re.hh, re.mid);
             w[s * 3 + q].im = fx::value(im.hh, im.mid);
+            if (fx::guard_large(w[s * 3 + q].re, w[s * 3 + q].im)) large |= 1u << (s * 3 + q);
         }
     }
     // rebuild (w, sg B_mu^H w)
@@ -258,52 +256,35 @@ __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool p
 #undef FX_REBUILD
 }
 
-// The hop sum of one (site, RHS) in FP64 (sites with an Inf or NaN around them; loops kept
-// rolled: rarely taken)
-__device__ __noinline__ void hops_fp64(const FxArgs &a, size_t P, const unsigned *nbr, const unsigned *lks, int sf,
-                                       double2 *acc) {
-    for (int e = 0; e < 12; e++) acc[e] = make_double2(0.0, 0.0);
-#pragma unroll 1
-    for (int hop = 0; hop < 8; hop++) {
-        const int mu = hop >> 1, sg = (hop & 1) ? -sf : sf;
-        const double2 *g = a.g64 + (size_t)mu * 9 * a.Vg + lks[hop];
-        double2 h[2][3], w[2][3];
-        for (int s = 0; s < 2; s++)
-            for (int c = 0; c < 3; c++) {
-                const int part = mu <= 1 ? 1 - s : s;
-                const double2 u = a.in[(size_t)(s * 3 + c) * P + nbr[hop]];
-                const double2 v = a.in[(size_t)(6 + part * 3 + c) * P + nbr[hop]];
-                const bool neg = ((mu == 1 && s == 0) || (mu == 2 && s == 1)) != (sg < 0);
-                double2 q = (mu == 0 || mu == 2) ? make_double2(-v.y, v.x) : v;
-                h[s][c] = neg ? make_double2(u.x - q.x, u.y - q.y) : make_double2(u.x + q.x, u.y + q.y);
-            }
-        for (int s = 0; s < 2; s++)
-            for (int i = 0; i < 3; i++) {
-                double2 z = make_double2(0.0, 0.0);
-                for (int b = 0; b < 3; b++) {
-                    double2 u = g[(size_t)((hop & 1) ? b * 3 + i : i * 3 + b) * a.Vg];
-                    if (hop & 1) u.y = -u.y;
-                    z.x += u.x * h[s][b].x - u.y * h[s][b].y;
-                    z.y += u.x * h[s][b].y + u.y * h[s][b].x;
-                }
-                w[s][i] = z;
-            }
-        for (int s = 0; s < 2; s++)
-            for (int c = 0; c < 3; c++) {
-                acc[s * 3 + c].x += w[s][c].x;
-                acc[s * 3 + c].y += w[s][c].y;
-                const double2 v = w[mu <= 1 ? 1 - s : s][c];
-                const bool neg = ((mu == 0) || (mu == 1 && s == 1) || (mu == 2 && s == 0)) != (sg < 0);
-                const double2 q = (mu == 0 || mu == 2) ? make_double2(-v.y, v.x) : v;
-                acc[6 + s * 3 + c].x += neg ? -q.x : q.x;
-                acc[6 + s * 3 + c].y += neg ? -q.y : q.y;
-            }
+// The elements g0 + i, i in todo, in FP64 and through the epilogue: two at a time, 16 lanes each.
+// Returns what this lane's RHS gains in |result|^2.  prod: the warp's scratch.
+template <bool DAG, int EPI>
+__device__ __noinline__ double elements_fp64(const SplitArgs &a, unsigned todo, unsigned g0, Cx<double> (*prod)[8][2][3]) {
+    const int lane = threadIdx.x & 31, grp = lane >> 4;
+    const LaneRole role = lane_role<DAG>(lane & 15);
+    double sum = 0.0;
+    while (todo) {
+        const int i0 = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int i1 = __ffs(todo) - 1;  // -1: none
+        todo &= todo - 1;
+        const int i = grp ? i1 : i0;
+        const unsigned g = g0 + (i < 0 ? 0 : i);
+        const double n = split_site<DAG, EPI>(a, role, i >= 0, g >> a.kshift, g & (a.k - 1), prod[grp]);
+        if (EPI != SPL_PLAIN) {
+            const double n0 = __shfl_sync(0xffffffffu, n, 0), n1 = __shfl_sync(0xffffffffu, n, 16);
+            if (lane == i0) sum += n0;
+            if (lane == i1) sum += n1;
+        }
     }
+    return sum;
 }
 
 template <bool DAG, int EPI>
-__global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const FxArgs a) {
+__global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const __grid_constant__ FxArgs args) {
     __shared__ double smem[(FX_TPB / 32) * MAX_RHS];
+    __shared__ Cx<double> prod[FX_TPB / 32][2][8][2][3];
+    const SplitArgs &a = args.s;
     if (EPI == SPL_NORM || EPI == SPL_CG) {
         bool any = false;
         for (unsigned q = 0; q < a.k; q++) any = any || a.st[q].active;
@@ -311,102 +292,110 @@ __global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const FxArgs a) {
     }
     const unsigned total = a.V << a.kshift;
     const size_t P = total;
-    const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2;
+    const unsigned s1 = a.L0, s2 = a.L0 * a.L1, s3 = s2 * a.L2, lane = threadIdx.x & 31;
     double nrm = 0.0;
-    for (unsigned g = blockIdx.x * FX_TPB + threadIdx.x; g < total; g += gridDim.x * FX_TPB) {
-        const unsigned s = g >> a.kshift, r = g & (a.k - 1);
-        unsigned x, y, z, t, sl;
-        if (a.eo >= 0) {
-            const unsigned rest = a.lh > 1 ? fastdiv(s, a.dh) : s, q2 = fastdiv(rest, a.d1);
-            t = fastdiv(q2, a.d2);
-            y = rest - q2 * a.L1;
-            z = q2 - t * a.L2;
-            x = 2 * (s - rest * a.lh) + ((a.eo + y + z + t) & 1);
-            sl = x + rest * a.L0;
-        } else {
-            const unsigned q1 = fastdiv(s, a.d0), q2 = fastdiv(q1, a.d1);
-            t = fastdiv(q2, a.d2);
-            x = s - q1 * a.L0;
-            y = q1 - q2 * a.L1;
-            z = q2 - t * a.L2;
-            sl = s;
-        }
-        // neighbour of hop h = 2 mu + (backward) as a lattice site
-        auto neighbour = [&](int h) {
-            const int mu = h >> 1;
-            const unsigned c = mu == 0 ? x : (mu == 1 ? y : (mu == 2 ? z : t));
-            const unsigned L = mu == 0 ? a.L0 : (mu == 1 ? a.L1 : (mu == 2 ? a.L2 : a.L3));
-            const unsigned st = mu == 0 ? 1u : (mu == 1 ? s1 : (mu == 2 ? s2 : s3));
-            return (h & 1) ? (c == 0 ? sl + (L - 1) * st : sl - st) : (c == L - 1 ? sl - (L - 1) * st : sl + st);
-        };
-        auto field_index = [&](unsigned nl) { return ((a.eo >= 0 ? nl >> 1 : nl) << a.kshift) + r; };
-        int e[8], em = 1;
-#pragma unroll
-        for (int h = 0; h < 8; h++) {
-            e[h] = __ldg(a.ex + field_index(neighbour(h)));
-            em = max(em, e[h]);
-        }
-        unsigned long long shifts = 0;  // alignment of each hop, 8 bits each
-#pragma unroll
-        for (int h = 0; h < 8; h++) shifts |= (unsigned long long)min(em - e[h], 63) << (8 * h);
-        double2 hs[12];  // hop sum
-        if (em < fx::SPECIAL) {
-            I2 acc[12];
-#pragma unroll
-            for (int q = 0; q < 12; q++) acc[q].re = acc[q].im = 0;
-            unsigned nl = neighbour(0);
-#pragma unroll 1
-            for (int h = 0; h < 8; h++) {
-                const bool bwd = h & 1;
-                // ask L1 for the next hop's data while this one is computed
-                const unsigned nx = h < 7 ? neighbour(h + 1) : nl;
-                prefetch_hop_fx(a, (h + 1) >> 1, field_index(nx), bwd ? sl : nx);
-                hop_fx(a, h >> 1, bwd, DAG != bwd, field_index(nl), bwd ? nl : sl, (int)(shifts & 63), acc);
-                shifts >>= 8;
-                nl = nx;
-            }
-#pragma unroll
-            for (int q = 0; q < 12; q++) hs[q] = make_double2(fx::to_double(acc[q].re, em), fx::to_double(acc[q].im, em));
-        } else {
-            unsigned nbr[8], lks[8];
-#pragma unroll 1
-            for (int h = 0; h < 8; h++) {
-                const unsigned nl = neighbour(h);
-                nbr[h] = field_index(nl);
-                lks[h] = (h & 1) ? nl : sl;
-            }
-            hops_fp64(a, P, nbr, lks, DAG ? +1 : -1, hs);
-        }
-        // diag * centre + hcoef * hops, then the epilogue, component by component
-        const double d = a.diag, hc = a.hcoef;
-        double al = 0.0;
-        if (EPI == SPL_CG) {
-            const CGScalars &st = a.st[r];
-            al = st.active ? st.alpha : 0.0;
-        }
-        double n2 = 0.0;
-#pragma unroll
-        for (int q = 0; q < 12; q++) {
-            const size_t o = (size_t)q * P + g;
-            const double2 c0 = a.cen ? a.cen[o] : make_double2(0.0, 0.0);
-            double2 w = make_double2(d * c0.x + hc * hs[q].x, d * c0.y + hc * hs[q].y);
-            if (EPI == SPL_PLAIN || EPI == SPL_NORM) {
-                a.out[o] = w;
-            } else if (EPI == SPL_CG) {
-                if (a.save_t) a.tsave[(size_t)q * a.V + s] = w;
-                double2 rr = a.r[o];
-                rr.x -= al * w.x;
-                rr.y -= al * w.y;
-                a.r[o] = rr;
-                w = rr;
+    // a warp's lanes make the same number of passes (elements_fp64 takes them all)
+    for (unsigned g0 = blockIdx.x * FX_TPB + (threadIdx.x & ~31u); g0 < total; g0 += gridDim.x * FX_TPB) {
+        const unsigned g = g0 + lane;
+        bool fp64 = false;  // left to elements_fp64
+        if (g < total) {
+            const unsigned s = g >> a.kshift, r = g & (a.k - 1);
+            unsigned x, y, z, t, sl;
+            if (a.eo >= 0) {
+                const unsigned rest = a.lh > 1 ? fastdiv(s, a.dh) : s, q2 = fastdiv(rest, a.d1);
+                t = fastdiv(q2, a.d2);
+                y = rest - q2 * a.L1;
+                z = q2 - t * a.L2;
+                x = 2 * (s - rest * a.lh) + ((a.eo + y + z + t) & 1);
+                sl = x + rest * a.L0;
             } else {
-                const double2 bb = a.b[o];
-                w = make_double2(bb.x - w.x, bb.y - w.y);
-                a.r[o] = w;
+                const unsigned q1 = fastdiv(s, a.d0), q2 = fastdiv(q1, a.d1);
+                t = fastdiv(q2, a.d2);
+                x = s - q1 * a.L0;
+                y = q1 - q2 * a.L1;
+                z = q2 - t * a.L2;
+                sl = s;
             }
-            if (EPI != SPL_PLAIN) n2 += w.x * w.x + w.y * w.y;
+            // neighbour of hop h = 2 mu + (backward) as a lattice site
+            auto neighbour = [&](int h) {
+                const int mu = h >> 1;
+                const unsigned c = mu == 0 ? x : (mu == 1 ? y : (mu == 2 ? z : t));
+                const unsigned L = mu == 0 ? a.L0 : (mu == 1 ? a.L1 : (mu == 2 ? a.L2 : a.L3));
+                const unsigned st = mu == 0 ? 1u : (mu == 1 ? s1 : (mu == 2 ? s2 : s3));
+                return (h & 1) ? (c == 0 ? sl + (L - 1) * st : sl - st) : (c == L - 1 ? sl - (L - 1) * st : sl + st);
+            };
+            auto field_index = [&](unsigned nl) { return ((a.eo >= 0 ? nl >> 1 : nl) << a.kshift) + r; };
+            int e[8], em = 1;
+            unsigned sp0 = 0, sp1 = 0;  // nonzero spins of the neighbours in x and y, in z and t
+#pragma unroll
+            for (int h = 0; h < 8; h++) {
+                const int w = __ldg(args.ex + field_index(neighbour(h)));
+                e[h] = w & 0x7ff;
+                em = max(em, e[h]);
+                (h < 4 ? sp0 : sp1) |= (unsigned)w >> fx::NZ;
+            }
+            unsigned long long shifts = 0;  // alignment of each hop, 8 bits each
+#pragma unroll
+            for (int h = 0; h < 8; h++) shifts |= (unsigned long long)min(em - e[h], 63) << (8 * h);
+            unsigned formed = fx::guard_formed(sp0, true) | (fx::guard_formed(sp1, false) << 8), large = 0;
+            fp64 = fx::exponent_bad(em, sp0 | sp1);
+            if (!fp64) {
+                I2 acc[12];
+#pragma unroll
+                for (int q = 0; q < 12; q++) acc[q].re = acc[q].im = 0;
+                unsigned nl = neighbour(0);
+#pragma unroll 1
+                for (int h = 0; h < 8; h++) {
+                    const bool bwd = h & 1;
+                    // ask L1 for the next hop's data while this one is computed
+                    const unsigned nx = h < 7 ? neighbour(h + 1) : nl;
+                    prefetch_hop_fx(args, (h + 1) >> 1, field_index(nx), bwd ? sl : nx);
+                    hop_fx(args, h >> 1, bwd, DAG != bwd, field_index(nl), bwd ? nl : sl, (int)(shifts & 63), acc, large);
+                    shifts >>= 8;
+                    nl = nx;
+                    if (h == 3) large <<= 8;  // the x and y hops are done
+                }
+                fp64 = fx::guard_bad(formed & 63, large >> 8, formed >> 8, large & 63);
+                if (!fp64) {
+                    // diag * centre + hcoef * hops, then the epilogue, component by component
+                    const double d = a.diag, hc = a.hcoef;
+                    double al = 0.0;
+                    if (EPI == SPL_CG) {
+                        const CGScalars &st = a.st[r];
+                        al = st.active ? st.alpha : 0.0;
+                    }
+                    const double2 *cen = static_cast<const double2 *>(a.cen);
+                    double2 *res = static_cast<double2 *>(a.r);
+                    double n2 = 0.0;
+#pragma unroll
+                    for (int q = 0; q < 12; q++) {
+                        const size_t o = (size_t)q * P + g;
+                        const double2 c0 = cen ? cen[o] : make_double2(0.0, 0.0);
+                        double2 w = make_double2(d * c0.x + hc * fx::to_double(acc[q].re, em),
+                                                 d * c0.y + hc * fx::to_double(acc[q].im, em));
+                        if (EPI == SPL_PLAIN || EPI == SPL_NORM) {
+                            static_cast<double2 *>(a.out)[o] = w;
+                        } else if (EPI == SPL_CG) {
+                            if (a.save_t) static_cast<double2 *>(a.tsave)[(size_t)q * a.V + s] = w;
+                            double2 rr = res[o];
+                            rr.x -= al * w.x;
+                            rr.y -= al * w.y;
+                            res[o] = rr;
+                            w = rr;
+                        } else {
+                            const double2 bb = static_cast<const double2 *>(a.b)[o];
+                            w = make_double2(bb.x - w.x, bb.y - w.y);
+                            res[o] = w;
+                        }
+                        if (EPI != SPL_PLAIN) n2 += w.x * w.x + w.y * w.y;
+                    }
+                    nrm += n2;
+                }
+            }
         }
-        nrm += n2;
+        __syncwarp();
+        const unsigned todo = __ballot_sync(0xffffffffu, fp64);
+        if (todo) nrm += elements_fp64<DAG, EPI>(a, todo, g0, prod[threadIdx.x >> 5]);
     }
     if (EPI == SPL_PLAIN) return;
     const double bs = block_reduce_rhs(nrm, (int)a.k, smem);
@@ -421,7 +410,7 @@ __global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const FxArgs a) {
 
 template <int EPI>
 cudaError_t fx_launch(bool dag, const FxArgs &a, int cap, cudaStream_t s) {
-    const long n = (long)a.V << a.kshift;
+    const long n = (long)a.s.V << a.s.kshift;
     long grid = (n + FX_TPB - 1) / FX_TPB;
     const long most = (long)device_sm_count() * 4;  // resident blocks
     if (EPI != SPL_PLAIN && grid > most) grid = most;
@@ -449,47 +438,22 @@ cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaSt
 cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Field t_save, CGScalars *st, History h,
                              int iter, bool set_rho, RedScratch red, cudaStream_t s) {
     FxArgs a;
-    memset(&a, 0, sizeof(a));
-    a.V = (unsigned)(c.eo_parity >= 0 ? c.V / 2 : c.V);
-    a.k = (unsigned)c.k;
-    while ((1u << a.kshift) < a.k) a.kshift++;
-    const unsigned n = a.V << a.kshift;
+    split_args(a.s, c);
+    if (c.eo_parity >= 0 && c.diag == 0.0) a.s.cen = nullptr;
+    split_reduction(a.s, st, h, iter, red);
+    a.s.r = r.v.data;
+    a.s.b = b.v.data;
+    a.s.tsave = t_save.v.data;
+    a.s.save_t = t_save.v.data != nullptr;
+    a.s.set_rho = set_rho;
     a.fx = static_cast<const longlong2 *>(c.fx.data);
     a.ex = c.fx.ex;
-    a.in = static_cast<const double2 *>(c.in.v.data);
-    a.cen = static_cast<const double2 *>(c.eo_parity >= 0 ? (c.diag != 0.0 ? c.cen.v.data : nullptr) : c.in.v.data);
     a.g = static_cast<const int4 *>(c.fx.links);
-    a.g64 = static_cast<const double2 *>(c.gauge.data);
-    a.out = static_cast<double2 *>(c.out.v.data);
-    a.b = static_cast<const double2 *>(b.v.data);
-    a.r = static_cast<double2 *>(r.v.data);
-    a.tsave = static_cast<double2 *>(t_save.v.data);
-    a.save_t = t_save.v.data != nullptr;
-    a.L0 = c.L[0];
-    a.L1 = c.L[1];
-    a.L2 = c.L[2];
-    a.L3 = c.L[3];
-    a.d0 = fastdiv_make(a.L0);
-    a.d1 = fastdiv_make(a.L1);
-    a.d2 = fastdiv_make(a.L2);
-    a.lh = a.L0 / 2;
-    if (a.lh >= 2) a.dh = fastdiv_make(a.lh);
-    a.Vg = (unsigned)c.V;
-    a.eo = c.eo_parity;
-    a.diag = c.diag;
-    a.hcoef = c.hcoef;
-    a.st = st;
-    a.h_alpha = h.alpha;
-    a.h_beta = h.beta;
-    a.h_rho = h.rho;
-    a.iter = iter;
-    a.jbase = h.jbase;
-    a.set_rho = set_rho;
-    a.partials = red.partials;
-    a.counter = red.counter;
+    const unsigned n = a.s.V << a.s.kshift;
     {
         long grid = (n + FX_TPB - 1) / FX_TPB;
-        k_to_fx<<<(int)grid, FX_TPB, 0, s>>>(a.in, static_cast<longlong2 *>(c.fx.data), c.fx.ex, n);
+        k_to_fx<<<(int)grid, FX_TPB, 0, s>>>(static_cast<const double2 *>(c.in.v.data),
+                                                static_cast<longlong2 *>(c.fx.data), c.fx.ex, n);
     }
     switch (epi) {
         case SPL_PLAIN: return fx_launch<SPL_PLAIN>(c.dagger, a, 0, s);

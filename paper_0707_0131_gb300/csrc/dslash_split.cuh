@@ -187,6 +187,30 @@ __device__ __forceinline__ double group_norm2(bool mine, Cx<double> o) {
     return n;
 }
 
+// Site s, RHS r through the epilogue (see launch_dslash, _norm, _cg and _resid in kernels.cuh);
+// returns the group's |result|^2 (0 for SPL_PLAIN).  Collective over the warp, live uniform over
+// a 16-lane group.
+template <bool DAG, int EPI>
+__device__ __forceinline__ double split_site(const SplitArgs &a, const LaneRole &role, bool live, unsigned s, unsigned r,
+                                             Cx<double> (*prod)[2][3]) {
+    const int l = role.l;
+    const unsigned oo = s * a.out_x + r * a.out_r;
+    const bool mine = live && l < 12;
+    Cx<double> e0 = cmk<double>(0, 0);
+    if (EPI == SPL_CG && mine) e0 = load_comp(a.r, a.out_c, oo, l);
+    if (EPI == SPL_RESID && mine) e0 = load_comp(a.b, a.out_c, oo, l);
+    Cx<double> o = split_component<DAG>(a, role, live, s, r, prod);
+    if (EPI == SPL_RESID) o = e0 - o;
+    if (EPI == SPL_CG) {
+        const CGScalars &st = a.st[r];
+        const double al = st.active ? st.alpha : 0.0;
+        if (mine && a.save_t) store_comp(a.tsave, a.V, s, l, o);  // single RHS
+        o = cmk<double>(e0.re - al * o.re, e0.im - al * o.im);
+    }
+    if (mine) store_comp(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
+    return EPI != SPL_PLAIN ? group_norm2(mine, o) : 0.0;
+}
+
 template <bool DAG, int EPI>
 __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
     __shared__ Cx<double> prod[8][8][2][3];  // [group][hop][spin][colour]
@@ -206,21 +230,7 @@ __global__ void __launch_bounds__(128) k_dslash_split(const SplitArgs a) {
         const unsigned g = it * step + blockIdx.x * (blockDim.x >> 4) + grp;
         const bool live = g < total;  // uniform over a group, not over a warp
         const unsigned s = live ? g >> a.kshift : 0u, r = g & (a.k - 1);
-        const unsigned oo = s * a.out_x + r * a.out_r;
-        const bool mine = live && l < 12;
-        Cx<double> e0 = cmk<double>(0, 0);
-        if (EPI == SPL_CG && mine) e0 = load_comp(a.r, a.out_c, oo, l);
-        if (EPI == SPL_RESID && mine) e0 = load_comp(a.b, a.out_c, oo, l);
-        Cx<double> o = split_component<DAG>(a, role, live, s, r, prod[grp]);
-        if (EPI == SPL_RESID) o = e0 - o;
-        if (EPI == SPL_CG) {
-            const CGScalars &st = a.st[r];
-            const double al = st.active ? st.alpha : 0.0;
-            if (mine && a.save_t) store_comp(a.tsave, a.V, s, l, o);  // single RHS
-            o = cmk<double>(e0.re - al * o.re, e0.im - al * o.im);
-        }
-        if (mine) store_comp(EPI == SPL_CG || EPI == SPL_RESID ? a.r : a.out, a.out_c, oo, l, o);
-        if (EPI != SPL_PLAIN) nrm += group_norm2(mine, o);  // a group's RHS is the same in every pass
+        nrm += split_site<DAG, EPI>(a, role, live, s, r, prod[grp]);  // a group's RHS is the same in every pass
     }
     if (EPI == SPL_PLAIN) return;
     const int ngrp = blockDim.x >> 4, k = (int)a.k;

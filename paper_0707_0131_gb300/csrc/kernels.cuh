@@ -167,6 +167,7 @@ cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Fie
 // (dslash_split.cuh): 4096 pairs 27 : 17 us, 6144 27 : 21, 8192 27 : 26, 16384 29 : 38, 41472
 // 31 : 78 (one wave of latency on this side, FP64 issue time on the other).
 constexpr long FX_MIN = 8192;
+constexpr long FX_MAX = (1L << 32) / 12 - 1;  // 32-bit component offsets
 size_t fx_field_bytes(long n);
 size_t fx_link_bytes(long V);
 cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaStream_t s);
