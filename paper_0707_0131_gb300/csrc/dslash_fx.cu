@@ -16,9 +16,9 @@
 // products are all small against that one is not kept (fxmath.h has the bound and the guard): the
 // warp forms it again in FP64, 16 lanes to an element (dslash_split.cuh).  The same path takes
 // elements with an Inf or NaN among their neighbours, and those near the ends of the exponent
-// range.  Links must be unitary to 1% (checked when an operator is created; the sums of eight hops
-// then stay below 2^63); other operators keep the FP64 stencil, and so do launches too small to
-// fill the GPU (FX_MIN).
+// range.  Links are held relative to a power of two for which the sums of eight hops stay below
+// 2^63 (link_scale, found when an operator is created).  Operators whose links differ too much in
+// size keep the FP64 stencil, and so do launches too small to fill the GPU (FX_MIN).
 //
 // What bounds it now: the wide multiply-adds (1728 per site, 2 cycles each on the heavy half of
 // the FMA pipe, 46% busy), integer ALU (39%) and the latency of the neighbour loads at 16 warps
@@ -31,6 +31,7 @@
 // Four blocks per SM (128 registers, ~170 to 230 bytes spilled) beat three (294 us) and two (377
 // us); without the L1 prefetch of the next hop three took 311 us; with the eight hops unrolled,
 // 685.
+#include <cmath>
 #include <cstring>
 
 #include "dslash_split.cuh"
@@ -54,6 +55,7 @@ struct FxArgs {
     const longlong2 *fx;  // hop input in fixed point (re, im), tiled, 12 components
     const int *ex;        // its exponent words: [V][k]
     const int4 *g;        // links, limbs (re hi, re lo, im hi, im lo): [mu] tiled, 9 components
+    int gscale;           // ... of links 2^-gscale
     SplitArgs s;          // the call in FP64
 };
 
@@ -96,27 +98,46 @@ __global__ void __launch_bounds__(FX_TPB) k_to_fx(const double2 *__restrict__ in
 
 __host__ __device__ constexpr size_t fx_link_plane(unsigned V) { return (size_t)((V + TILE - 1) / TILE) * TILE * 9; }
 
-// links [mu][9][V] FP64 -> limbs of u 2^58; *bad is set unless every row and column has norm 1
-// to 1% (NaN and Inf included)
-__global__ void k_links_fx(const double2 *__restrict__ g, int4 *__restrict__ out, unsigned V, int *bad) {
+// high words of the largest and of the smallest nonzero squared norm of a row or column of the links
+// [mu][9][V] (Inf and NaN are above all others); range[0] starts as 0, range[1] as the largest word
+__global__ void k_links_range(const double2 *__restrict__ g, unsigned V, unsigned *range) {
+    unsigned top = 0, bottom = 0xffffffffu;
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < 4u * V; i += gridDim.x * blockDim.x) {
         const unsigned mu = i / V, s = i - mu * V;
         const double2 *p = g + (size_t)mu * 9 * V + s;
-        double row[3] = {0, 0, 0}, col[3] = {0, 0, 0};
+        double norm[6] = {0, 0, 0, 0, 0, 0};
         for (int e = 0; e < 9; e++) {
             const double2 u = p[(size_t)e * V];
             const double n = u.x * u.x + u.y * u.y;
-            row[e / 3] += n;
-            col[e % 3] += n;
+            norm[e / 3] += n;
+            norm[3 + e % 3] += n;
+        }
+        for (int q = 0; q < 6; q++) {
+            const unsigned w = (unsigned)__double2hiint(norm[q]) & 0x7fffffffu;
+            top = max(top, w);
+            if (w) bottom = min(bottom, w);
+        }
+    }
+    top = __reduce_max_sync(0xffffffffu, top);
+    bottom = __reduce_min_sync(0xffffffffu, bottom);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(range, top);
+        atomicMin(range + 1, bottom);
+    }
+}
+
+// links [mu][9][V] FP64 -> limbs of u 2^(58 - scale)
+__global__ void k_links_fx(const double2 *__restrict__ g, int4 *__restrict__ out, unsigned V, double unit) {
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < 4u * V; i += gridDim.x * blockDim.x) {
+        const unsigned mu = i / V, s = i - mu * V;
+        const double2 *p = g + (size_t)mu * 9 * V + s;
+        for (int e = 0; e < 9; e++) {
+            const double2 u = p[(size_t)e * V];
             int4 l;
-            fx::limbs(__double2ll_rn(u.x * 0x1p58), l.x, l.y);
-            fx::limbs(__double2ll_rn(u.y * 0x1p58), l.z, l.w);
+            fx::limbs(__double2ll_rn(u.x * unit), l.x, l.y);
+            fx::limbs(__double2ll_rn(u.y * unit), l.z, l.w);
             out[mu * fx_link_plane(V) + tiled(s, 9) + e * TILE] = l;
         }
-        bool ok = true;
-        for (int q = 0; q < 3; q++)
-            ok = ok && row[q] > 0.98 && row[q] < 1.02 && col[q] > 0.98 && col[q] < 1.02;
-        if (!ok) *bad = 1;
     }
 }
 
@@ -338,7 +359,8 @@ __global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const __grid_constant__
 #pragma unroll
             for (int h = 0; h < 8; h++) shifts |= (unsigned long long)min(em - e[h], 63) << (8 * h);
             unsigned formed = fx::guard_formed(sp0, true) | (fx::guard_formed(sp1, false) << 8), large = 0;
-            fp64 = fx::exponent_bad(em, sp0 | sp1);
+            const int er = em + args.gscale;  // of the results
+            fp64 = fx::exponent_bad(em, sp0 | sp1) || fx::exponent_bad(er, sp0 | sp1);
             if (!fp64) {
                 I2 acc[12];
 #pragma unroll
@@ -371,8 +393,8 @@ __global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const __grid_constant__
                     for (int q = 0; q < 12; q++) {
                         const size_t o = (size_t)q * P + g;
                         const double2 c0 = cen ? cen[o] : make_double2(0.0, 0.0);
-                        double2 w = make_double2(d * c0.x + hc * fx::to_double(acc[q].re, em),
-                                                 d * c0.y + hc * fx::to_double(acc[q].im, em));
+                        double2 w = make_double2(d * c0.x + hc * fx::to_double(acc[q].re, er),
+                                                 d * c0.y + hc * fx::to_double(acc[q].im, er));
                         if (EPI == SPL_PLAIN || EPI == SPL_NORM) {
                             static_cast<double2 *>(a.out)[o] = w;
                         } else if (EPI == SPL_CG) {
@@ -426,12 +448,25 @@ cudaError_t fx_launch(bool dag, const FxArgs &a, int cap, cudaStream_t s) {
 size_t fx_field_bytes(long n) { return (size_t)((n + TILE - 1) / TILE) * TILE * 12 * 16; }
 size_t fx_link_bytes(long V) { return 4 * fx_link_plane((unsigned)V) * 16; }
 
-cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaStream_t s) {
+cudaError_t launch_links_range(const void *g64, long V, unsigned *range, cudaStream_t s) {
+    ProfScope prof("links_range", (double)V * 4 * 144.0, s);
+    long grid = (4 * V + 127) / 128;
+    const long cap = (long)device_sm_count() * 16;
+    if (grid > cap) grid = cap;
+    cudaError_t e = cudaMemsetAsync(range, 0, sizeof(unsigned), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(range + 1, 0xff, sizeof(unsigned), s);
+    if (e != cudaSuccess) return e;
+    k_links_range<<<(int)grid, 128, 0, s>>>(static_cast<const double2 *>(g64), (unsigned)V, range);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int scale, cudaStream_t s) {
     ProfScope prof("links_fx", (double)V * 4 * 288.0, s);
     long grid = (4 * V + 127) / 128;
     const long cap = (long)device_sm_count() * 16;
     if (grid > cap) grid = cap;
-    k_links_fx<<<(int)grid, 128, 0, s>>>(static_cast<const double2 *>(g64), static_cast<int4 *>(gfx), (unsigned)V, bad);
+    k_links_fx<<<(int)grid, 128, 0, s>>>(static_cast<const double2 *>(g64), static_cast<int4 *>(gfx), (unsigned)V,
+                                         ldexp(1.0, 58 - scale));
     return cudaGetLastError();
 }
 
@@ -449,6 +484,7 @@ cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Fie
     a.fx = static_cast<const longlong2 *>(c.fx.data);
     a.ex = c.fx.ex;
     a.g = static_cast<const int4 *>(c.fx.links);
+    a.gscale = c.fx.scale;
     const unsigned n = a.s.V << a.s.kshift;
     {
         long grid = (n + FX_TPB - 1) / FX_TPB;

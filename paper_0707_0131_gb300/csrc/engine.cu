@@ -28,6 +28,7 @@
 
 #include "dense.h"
 #include "eigcg.h"
+#include "fxmath.h"
 #include "kernels.cuh"
 #include "prof.h"
 
@@ -202,7 +203,8 @@ struct eig_op_s {
     int max_rhs;
     double delta;
     DevBuf gauge64, gauge_in;
-    DevBuf gauge_fx;  // the FP64 links as limbs (dslash_fx.cu); empty if they are not unitary
+    DevBuf gauge_fx;  // the FP64 links 2^-fx_scale as limbs (dslash_fx.cu); empty if they do not suit
+    int fx_scale = 0;
     DevBuf fx_ex;     // workspace: exponents of the fixed-point field (which sits in nat_in)
     DevBuf gauge_alt;                    // FP32 ops: the links in the other FP32 format
     int gf_alt = -1;
@@ -283,6 +285,7 @@ struct eig_op_s {
             c.fx.data = nat_in.p;
             c.fx.ex = fx_ex.as<int>();
             c.fx.links = gauge_fx.p;
+            c.fx.scale = fx_scale;
         }
         return c;
     }
@@ -1490,16 +1493,15 @@ eig_status eig_op_create(const double *gauge, const int dims[4], double m_q, con
     CUDA_CK(cudaMemcpy(stage.p, gauge, stage.n, cudaMemcpyHostToDevice));
     op->gauge64.alloc((size_t)V * 4 * 9 * 16);
     CUDA_CK(launch_pack_gauge(stage.as<double>(), op->gauge64.p, GF_F64_18, V, 0));
-    if (op->Vf * K >= FX_MIN && op->gauge_fx.try_alloc(fx_link_bytes(V))) {
-        // the links as limbs of the fixed-point FP64 stencil, unless one is not unitary (or there
-        // is no room for them)
-        eig::DevBuf bad;
-        int h_bad = 1;
-        bad.alloc(sizeof(int));
-        CUDA_CK(cudaMemset(bad.p, 0, sizeof(int)));
-        CUDA_CK(launch_links_fx(op->gauge64.p, op->gauge_fx.p, V, bad.as<int>(), 0));
-        CUDA_CK(cudaMemcpy(&h_bad, bad.p, sizeof(int), cudaMemcpyDeviceToHost));
-        if (h_bad) op->gauge_fx.release();
+    if (op->Vf * K >= FX_MIN) {
+        // the links as limbs of the fixed-point FP64 stencil, where they suit it and there is room
+        eig::DevBuf range;
+        unsigned w[2] = {0, 0};
+        range.alloc(sizeof(w));
+        CUDA_CK(launch_links_range(op->gauge64.p, V, range.as<unsigned>(), 0));
+        CUDA_CK(cudaMemcpy(w, range.p, sizeof(w), cudaMemcpyDeviceToHost));
+        if (fx::link_scale(w[0], w[1], op->fx_scale) && op->gauge_fx.try_alloc(fx_link_bytes(V)))
+            CUDA_CK(launch_links_fx(op->gauge64.p, op->gauge_fx.p, V, op->fx_scale, 0));
     }
     if (op->prec != P64) {
         size_t gb = op->gf_inner == GF_F32_12 ? 48 : (op->gf_inner == GF_F32_18 ? 72 : 24);

@@ -8,7 +8,8 @@
 // in units of I as  hi hi + (hi lo + lo hi) 2^-29;  the dropped lo lo 2^-58 is at most 1/4 unit.
 //
 // Errors of one hop component w = sum over 3 colours of u (a +- b), in units of I (2^-57 of the
-// next power of two above the largest component M of the eight neighbours):
+// next power of two above the largest component M of the eight neighbours), for links whose rows
+// have norm 1:
 //   inputs     to_fixed rounds by 1/2, align by 1/2 of what is left: at most 3/4 per real, 3/2 per
 //              real of a +- b, and 3/2 sqrt(6) < 3.7 over a row of norm 1
 //   links      1/2 2^-58 on six |a +- b| <= 2^58: 3
@@ -129,6 +130,17 @@ FX_HD void mul_add(Acc &a, int uh, int ul, int h, int l) {
     wide_add(a.mid, ul, h);
 }
 FX_HD long long value(long long hh, long long mid) { return hh + ((mid + (1ll << (LIMB - 1))) >> LIMB); }
+
+// The power of two that links are held relative to: the largest squared norm of a row or column, as
+// its high word top, then lies between 1/2 and 2 (a norm of sqrt 2 keeps the sums of eight hops below
+// 2^63, and the bounds above grow by it).  False where the fixed-point form is not for these links:
+// Inf or NaN, near the ends of the exponent range, all zero, or the smallest nonzero norm (bottom) less
+// than 1/16 of the largest, where too many elements would fail the guard.
+FX_HD bool link_scale(unsigned top, unsigned bottom, int &scale) {
+    const int et = (int)(top >> 20) - 1022, eb = (int)(bottom >> 20) - 1022;  // norms^2 in [2^(e-1), 2^e)
+    scale = et >= 1 ? et / 2 : -((1 - et) / 2);
+    return top < 0x7fe00000u && et > -900 && et < 900 && et - eb <= 8;
+}
 
 // The guard.  Exponent words hold a block's exponent and, from bit NZ on, which of its four spins
 // have a nonzero component.  Blocks whose largest exponent lies outside [EX_LOW, EX_HIGH) are left

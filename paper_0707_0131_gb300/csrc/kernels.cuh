@@ -72,11 +72,13 @@ struct History {
 };
 
 // Scratch and links of the fixed-point FP64 stencil (dslash_fx.cu): 192 bytes per (site, RHS)
-// of the input, one int each, and the links as limbs; links == nullptr: not available.
+// of the input, one int each, and the links as limbs of links 2^-scale; links == nullptr: not
+// available.
 struct FxScratch {
     void *data = nullptr;
     int *ex = nullptr;
     const void *links = nullptr;
+    int scale = 0;
 };
 
 struct DslashCall {
@@ -158,11 +160,11 @@ int dslash32_best_gformat(long V, int k, int prec);
 int dslash32_choice(const DslashCall &c, int *variant);
 
 // dslash_fx.cu: the FP64 stencil in block fixed-point integer arithmetic (c.fx set), epilogue
-// epi of dslash_split.cuh; and the links as limbs, *bad (device) set where a link is not
-// unitary to 1%
+// epi of cg_scalars.cuh; the range of the links' norms and the links as limbs (fxmath.h,
+// link_scale)
 cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Field t_save, CGScalars *st, History h,
                              int iter, bool set_rho, RedScratch red, cudaStream_t s);
-// From this many (site, RHS) pairs on, FP64 launches of operators with unitary links take it.
+// From this many (site, RHS) pairs on, FP64 launches of operators that have the limbs take it.
 // Per product, conversion to fixed point included, against the hops spread over lanes
 // (dslash_split.cuh): 4096 pairs 27 : 17 us, 6144 27 : 21, 8192 27 : 26, 16384 29 : 38, 41472
 // 31 : 78 (one wave of latency on this side, FP64 issue time on the other).
@@ -170,7 +172,8 @@ constexpr long FX_MIN = 8192;
 constexpr long FX_MAX = (1L << 32) / 12 - 1;  // 32-bit component offsets
 size_t fx_field_bytes(long n);
 size_t fx_link_bytes(long V);
-cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int *bad, cudaStream_t s);
+cudaError_t launch_links_range(const void *g64, long V, unsigned *range, cudaStream_t s);
+cudaError_t launch_links_fx(const void *g64, void *gfx, long V, int scale, cudaStream_t s);
 
 // ---------------------------- blas.cu -------------------------------------------------
 // natural FP64 [k][V][12] complex  <->  internal field

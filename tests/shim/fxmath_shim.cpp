@@ -11,17 +11,21 @@ typedef _Float128 Q;
 extern "C" long long fx_to_fixed(double x, int e) { return fx::to_fixed(x, e); }
 extern "C" double fx_to_double(long long a, int e) { return fx::to_double(a, e); }
 extern "C" long long fx_align(long long a, int sh) { return fx::align(a, sh); }
+extern "C" int fx_link_scale(double top, double bottom, int *scale) {  // squared norms
+    return fx::link_scale((unsigned)(fx::bits(top) >> 32), (unsigned)(fx::bits(bottom) >> 32), *scale);
+}
 extern "C" long long fx_limbs(long long a) {  // hi 2^29 + lo, or a value far off if lo is out of range
     int hi, lo;
     fx::limbs(a, hi, lo);
     return lo < -(1 << 28) || lo >= (1 << 28) ? 1ll << 62 : (long long)hi * (1ll << 29) + lo;
 }
 
+// scale: the power of two the links are held relative to.
 // psi: neighbours [8][12] complex, hop 2 mu + (backward); u: their links [8][3][3] complex;
 // forward projectors I - g_mu, backward I + g_mu.  err: largest error of a component over 2^-53
 // times the sum of its terms |u_ab| |h_b|; units: largest error in units of the integers, the final
 // FP64 rounding taken off.  Returns 1 if the guard keeps the fixed-point result.
-extern "C" int fx_element(const double *psi, const double *u, double *err, double *units) {
+extern "C" int fx_element(const double *psi, const double *u, int scale, double *err, double *units) {
     static const int part[4][2] = {{1, 0}, {1, 0}, {0, 1}, {0, 1}};
     static const int fre[4][2] = {{0, 0}, {-1, 1}, {0, 0}, {1, 1}}, fim[4][2] = {{1, 1}, {0, 0}, {1, -1}, {0, 0}};
     int ex[8], em = 1;
@@ -61,8 +65,8 @@ extern "C" int fx_element(const double *psi, const double *u, double *err, doubl
                     const int e = 3 * s + b, l = (h & 1) ? 3 * b + q : 3 * q + b;
                     const double ur = g[2 * l], ui = (h & 1) ? -g[2 * l + 1] : g[2 * l + 1];
                     int ah, al, bh, bl, rh, rl, ih, il;
-                    fx::limbs(std::llrint(ur * 0x1p58), ah, al);
-                    fx::limbs(std::llrint(ui * 0x1p58), bh, bl);
+                    fx::limbs(std::llrint(ur * std::ldexp(1.0, 58 - scale)), ah, al);
+                    fx::limbs(std::llrint(ui * std::ldexp(1.0, 58 - scale)), bh, bl);
                     fx::limbs(H[e][0], rh, rl);
                     fx::limbs(H[e][1], ih, il);
                     fx::mul_add(re, ah, al, rh, rl);
@@ -89,16 +93,16 @@ extern "C" int fx_element(const double *psi, const double *u, double *err, doubl
         }
     }
     *err = *units = 0;
-    const Q unit = (Q)std::ldexp(1.0, em - 1079 + 500) * (Q)0x1p-500;
+    const Q unit = (Q)std::ldexp(1.0, em + scale - 1079 + 500) * (Q)0x1p-500;
     for (int e = 0; e < 12; e++)
         for (int c = 0; c < 2; c++) {
-            Q d = (Q)fx::to_double(acc[e][c], em) - exact[e][c], a = exact[e][c];
+            Q d = (Q)fx::to_double(acc[e][c], em + scale) - exact[e][c], a = exact[e][c];
             d = d < 0 ? -d : d;
             a = a < 0 ? -a : a;
             if (terms[e] > 0) *err = std::max(*err, (double)(d / terms[e]) * 0x1p53);
             else if (d > 0) *err = INFINITY;
             *units = std::max(*units, (double)((d - a * (Q)0x1p-53) / unit));
         }
-    return !fx::exponent_bad(em, sp0 | sp1) &&
+    return !fx::exponent_bad(em, sp0 | sp1) && !fx::exponent_bad(em + scale, sp0 | sp1) &&
            !fx::guard_bad(fx::guard_formed(sp0, true), large >> 8, fx::guard_formed(sp1, false), large & 63);
 }

@@ -124,3 +124,44 @@ def test_colours_of_unit_links_stay_apart(api, even_odd, prec):
         assert np.all(np.abs(two - one) <= bar)
         assert np.all(two[..., 2] == 0)
     op.close()
+
+
+@pytest.mark.parametrize("sizes", [(3.0, 3.0, 3.0, 3.0), (0.06, 0.06, 0.06, 0.06), (1.0, 0.5, 1.2, 0.2), (1e30, 1e30, 1e30, 1e29)])
+def test_links_of_other_sizes(api, sizes):
+    """Links that are not unitary (smeared, anisotropic): the bound of unit rows times sqrt 2 for the
+    power of two they are held relative to, as above, (71 sqrt 2 + 16) / 2 < 60."""
+    dims, m_q = (8, 8, 8, 8), 0.05
+    gauge = fx.make_gauge(dims, 95) * np.array(sizes)[:, None, None]
+    op = api.Op(gauge, dims, m_q, prec=64, max_rhs=2)
+    psi = _field(np.random.default_rng(96), "gauss", (2, op.V, 4, 3))
+    for which in (0, 1):
+        one, two = np.empty_like(psi), np.empty_like(psi)
+        for r in range(2):
+            op.apply(which, np.ascontiguousarray(psi[r:r + 1]), one[r:r + 1], 1)
+        op.apply(which, psi, two, 2)
+        bar = U53 * (60 * _hop_terms(gauge, dims, psi, which == 1) + 4 * (4 + m_q) * np.abs(psi))
+        assert np.all(np.abs(two - one) <= bar), which
+    op.close()
+
+
+def test_links_of_other_sizes_are_as_fast(api):
+    """The residuals' product of a mixed operator costs the same whatever the size of the links (it took
+    twice as long where they were left to the FP64 stencil)."""
+    import time
+
+    import torch
+
+    dims = (12, 12, 12, 24)
+    best = []
+    for size in (1.0, 3.0):
+        op = api.Op(size * fx.make_gauge(dims, 97), dims, 0.05, prec=32)
+        x = torch.randn(op.V * 12, dtype=torch.complex128, device="cuda")
+        y = torch.empty_like(x)
+        t = []
+        for _ in range(30):
+            t0 = time.perf_counter()
+            op.apply(3, x, y)
+            t.append(time.perf_counter() - t0)
+        best.append(min(t))
+        op.close()
+    assert best[1] <= 1.4 * best[0], best

@@ -32,7 +32,8 @@ def lib():
                             ("fx_to_double", [ctypes.c_longlong, ctypes.c_int], ctypes.c_double),
                             ("fx_align", [ctypes.c_longlong, ctypes.c_int], ctypes.c_longlong),
                             ("fx_limbs", [ctypes.c_longlong], ctypes.c_longlong),
-                            ("fx_element", [P, P, P, P], ctypes.c_int)]:
+                            ("fx_element", [P, P, ctypes.c_int, P, P], ctypes.c_int),
+                            ("fx_link_scale", [ctypes.c_double, ctypes.c_double, ctypes.POINTER(ctypes.c_int)], ctypes.c_int)]:
         f = getattr(L, name)
         f.argtypes, f.restype = args, res
     return L
@@ -106,7 +107,7 @@ def test_kept_elements_hold_every_component(lib, links, kind):
     for _ in range(1500):
         v = np.ascontiguousarray(_psi(rng, kind)).view(np.float64)
         u = np.ascontiguousarray(_links(rng, links)).view(np.float64)
-        keep = lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), ctypes.byref(err), ctypes.byref(units))
+        keep = lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), 0, ctypes.byref(err), ctypes.byref(units))
         assert units.value <= 70, (links, kind)
         if kind in ("large", "small"):  # Gaussian fields: kept wherever their exponents are
             assert bool(keep) == _in_range(v)
@@ -126,5 +127,33 @@ def test_ends_of_the_exponent_range_are_left_to_fp64(lib):
     for scale in (1e-285, 1e-295, 1e-308, 3e-310, 1e305, 1.7e308 / 8, 0.0):
         v = np.ascontiguousarray(np.clip(rng.normal(size=(8, 12, 2)), -4, 4) * scale)
         u = np.ascontiguousarray(_links(rng, "random")).view(np.float64)
-        assert lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), ctypes.byref(err), ctypes.byref(units)) == (
+        assert lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), 0, ctypes.byref(err), ctypes.byref(units)) == (
             scale == 0.0 or _in_range(v))
+
+
+@pytest.mark.parametrize("size", [3.0, 0.07, 1.0, 1.41, 1.42, 2.0 ** -60, 1e40])
+def test_links_of_other_sizes(lib, size):
+    """Rows of norm size: the scale keeps the largest squared norm between 1/2 and 2 (the integer sums then
+    stay below 2^63; an overflow would show), and the bounds of unit rows grow by sqrt 2."""
+    P = ctypes.POINTER(ctypes.c_double)
+    err, units, scale = ctypes.c_double(), ctypes.c_double(), ctypes.c_int()
+    assert lib.fx_link_scale(size ** 2, size ** 2, ctypes.byref(scale))
+    assert 0.5 <= size ** 2 / 4.0 ** scale.value <= 2
+    rng = np.random.default_rng(11)
+    for i in range(600):
+        v = rng.normal(size=(8, 12, 2))
+        if i % 3 == 0:  # the largest sums: every component at the top of its binade
+            v = np.sign(v) * (2 - 2.0 ** -52)
+        u = np.ascontiguousarray(size * _links(rng, ("random", "near unit", "unit")[i // 200])).view(np.float64)
+        v = np.ascontiguousarray(v)
+        keep = lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), scale, ctypes.byref(err), ctypes.byref(units))
+        assert units.value <= 70 * 2 ** 0.5
+        if keep:
+            assert err.value <= 71 * 2 ** 0.5
+
+
+def test_links_that_do_not_suit(lib):
+    s = ctypes.c_int()
+    for top, bottom, ok in [(1.0, 1.0, 1), (1.0, 1 / 200, 1), (1.0, 1 / 600, 0), (0.0, 0.0, 0), (float("inf"), 1.0, 0),
+                            (float("nan"), 1.0, 0), (1e-300, 1e-300, 0), (1e300, 1e300, 0)]:
+        assert lib.fx_link_scale(top, bottom, ctypes.byref(s)) == ok, (top, bottom)
