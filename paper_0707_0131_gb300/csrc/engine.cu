@@ -15,6 +15,7 @@
 // FP32 between reliable updates, which add it into an FP64 solution and replace r
 // by the FP64 true residual b - A x when ||r|| has fallen by reliable_delta.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <complex>
@@ -57,17 +58,37 @@ static thread_local std::string g_last_error;
 // (recursive: a destroy holds it over the sync and the frees of its buffers).
 static std::recursive_mutex g_capture_mu;
 
+// Gives back what the operator that this thread works on can do without (drop_fixed_point); false
+// if there is nothing.
+static bool drop_optional();
+
+// device bytes held by all buffers of the process
+static std::atomic<size_t> g_dev_bytes{0};
+
 struct DevBuf {
     void *p = nullptr;
     size_t n = 0;
-    void alloc(size_t bytes) {
+    // optional: a buffer that its operator works without; makes no room for itself
+    void alloc(size_t bytes, bool optional = false) {
         release();
         if (bytes == 0) return;
+        try {
+            alloc_once(bytes);
+        } catch (const Error &e) {
+            if (e.st != EIG_ERR_OOM || optional || !drop_optional()) throw;
+            alloc_once(bytes);
+        }
+    }
+    void alloc_once(size_t bytes) {
         // test hook (EIG_TEST_ALLOC_LIMIT=<bytes>): a fake of a failing cudaMalloc for
         // larger requests, so that the out-of-memory path runs without exhausting a GPU
         if (const char *ev = getenv("EIG_TEST_ALLOC_LIMIT"))
             if (bytes > std::strtoull(ev, nullptr, 10))
                 throw Error{EIG_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed (test limit)"};
+        // ... and EIG_TEST_ALLOC_TOTAL=<bytes>: of a device that holds no more than that in all
+        if (const char *ev = getenv("EIG_TEST_ALLOC_TOTAL"))
+            if (g_dev_bytes + bytes > std::strtoull(ev, nullptr, 10))
+                throw Error{EIG_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed (test total)"};
         cudaError_t e = cudaMalloc(&p, bytes);
         if (e != cudaSuccess) {
             p = nullptr;
@@ -75,11 +96,12 @@ struct DevBuf {
             throw Error{EIG_ERR_OOM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed"};
         }
         n = bytes;
+        g_dev_bytes += bytes;
     }
-    // false (and empty) where alloc would report EIG_ERR_OOM
+    // false (and empty) where an optional alloc would report EIG_ERR_OOM
     bool try_alloc(size_t bytes) {
         try {
-            alloc(bytes);
+            alloc(bytes, true);
         } catch (const Error &e) {
             if (e.st != EIG_ERR_OOM) throw;
             return false;
@@ -93,6 +115,7 @@ struct DevBuf {
         if (p) {
             std::lock_guard<std::recursive_mutex> cap_lock(g_capture_mu);
             cudaFree(p);
+            g_dev_bytes -= n;
         }
         p = nullptr;
         n = 0;
@@ -203,9 +226,12 @@ struct eig_op_s {
     int max_rhs;
     double delta;
     DevBuf gauge64, gauge_in;
-    DevBuf gauge_fx;  // the FP64 links 2^-fx_scale as limbs (dslash_fx.cu); empty if they do not suit
+    // fixed-point FP64 stencil (dslash_fx.cu), for operators with fx_ok: the links 2^-fx_scale as
+    // limbs, and (workspace) the exponents of the fixed-point field, which sits in nat_in.  Optional:
+    // both empty where there was no room, until the workspace is allocated again
+    DevBuf gauge_fx, fx_ex;
+    bool fx_ok = false;
     int fx_scale = 0;
-    DevBuf fx_ex;     // workspace: exponents of the fixed-point field (which sits in nat_in)
     DevBuf gauge_alt;                    // FP32 ops: the links in the other FP32 format
     int gf_alt = -1;
     // workspace
@@ -342,9 +368,34 @@ namespace eig {
 
 static void set_error(const Error &e) { g_last_error = e.msg; }
 
+// Gives back the buffers of the fixed-point form (and the graphs that point into them): the FP64
+// stencil does its work until the workspace is allocated again.
+static bool drop_fixed_point(eig_op_s *op) {
+    if (!op->gauge_fx.p && !op->fx_ex.p) return false;
+    std::lock_guard<std::recursive_mutex> cap_lock(g_capture_mu);
+    for (auto &g : op->graphs)
+        if (g.exec) cudaGraphExecDestroy(g.exec);
+    op->graphs.clear();
+    op->fx_ex.release();
+    op->gauge_fx.release();
+    return true;
+}
+
+// An operator in use by one call: its lock, and its optional buffers as what an allocation of the call
+// that finds no room may give back.
+static thread_local eig_op_s *g_room_op = nullptr;
+struct OpUse {
+    std::lock_guard<std::mutex> lk;
+    eig_op_s *prev;
+    explicit OpUse(eig_op_s *op) : lk(op->mu), prev(g_room_op) { g_room_op = op; }
+    ~OpUse() { g_room_op = prev; }
+};
+static bool drop_optional() { return g_room_op && drop_fixed_point(g_room_op); }
+
 // The workspace of an op: the Krylov fields for max_rhs RHS, FP64 staging and the
 // natural-layout staging (fields of Vf sites: half-lattice fields for the odd-even form).
-// Allocated when the op is created; eig_op_trim releases it together with the eigCG window
+// Allocated when the op is created (after everything the op cannot do without, the fixed-point form
+// of the FP64 stencil, if there is room); eig_op_trim releases it together with the eigCG window
 // and the CUDA graphs that point into it, and the next call that needs it allocates it again.
 static void ensure_workspace(eig_op_s *op) {
     if (op->ws) return;
@@ -368,14 +419,25 @@ static void ensure_workspace(eig_op_s *op) {
         op->full64.alloc(P64, V, K);
         op->be64.alloc(P64, Vf, K);
     }
-    if (op->gauge_fx.p && !(op->fx_ex.try_alloc((size_t)Vf * K * sizeof(int)) &&
-                            op->nat_in.try_alloc(fx_field_bytes(V * K)))) {  // at least V * 12 * 16 * K
-        // the fixed-point form is optional: without room for it the FP64 stencil does its work
-        op->fx_ex.release();
-        op->gauge_fx.release();
+    const size_t nat = (size_t)V * 12 * 16 * K;
+    op->nat_in.alloc(nat);
+    op->nat_out.alloc(nat);
+    if (op->fx_ok) {
+        bool room = op->gauge_fx.p != nullptr;
+        if (!room && op->gauge_fx.try_alloc(fx_link_bytes(V))) {
+            std::lock_guard<std::recursive_mutex> cap_lock(g_capture_mu);
+            CUDA_CK(launch_links_fx(op->gauge64.p, op->gauge_fx.p, V, op->fx_scale, 0));
+            CUDA_CK(cudaStreamSynchronize(0));
+            room = true;
+        }
+        room = room && op->fx_ex.try_alloc((size_t)Vf * K * sizeof(int));
+        const size_t field = fx_field_bytes(V * K);  // nat rounded up to whole tiles
+        if (room && field > nat) {
+            room = op->nat_in.try_alloc(field);
+            if (!room) op->nat_in.alloc(nat);
+        }
+        if (!room) drop_fixed_point(op);
     }
-    if (!op->nat_in.p) op->nat_in.alloc((size_t)V * 12 * 16 * K);
-    op->nat_out.alloc((size_t)V * 12 * 16 * K);
     op->ws = true;
 }
 
@@ -1494,14 +1556,13 @@ eig_status eig_op_create(const double *gauge, const int dims[4], double m_q, con
     op->gauge64.alloc((size_t)V * 4 * 9 * 16);
     CUDA_CK(launch_pack_gauge(stage.as<double>(), op->gauge64.p, GF_F64_18, V, 0));
     if (op->Vf * K >= FX_MIN) {
-        // the links as limbs of the fixed-point FP64 stencil, where they suit it and there is room
+        // whether the links suit the fixed-point FP64 stencil
         eig::DevBuf range;
         unsigned w[2] = {0, 0};
         range.alloc(sizeof(w));
         CUDA_CK(launch_links_range(op->gauge64.p, V, range.as<unsigned>(), 0));
         CUDA_CK(cudaMemcpy(w, range.p, sizeof(w), cudaMemcpyDeviceToHost));
-        if (fx::link_scale(w[0], w[1], op->fx_scale) && op->gauge_fx.try_alloc(fx_link_bytes(V)))
-            CUDA_CK(launch_links_fx(op->gauge64.p, op->gauge_fx.p, V, op->fx_scale, 0));
+        op->fx_ok = fx::link_scale(w[0], w[1], op->fx_scale);
     }
     if (op->prec != P64) {
         size_t gb = op->gf_inner == GF_F32_12 ? 48 : (op->gf_inner == GF_F32_18 ? 72 : 24);
@@ -1519,6 +1580,7 @@ eig_status eig_op_create(const double *gauge, const int dims[4], double m_q, con
         std::lock_guard<std::recursive_mutex> cap_lock(g_capture_mu);
         CUDA_CK(cudaDeviceSynchronize());
     }
+    OpUse use(op.get());
     ensure_workspace(op.get());
     op->st.alloc(sizeof(CGScalars) * MAX_RHS);
     op->st_h.ensure(sizeof(CGScalars) * MAX_RHS);
@@ -1543,7 +1605,7 @@ eig_status eig_op_destroy(eig_op op) {
 eig_status eig_op_trim(eig_op op, size_t *freed) {
     API_BEGIN
     ARG_CHECK(op, "null argument");
-    std::lock_guard<std::mutex> lk(op->mu);
+    OpUse lk(op);
     std::lock_guard<std::recursive_mutex> cap_lock(g_capture_mu);  // held over the sync and the frees
     CUDA_CK(cudaDeviceSynchronize());
     size_t bytes = 0;
@@ -1564,7 +1626,7 @@ eig_status eig_op_apply(eig_op op, int which, const double *in, double *out, int
     ARG_CHECK(which != 3 || op->prec != P64, "which = 3 needs an FP32 or FP16 op");
     ARG_CHECK(which != 3 || !op->eo, "which = 3 is not available for odd-even operators");
     ARG_CHECK(k >= 1 && k <= op->max_rhs && (k & (k - 1)) == 0, "k must be a power of two <= max_rhs");
-    std::lock_guard<std::mutex> lk(op->mu);
+    OpUse lk(op);
     ensure_workspace(op);
     cudaStream_t s = (cudaStream_t)stream;
     if (which == 3) {  // A = M^H M as the residuals of a mixed-precision op take it
@@ -1624,9 +1686,18 @@ eig_status eig_basis_create(eig_op op, int max_vecs, eig_basis *out) {
     std::unique_ptr<eig_basis_s> B(new eig_basis_s());
     B->op = op;
     B->max_vecs = max_vecs;
-    B->U.alloc((size_t)max_vecs * op->wfield_bytes());
-    B->pend.alloc((size_t)MAX_NEV * op->wfield_bytes());
-    B->W.alloc((size_t)MAX_NEV * op->wfield_bytes());
+    auto buffers = [&] {
+        B->U.alloc((size_t)max_vecs * op->wfield_bytes());
+        B->pend.alloc((size_t)MAX_NEV * op->wfield_bytes());
+        B->W.alloc((size_t)MAX_NEV * op->wfield_bytes());
+    };
+    try {
+        buffers();
+    } catch (const Error &e) {  // once more with what the op can give back
+        if (e.st != EIG_ERR_OOM) throw;
+        OpUse use(op);
+        buffers();
+    }
     *out = B.release();
     API_END
 }
@@ -1681,7 +1752,7 @@ static eig_status eigcg_impl(eig_op op, eig_basis basis, const double *b, double
     ARG_CHECK(tol > 0.0 && tol < 1.0, "tol must be in (0, 1)");
     ARG_CHECK(max_iter >= 1 && max_iter <= 10000000, "max_iter out of range");
     ARG_CHECK(!basis || basis->op == op, "basis belongs to another op");
-    std::lock_guard<std::mutex> lk(op->mu);
+    OpUse lk(op);
     ensure_workspace(op);
     auto t0 = std::chrono::steady_clock::now();
     cudaStream_t s = (cudaStream_t)stream;
@@ -1842,7 +1913,7 @@ eig_status eig_basis_grow(eig_basis B, void *stream) {
     API_BEGIN
     ARG_CHECK(B, "null argument");
     std::lock_guard<std::mutex> lk(B->mu);
-    std::lock_guard<std::mutex> lk2(B->op->mu);
+    OpUse lk2(B->op);
     ensure_workspace(B->op);
     eig_op_s *op = B->op;
     cudaStream_t s = (cudaStream_t)stream;
@@ -1965,7 +2036,7 @@ eig_status eig_basis_deflate(eig_basis B, const double *b, const double *x_in, d
     eig_op_s *op = B->op;
     ARG_CHECK(k >= 1 && k <= op->max_rhs && (k & (k - 1)) == 0, "k must be a power of two <= max_rhs");
     std::lock_guard<std::mutex> lk(B->mu);
-    std::lock_guard<std::mutex> lk2(op->mu);
+    OpUse lk2(op);
     ensure_workspace(op);
     cudaStream_t s = (cudaStream_t)stream;
     Field b64 = op->b64.view(k), x64 = op->x64.view(k), r64 = (op->prec == P64 ? op->r : op->r64).view(k);
@@ -2002,7 +2073,7 @@ eig_status eig_initcg_solve(eig_op op, eig_basis basis, const double *b, double 
     ARG_CHECK(tol > 0.0 && tol < 1.0, "tol must be in (0, 1)");
     ARG_CHECK(max_iter >= 1 && max_iter <= 10000000, "max_iter out of range");
     ARG_CHECK(!basis || basis->op == op, "basis belongs to another op");
-    std::lock_guard<std::mutex> lk(op->mu);
+    OpUse lk(op);
     ensure_workspace(op);
     auto t0 = std::chrono::steady_clock::now();
     cudaStream_t s = (cudaStream_t)stream;
@@ -2084,7 +2155,7 @@ eig_status eig_bicgstab_solve(eig_op op, eig_basis basis, const double *b, doubl
     ARG_CHECK(max_iter >= 1 && max_iter <= 10000000, "max_iter out of range");
     ARG_CHECK(defl_vecs >= 0, "defl_vecs must be >= 0");
     ARG_CHECK(!basis || basis->op == op, "basis belongs to another op");
-    std::lock_guard<std::mutex> lk(op->mu);
+    OpUse lk(op);
     ensure_workspace(op);
     auto t0 = std::chrono::steady_clock::now();
     cudaStream_t s = (cudaStream_t)stream;
@@ -2187,7 +2258,7 @@ eig_status eig_basis_ritz(eig_basis B, double *evals, double *resnorms, int *n, 
     API_BEGIN
     ARG_CHECK(B && evals && n, "null argument");
     std::lock_guard<std::mutex> lk(B->mu);
-    std::lock_guard<std::mutex> lk2(B->op->mu);
+    OpUse lk2(B->op);
     ensure_workspace(B->op);
     eig_op_s *op = B->op;
     cudaStream_t s = (cudaStream_t)stream;
@@ -2233,7 +2304,7 @@ eig_status eig_basis_vector(eig_basis B, int j, double *out, void *stream) {
     API_BEGIN
     ARG_CHECK(B && out, "null argument");
     ARG_CHECK(j >= 0 && j < B->l, "j out of range");
-    std::lock_guard<std::mutex> lk(B->op->mu);
+    OpUse lk(B->op);
     ensure_workspace(B->op);
     eig_op_s *op = B->op;
     cudaStream_t s = (cudaStream_t)stream;
@@ -2264,7 +2335,7 @@ eig_status eig_basis_h(eig_basis B, double *out) {
 eig_status eig_basis_save(eig_basis B, const char *path, void *stream) {
     API_BEGIN
     ARG_CHECK(B && path, "null argument");
-    std::lock_guard<std::mutex> lk(B->op->mu);
+    OpUse lk(B->op);
     ensure_workspace(B->op);
     eig_op_s *op = B->op;
     cudaStream_t s = (cudaStream_t)stream;
@@ -2310,7 +2381,7 @@ eig_status eig_basis_save(eig_basis B, const char *path, void *stream) {
 eig_status eig_basis_load(eig_basis B, const char *path, void *stream) {
     API_BEGIN
     ARG_CHECK(B && path, "null argument");
-    std::lock_guard<std::mutex> lk(B->op->mu);
+    OpUse lk(B->op);
     ensure_workspace(B->op);
     eig_op_s *op = B->op;
     cudaStream_t s = (cudaStream_t)stream;
