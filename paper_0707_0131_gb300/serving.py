@@ -46,6 +46,11 @@ KEEP_IDLE_S = 0.05
 KEEP_WAIT_S = 0.5
 
 
+# (site, RHS) pairs from which an operator holds the fixed-point form of its FP64 stencil (FX_MIN of
+# the library)
+FX_MIN_PAIRS = 8192
+
+
 @dataclass
 class OpSpec:
     key: str
@@ -72,9 +77,10 @@ class OpSpec:
         """Device bytes an operator keeps while idle: links in all forms, the basis."""
         V = int(np.prod(self.dims))
         wide = 192 if self.prec == 64 else 96
-        # FP64 links, their fixed-point limbs and the inner formats
-        # (FP32 ops keep both the 12- and the 18-real form, FP16 ops the 12-real one)
-        links = V * 4 * (144 + 144 + {64: 0, 32: 48 + 72, 16: 48}[self.prec])
+        # FP64 links, their fixed-point limbs (operators of FX_MIN_PAIRS or more) and the inner
+        # formats (FP32 ops keep both the 12- and the 18-real form, FP16 ops the 12-real one)
+        limbs = 144 if V * self.max_rhs >= FX_MIN_PAIRS else 0
+        links = V * 4 * (144 + limbs + {64: 0, 32: 48 + 72, 16: 48}[self.prec])
         basis = V * wide * (self.basis_max + self.nev + 16 + 16)
         return links + basis
 
@@ -84,7 +90,8 @@ class OpSpec:
         V = int(np.prod(self.dims))
         sp = {64: 192, 32: 96, 16: 52}[self.prec]
         wide = 192 if self.prec == 64 else 96
-        work = V * self.max_rhs * (3 * sp + 5 * 192 + 2 * wide + 2 * 192 + 4) + V * 96 * 4
+        exponents = 4 if V * self.max_rhs >= FX_MIN_PAIRS else 0
+        work = V * self.max_rhs * (3 * sp + 5 * 192 + 2 * wide + 2 * 192 + exponents) + V * 96 * 4
         window = V * wide * (self.m + 3)
         return work + window
 
