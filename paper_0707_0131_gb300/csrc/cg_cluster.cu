@@ -25,9 +25,9 @@
 // launch_dslash_cg (kernels.cuh), the arithmetic that of dslash32.cuh.
 #include <algorithm>
 #include <cstring>
-#include <mutex>
 
 #include "cg_scalars.cuh"
+#include "device_cache.h"
 #include "dslash32.cuh"
 #include "prof.h"
 
@@ -392,27 +392,34 @@ void cluster_config(long n, int k, int gformat, cudaStream_t s, cudaLaunchConfig
     cfg.numAttrs = 1;
 }
 
-// whether this GPU can hold a cluster of 16 with the largest CTAs (asked once)
+// a cluster of 16 and its shared memory are opt-ins, per device; always those of the largest CTAs, so
+// that threads that launch at the same time set the same
+cudaError_t cluster_attributes(int gformat) {
+    const void *kern = (const void *)cluster_kernel(gformat);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    cluster_config(CG_CLUSTER_MAX, 1, gformat, 0, cfg, attr);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
+}
+
+// whether the current GPU can hold a cluster of 16 with the largest CTAs
 bool cluster_fits(int gformat) {
-    static std::mutex mu;
-    static int fits[2] = {-1, -1};
-    std::lock_guard<std::mutex> lk(mu);
-    int &f = fits[gformat == GF_F32_12 ? 0 : 1];
-    if (f < 0) {
-        f = 0;
+    static DeviceCache fits[2];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    return fits[gformat == GF_F32_12 ? 0 : 1].get(dev, [&] {
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr;
         cluster_config(CG_CLUSTER_MAX, 1, gformat, 0, cfg, attr);
-        const void *kern = (const void *)cluster_kernel(gformat);
         int clusters = 0;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes) ==
-                cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters >= 1)
-            f = 1;
+        cudaError_t e = cluster_attributes(gformat);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveClusters(&clusters, (const void *)cluster_kernel(gformat), &cfg);
         cudaGetLastError();
-    }
-    return f == 1;
+        return e == cudaSuccess ? (clusters >= 1 ? 1 : 0) : -1;
+    });
 }
 
 }  // namespace
@@ -460,6 +467,8 @@ cudaError_t launch_cg_cluster(const DslashCall &c, const CgCluster &q, CGScalars
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     cluster_config((long)a.n, c.k, c.gformat, s, cfg, attr);
+    const cudaError_t e = cluster_attributes(c.gformat);
+    if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, cluster_kernel(c.gformat), a);
 }
 
