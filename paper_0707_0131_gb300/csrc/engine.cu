@@ -822,6 +822,13 @@ static bool cg_graphs_enabled() {
     return !(e && e[0] == '0');
 }
 
+// Small FP32 lattices iterate inside one thread-block cluster (cg_cluster.cu) unless EIG_CG_CLUSTER=0
+// is set (read at every solve's launches; the launches of larger lattices then).
+static bool cg_cluster_enabled() {
+    const char *e = getenv("EIG_CG_CLUSTER");
+    return !(e && e[0] == '0');
+}
+
 // The graph of CHECK iterations j0 + 1 .. j0 + CHECK for this solve's buffers (j0 is
 // read by the kernels from op->jbase_dev), captured on first use.
 static cudaGraphExec_t cg_graph(Solve &sv, eig_op_s *op) {
@@ -956,7 +963,7 @@ static bool cg_run(Solve &sv, int max_iter, Window *w, eig_op_s *op) {
         if (!restart_now && !sv.sp && sv.j + 1 <= max_iter) {
             // small lattices: the iterations up to the next check (or a full window) as one launch
             const DslashCall c = op->call(sv.p, sv.u, false, op->prec == P64);
-            if (!op->eo && cg_cluster_takes(c)) {
+            if (!op->eo && cg_cluster_takes(c) && cg_cluster_enabled()) {
                 CgCluster q;
                 q.p = sv.p;
                 q.r = sv.r;
