@@ -410,28 +410,30 @@ __device__ __forceinline__ void sum_partials(const double *partials, int nout, d
 constexpr int WR_MAXOUT = 32;
 constexpr int WR_THREADS = 128;
 
-// FP64: thread per (row, output); NO = 8, 16 or 32 bounds the outputs.  The kernel is bound by
-// FP64 issue (~64 cycles per warp instruction): with one thread per row a 4^4 window (3072
-// rows, m = 24, 16 outputs) kept 24 blocks busy with 1536 FMAs per thread (84 us); spread over
-// the outputs it fills the GPU.  A block reads all m columns of its rows before it writes any.
-template <int NO>
-__global__ void __launch_bounds__(WR_THREADS) k_window_restart64(ColSet Vw, int m, const double *QZ, int nout,
-                                                                 const double2 *t, const double2 *tp,
-                                                                 const double *beta_dev, long nrows, double *partials,
-                                                                 unsigned *counter, double *wv) {
+// FP64: thread per (row, output), R rows per block and pass.  The kernel is bound by FP64 issue (~64
+// cycles per warp instruction): with one thread per row a 4^4 window (3072 rows, m = 24, 16 outputs)
+// kept 24 blocks busy with 1536 FMAs per thread (84 us); spread over the outputs it fills the GPU.
+// Idle lanes cost what busy ones do, so R nout fills whole warps as far as it can (wr64_rows): with
+// the outputs padded to 8, 16 or 32, 16^4 sites, m = 100 took 8.6 ms for 16 outputs and 17.2 for 18, 20
+// or 32; now 8.7, 9.9, 11.0 and 17.3 (m = 24: 2 outputs 1.10 -> 0.29 ms, 10 outputs 2.19 -> 1.40).
+// A block reads all m columns of its rows before it writes any.
+constexpr int WR64_THREADS = 256;  // at most
+__global__ void __launch_bounds__(WR64_THREADS) k_window_restart64(ColSet Vw, int m, const double *QZ, int nout, int R,
+                                                                   const double2 *t, const double2 *tp,
+                                                                   const double *beta_dev, long nrows, double *partials,
+                                                                   unsigned *counter, double *wv) {
     extern __shared__ __align__(16) unsigned char sm_raw[];
     double2 *Qs = reinterpret_cast<double2 *>(sm_raw);  // [m][nout]
-    __shared__ double2 red[WR_THREADS];
+    __shared__ double2 red[WR64_THREADS];
     for (int L = threadIdx.x; L < m * nout; L += blockDim.x) Qs[L] = make_double2(QZ[2 * L], QZ[2 * L + 1]);
     __syncthreads();
-    constexpr int R = WR_THREADS / NO;  // rows per block and pass
-    const int c = threadIdx.x % NO, rr = threadIdx.x / NO;
+    const int c = threadIdx.x % nout, rr = threadIdx.x / nout;
     const double beta = *beta_dev;
     double2 *base = static_cast<double2 *>(Vw.base);
     double2 ws = make_double2(0.0, 0.0);
     for (long r0 = (long)blockIdx.x * R; r0 < nrows; r0 += (long)gridDim.x * R) {
         const long row = r0 + rr;
-        const bool on = row < nrows && c < nout;
+        const bool on = row < nrows && rr < R;
         double re = 0.0, im = 0.0;
         if (on)
             for (int a = 0; a < m; a++) {
@@ -457,7 +459,7 @@ __global__ void __launch_bounds__(WR_THREADS) k_window_restart64(ColSet Vw, int 
     if (threadIdx.x < nout) {
         double2 s = make_double2(0.0, 0.0);
         for (int q = 0; q < R; q++) {
-            const double2 z = red[q * NO + threadIdx.x];
+            const double2 z = red[q * nout + threadIdx.x];
             s.x += z.x;
             s.y += z.y;
         }
@@ -585,6 +587,22 @@ __global__ void __launch_bounds__(WR_THREADS) k_window_restart32(ColSet Vw, int 
     if (threadIdx.x == 0) *counter = 0u;
 }
 
+// rows per block and pass of k_window_restart64: of the blocks of 128 to 256 threads the one with the
+// fewest idle lanes, the smallest of those
+static int wr64_rows(int nout) {
+    int best = 0, best_idle = 0, best_n = 1;
+    for (int R = 1; R * nout <= WR64_THREADS; R++) {
+        const int n = (R * nout + 31) / 32 * 32, idle = n - R * nout;
+        if (n < 128) continue;
+        if (!best || (long)idle * best_n < (long)best_idle * n) {
+            best = R;
+            best_idle = idle;
+            best_n = n;
+        }
+    }
+    return best;
+}
+
 cudaError_t launch_window_restart(ColSet Vw, int m, const double *QZ, int nout, const void *t, const void *t_prev,
                                   const double *beta_dev, long nrows, double *wv, RedScratch red, cudaStream_t s) {
     if (nout < 1 || nout > WR_MAXOUT || m < nout || !Vw.col_off) return cudaErrorInvalidValue;
@@ -596,20 +614,14 @@ cudaError_t launch_window_restart(ColSet Vw, int m, const double *QZ, int nout, 
     const long pcap = (long)red.max_blocks * MAX_RHS * 64 / (nout * 2);
     if (grid > pcap) grid = pcap;
     if (Vw.f64) {
-#define EIG_WR64(NO)                                                                                            \
-    do {                                                                                                        \
-        const long g64 = (nrows + WR_THREADS / NO - 1) / (WR_THREADS / NO);                                     \
-        if (grid < cap && g64 > grid) grid = g64 < cap ? g64 : cap;                                             \
-        if (grid > pcap) grid = pcap;                                                                           \
-        cudaFuncSetAttribute(k_window_restart64<NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
-        k_window_restart64<NO><<<(int)grid, WR_THREADS, smem, s>>>(                                             \
-            Vw, m, QZ, nout, static_cast<const double2 *>(t), static_cast<const double2 *>(t_prev), beta_dev,   \
-            nrows, red.partials, red.counter, wv);                                                              \
-    } while (0)
-        if (nout <= 8) EIG_WR64(8);
-        else if (nout <= 16) EIG_WR64(16);
-        else EIG_WR64(32);
-#undef EIG_WR64
+        const int R = wr64_rows(nout), threads = (R * nout + 31) / 32 * 32;
+        grid = (nrows + R - 1) / R;
+        if (grid > cap) grid = cap;
+        if (grid > pcap) grid = pcap;
+        cudaFuncSetAttribute(k_window_restart64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        k_window_restart64<<<(int)grid, threads, smem, s>>>(Vw, m, QZ, nout, R, static_cast<const double2 *>(t),
+                                                            static_cast<const double2 *>(t_prev), beta_dev, nrows,
+                                                            red.partials, red.counter, wv);
     } else {
 #define EIG_WR32(NO)                                                                                       \
     do {                                                                                                   \
