@@ -1,0 +1,47 @@
+"""The host solves that advance several chains side by side (dense.cpp, no GPU): any number of columns gives
+the bits that each has alone, and a few columns cost less than a full block."""
+import time
+
+import numpy as np
+import pytest
+
+from test_host_dense import P, lib, rand_herm  # noqa: F401 (lib is a fixture)
+
+
+def _best(f, n=9):
+    t = []
+    for _ in range(n):
+        t0 = time.perf_counter()
+        f()
+        t.append(time.perf_counter() - t0)
+    return min(t)
+
+
+def _system(n, k):
+    rng = np.random.default_rng(n)
+    H = rand_herm(rng, n) + 4 * np.sqrt(n) * np.eye(n)
+    B = rng.standard_normal((k, n)) + 1j * rng.standard_normal((k, n))
+    return H, B
+
+
+@pytest.mark.parametrize("n", [1, 2, 37, 96])
+@pytest.mark.parametrize("k", [1, 2, 3, 4, 5, 8, 11, 16])
+def test_cholesky_columns_alone_and_together(lib, n, k):  # noqa: F811
+    H, B = _system(n, k)
+    X = B.copy()
+    assert lib.shim_cholesky_solve(n, P(H.copy()), P(X), k)
+    for c in range(k):
+        x = B[c:c + 1].copy()
+        assert lib.shim_cholesky_solve(n, P(H.copy()), P(x), 1)
+        assert np.array_equal(X[c], x[0])
+    assert np.abs(X @ H.T - B).max() < 1e-12 * n
+
+
+def test_few_cholesky_columns_cost_less(lib):  # noqa: F811
+    """The factorisation alone, then with 1 and with 8 columns: one column took as long as eight."""
+    n = 240
+    H, B = _system(n, 8)
+    t = {}
+    for k in (0, 1, 8):
+        t[k] = _best(lambda: lib.shim_cholesky_solve(n, P(H.copy()), P(B[:k].copy()), k))
+    assert t[1] - t[0] < 0.6 * (t[8] - t[0]), t
