@@ -24,16 +24,20 @@ def _system(n, k):
     return H, B
 
 
+def _solve(lib, H, B):  # noqa: F811
+    """Columns of H X = B, one per row of the result."""
+    h, x = H.copy(), B.copy()  # held while the library works on them
+    assert lib.shim_cholesky_solve(len(h), P(h), P(x), len(x))
+    return x
+
+
 @pytest.mark.parametrize("n", [1, 2, 37, 96])
 @pytest.mark.parametrize("k", [1, 2, 3, 4, 5, 8, 11, 16])
 def test_cholesky_columns_alone_and_together(lib, n, k):  # noqa: F811
     H, B = _system(n, k)
-    X = B.copy()
-    assert lib.shim_cholesky_solve(n, P(H.copy()), P(X), k)
+    X = _solve(lib, H, B)
     for c in range(k):
-        x = B[c:c + 1].copy()
-        assert lib.shim_cholesky_solve(n, P(H.copy()), P(x), 1)
-        assert np.array_equal(X[c], x[0])
+        assert np.array_equal(X[c], _solve(lib, H, B[c:c + 1])[0])
     assert np.abs(X @ H.T - B).max() < 1e-12 * n
 
 
@@ -43,5 +47,5 @@ def test_few_cholesky_columns_cost_less(lib):  # noqa: F811
     H, B = _system(n, 8)
     t = {}
     for k in (0, 1, 8):
-        t[k] = _best(lambda: lib.shim_cholesky_solve(n, P(H.copy()), P(B[:k].copy()), k))
+        t[k] = _best(lambda: _solve(lib, H, B[:k]))
     assert t[1] - t[0] < 0.6 * (t[8] - t[0]), t
