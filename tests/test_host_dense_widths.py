@@ -49,3 +49,30 @@ def test_few_cholesky_columns_cost_less(lib):  # noqa: F811
     for k in (0, 1, 8):
         t[k] = _best(lambda: _solve(lib, H, B[:k]))
     assert t[1] - t[0] < 0.6 * (t[8] - t[0]), t
+
+
+def _tridiag(lib, d, e, lo, hi):  # noqa: F811
+    w, Z = np.zeros(hi - lo), np.zeros((hi - lo, len(d)))
+    lib.shim_tridiag_eig(len(d), P(d), P(e), lo, hi, P(w), P(Z))
+    return w
+
+
+@pytest.mark.parametrize("n", [3, 24, 100])
+def test_eigenvalues_alone_and_together(lib, n):  # noqa: F811
+    rng = np.random.default_rng(n)
+    d, e = rng.standard_normal(n), rng.standard_normal(n)
+    ref = np.linalg.eigvalsh(np.diag(d) + np.diag(e[:-1], 1) + np.diag(e[:-1], -1))
+    alone = np.concatenate([_tridiag(lib, d, e, i, i + 1) for i in range(n)])
+    assert np.abs(alone - ref).max() < 1e-13 * n
+    for k in (1, 2, 3, 4, 5, 8, 9, 13):
+        for lo in (0, n // 2):
+            hi = min(n, lo + k)
+            assert np.array_equal(_tridiag(lib, d, e, lo, hi), alone[lo:hi])
+
+
+def test_few_eigenvalues_cost_less(lib):  # noqa: F811
+    """One or two eigenpairs of a tridiagonal took almost as long as eight."""
+    rng = np.random.default_rng(3)
+    d, e = rng.standard_normal(100), rng.standard_normal(100)
+    t = {k: _best(lambda: _tridiag(lib, d, e, 0, k), 200) for k in (1, 2, 8)}
+    assert t[1] < 0.42 * t[8] and t[2] < 0.5 * t[8], t  # 0.58 and 0.63 where all took a block of eight
