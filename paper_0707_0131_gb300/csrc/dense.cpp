@@ -212,8 +212,8 @@ void tridiag_eig(int n, const double *d, const double *e, int lo, int hi, double
     gl -= 2.0 * EPS * tnorm * n + pivmin;
     gu += 2.0 * EPS * tnorm * n + pivmin;
     // eigenvalues by bisection, eight in step, and what is left in a block of 1, 2, 4 or 8: a chain
-    // of padding costs what others do (n = 100, one eigenpair: 43
-    // us in a block of one, 85 in one of eight)
+    // of padding costs what others do (n = 100, one eigenpair: 43 us in a block of one, 85 in one
+    // of eight)
     for (int i0 = lo; i0 < hi; i0 += 8) {
         const int nl = std::min(8, hi - i0);
         double *wi = w + (i0 - lo);
