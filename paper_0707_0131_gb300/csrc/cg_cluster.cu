@@ -2,8 +2,8 @@
 //
 // On a lattice of a few thousand sites a CG iteration of three launches (p update, u = M p,
 // t = M^H u) is a chain of latencies: the launches, eight dependent rounds of L2 loads per
-// stencil in a few warps, and a last block that sums each reduction (8^4, one RHS: 21 us per
-// iteration replayed from a graph, 7 us per kernel).  Spreading the sites over more SMs does not
+// stencil in a few warps, and a last block that sums each reduction (8^4, one RHS: 18 us per
+// iteration replayed from a graph, 6 us per kernel).  Spreading the sites over more SMs does not
 // help: a grid-wide barrier through L2 cost more than the launch it replaced (21 us per
 // iteration with three of them in one cooperative launch).  Here 16 SMs hold the whole problem:
 // one cluster of 16 CTAs, one thread per (site, RHS), p, u and the links in shared memory, r and
@@ -19,7 +19,9 @@
 // but the window: the barrier's release waits for global stores, and its acquire drops the links
 // from L1 (with the links and x in global memory an iteration took 15.5 us).  Beyond 4096 (site,
 // RHS) pairs a thread would hold two and the graph of three launches is as fast (8^4, k = 2: 25
-// us per iteration).
+// us per iteration).  Up to there the cluster is the faster one at every width (us per iteration,
+// cluster : graph): 4^4, k = 1 10.1 : 17.4, k = 4 11.6 : 20.1, k = 8 14.8 : 22.1, k = 16 22.1 : 26.3;
+// 4^3x8, k = 8 17.0 : 21.9; 4x8^3, k = 2 14.6 : 20.1; 8^4, k = 1 14.4 : 18.1 (EIG_CG_CLUSTER=0).
 //
 // Steps, scalars and their order are those of launch_pupdate, launch_dslash_norm and
 // launch_dslash_cg (kernels.cuh), the arithmetic that of dslash32.cuh.
