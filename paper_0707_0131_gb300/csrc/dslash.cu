@@ -408,7 +408,7 @@ static bool split64(long n) {
 
 bool dslash_takes_natural(const DslashCall &c) {
     const long n = c.V * c.k;
-    return c.in.prec == P64 && c.eo_parity < 0 && split64(n) && (n < FX_MIN || !c.fx.links);
+    return c.in.prec == P64 && c.eo_parity < 0 && split64(n) && (n < FX_NAT_MIN || !c.fx.links);
 }
 
 template <int EPI>

@@ -169,6 +169,10 @@ cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Fie
 // (dslash_split.cuh): 4096 pairs 27 : 17 us, 6144 27 : 21, 8192 27 : 26, 16384 29 : 38, 41472
 // 31 : 78 (one wave of latency on this side, FP64 issue time on the other).
 constexpr long FX_MIN = 8192;
+// Products of the API from this many pairs on (natural layout in and out): the split form reads and
+// writes that layout itself, the fixed-point one needs two packing launches.  M / A of one call: 8192
+// pairs 51 / 75 us against split 41 / 66, 12288 50 / 75 : 48 / 79, 24576 58 / 90 : 73 / 130.
+constexpr long FX_NAT_MIN = 10240;
 constexpr long FX_MAX = (1L << 32) / 12 - 1;  // 32-bit component offsets
 size_t fx_field_bytes(long n);
 size_t fx_link_bytes(long V);

@@ -165,3 +165,24 @@ def test_links_of_other_sizes_are_as_fast(api):
         best.append(min(t))
         op.close()
     assert best[1] <= 1.4 * best[0], best
+
+
+@pytest.mark.parametrize("dims,k", [((7, 9, 7, 21), 1), ((8, 8, 8, 20), 1), ((7, 9, 7, 12), 2)])
+def test_device_vectors_on_both_sides_of_the_natural_rule(api, dims, k):
+    """Device vectors of 8192 to 10239 pairs are read and written where they are, host vectors and larger
+    device ones go through the fixed-point form: the same products (bounds of the components test)."""
+    import torch
+
+    m_q = 0.05
+    gauge = fx.make_gauge(dims, 98)
+    op = api.Op(gauge, dims, m_q, prec=64, max_rhs=k)
+    psi = _field(np.random.default_rng(99), "gauss", (k, op.V, 4, 3))
+    for which in (0, 1):
+        host = np.empty_like(psi)
+        op.apply(which, psi, host, k)
+        vin = torch.from_numpy(psi).cuda()
+        vout = torch.empty_like(vin)
+        op.apply(which, vin, vout, k)
+        bar = U53 * (44 * _hop_terms(gauge, dims, psi, which == 1) + 4 * (4 + m_q) * np.abs(psi))
+        assert np.all(np.abs(vout.cpu().numpy() - host) <= bar), which
+    op.close()
