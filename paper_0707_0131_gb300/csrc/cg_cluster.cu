@@ -14,9 +14,10 @@
 // the device scalars.
 //
 // 8^4, one RHS: 13.6 us per iteration (whole solve to 1e-8 at cond 1e4: 5.2 -> 4.0 ms); 4^4: 9.1.
-// About 4 us of it are the FP64 sums and divisions of the two reductions, most of the rest the
-// stencils' latency at two warps per sub-partition.  Nothing in the loop touches global memory
-// but the window: the barrier's release waits for global stores, and its acquire drops the links
+// Of about ten cycles per issue of a warp 3.1 wait for loads through distributed shared memory, 2.8
+// for the barriers and their release, at two warps per sub-partition; the FP64 sums and divisions of
+// the two reductions keep their pipes active for 1.2 us (profiles/cg_cluster_8x8.md).  Nothing in
+// the loop touches global memory but the window: the barrier's release waits for global stores, and its acquire drops the links
 // from L1 (with the links and x in global memory an iteration took 15.5 us).  Beyond 4096 (site,
 // RHS) pairs a thread would hold two and the graph of three launches is as fast (8^4, k = 2: 25
 // us per iteration).  Up to there the cluster is the faster one at every width (us per iteration,

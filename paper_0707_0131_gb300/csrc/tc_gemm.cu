@@ -32,8 +32,9 @@
 // groups of four warps on alternate K tiles, so that one group's waits hide behind the other's
 // work.  (With the split written back to shared memory and all eight warps on every tile, a 16
 // KB tile took ~2900 cycles whatever the basis size.)  16^3x32: 96 vectors, 16 RHS 936 -> 525 us
-// (2.7 TB/s); 20 to 30 vectors, 10 columns 890 -> 493 us.  A tile now takes ~1500 cycles: the
-// 8 MMAs issue in ~640, the rest is a worker warp's split and its share of the drain.
+// (2.7 TB/s); 20 to 30 vectors, 10 columns 890 -> 493 us.  A tile now takes ~1400 cycles
+// (profiles/tc_gemm_16x32.md: tensor pipe active 19%, ALU 28%): a worker warp's chain of loads, split,
+// stores to tensor memory and its share of the drain.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
