@@ -8,8 +8,8 @@
 //   k_to_fx      brings a field to integers I = x 2^(1079 - e), |I| <= 2^57, e the largest
 //                exponent of the 24 reals of a (site, RHS); FP64 bits beyond the 57 below a
 //                site's largest component are dropped;
-//   k_dslash_fx  aligns the eight neighbours of a site to their largest exponent (a shift),
-//                projects them by integer adds, multiplies by the links (two 29-bit limbs per
+//   k_dslash_fx  projects the eight neighbours of a site by integer adds, aligns the half spinors
+//                to their largest exponent (a shift), multiplies by the links (two 29-bit limbs per
 //                real, three wide multiply-adds per real product), sums the eight hops exactly
 //                and rounds once to FP64, where the centre term and the epilogue are formed.
 // The errors are at most 2^-50 of the largest neighbour component, so an element whose hop
@@ -21,16 +21,19 @@
 // size keep the FP64 stencil, and so do launches too small to fill the GPU (FX_MIN).
 //
 // What bounds it now: the wide multiply-adds (1728 per site, 2 cycles each on the heavy half of
-// the FMA pipe, 46% busy), integer ALU (39%) and the latency of the neighbour loads at 16 warps
-// per SM.  Measured per product, conversion included (the conversion alone 28 us, 5.4 TB/s):
-//   16^3x32, k = 4    FP64 850 us    fixed point 282 us (every element left to FP64: 1135 us)
+// the FMA pipe), integer ALU and the latency of the neighbour loads at 16 warps per SM.  Measured
+// per product, conversion included (the conversion alone 28 us, 5.4 TB/s):
+//   16^3x32, k = 4    FP64 850 us    fixed point 255 us (every element left to FP64: 1135 us)
+//   24^3x64, k = 16   FP64 22.8 ms   fixed point 6.34 ms; with the norm, CG and residual epilogues 7.4,
+//                     8.5 and 8.0 ms
 //   12^3x24, k = 8    double-float (44 bits; used for residual replacements before) 194 us plus
-//                     120 us of field conversions per A; fixed point 186 us
-// The guard keeps one bit per product; with sums of magnitudes in six registers the same product
-// took 303 us.
-// Four blocks per SM (128 registers, ~170 to 230 bytes spilled) beat three (294 us) and two (377
-// us); without the L1 prefetch of the next hop three took 311 us; with the eight hops unrolled,
-// 685.
+//                     120 us of field conversions per A; fixed point 171 us
+// The guard keeps one bit per product (sums of magnitudes in six registers: 303 us at 16^3x32).  Aligning
+// the 24 components of a neighbour instead of the 12 of its half spinor, separate sums of the middle
+// limbs and conjugating the links one by one took 282 us, and 8.6 ms for the residual at 24^3x64.
+// Four blocks per SM (128 registers, 32 to 76 bytes spilled) beat three and two (294 and 377 us when
+// four took 282); without the L1 prefetch of the next hop three took 311 us; with the eight hops
+// unrolled, 685.
 #include <cmath>
 #include <cstring>
 
@@ -170,7 +173,6 @@ __device__ __forceinline__ void prefetch_hop_fx(const FxArgs &a, int mu, unsigne
     const longlong2 *f = a.fx + tiled(o, 12);
 #pragma unroll
     for (int e = 0; e < 12; e++) asm volatile("prefetch.global.L1 [%0];" ::"l"(f + e * TILE));
-    if (mu > 3) return;
     const int4 *g = a.g + mu * fx_link_plane(a.s.Vg) + tiled(ls, 9);
 #pragma unroll
     for (int e = 0; e < 9; e++) asm volatile("prefetch.global.L1 [%0];" ::"l"(g + e * TILE));
@@ -189,8 +191,8 @@ __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool p
 #pragma unroll
     for (int e = 0; e < 12; e++) {
         const longlong2 d = __ldg(f + e * TILE);
-        v[e].re = fx::align(d.x, sh);
-        v[e].im = fx::align(d.y, sh);
+        v[e].re = d.x;
+        v[e].im = d.y;
     }
     // project: h = a + sg B_mu b (see dslash.cu for B_mu)
     I2 h[6];
@@ -218,9 +220,10 @@ __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool p
     int rh[6], rl[6], ih[6], il[6];
 #pragma unroll
     for (int e = 0; e < 6; e++) {
-        fx::limbs(h[e].re, rh[e], rl[e]);
-        fx::limbs(h[e].im, ih[e], il[e]);
+        fx::limbs(fx::align(h[e].re, sh), rh[e], rl[e]);
+        fx::limbs(fx::align(h[e].im, sh), ih[e], il[e]);
     }
+    const int sgn = bwd ? 1 : -1;  // of the links' imaginary parts in the real sums (bwd: conjugate links)
     const int4 *g = a.g + mu * fx_link_plane(a.s.Vg) + tiled(ls, 9);
     const int sq = bwd ? TILE : 3 * TILE, sb = bwd ? 3 * TILE : TILE;
     I2 w[6];
@@ -231,24 +234,30 @@ __device__ __forceinline__ void hop_fx(const FxArgs &a, int mu, bool bwd, bool p
 #pragma unroll
         for (int b = 0; b < 3; b++) {
             u[b] = __ldg(g + q * sq + b * sb);
-            if (bwd) {
-                u[b].z = -u[b].z;
-                u[b].w = -u[b].w;
-            }
         }
 #pragma unroll
         for (int s = 0; s < 2; s++) {
-            fx::Acc re{0, 0}, im{0, 0};
+            long long re = fx::MIDDLE, im = fx::MIDDLE;
 #pragma unroll
             for (int b = 0; b < 3; b++) {
                 const int e = s * 3 + b;
-                fx::mul_add(re, u[b].x, u[b].y, rh[e], rl[e]);
-                fx::mul_add(re, u[b].z, u[b].w, -ih[e], -il[e]);
-                fx::mul_add(im, u[b].x, u[b].y, ih[e], il[e]);
-                fx::mul_add(im, u[b].z, u[b].w, rh[e], rl[e]);
+                fx::mid_add(re, u[b].x, u[b].y, rh[e], rl[e]);
+                fx::mid_add(re, sgn * u[b].z, sgn * u[b].w, ih[e], il[e]);
+                fx::mid_add(im, u[b].x, u[b].y, ih[e], il[e]);
+                fx::mid_add(im, -sgn * u[b].z, -sgn * u[b].w, rh[e], rl[e]);
             }
-            w[s * 3 + q].re = fx::value(re.hh, re.mid);
-            w[s * 3 + q].im = fx::value(im.hh, im.mid);
+            fx::middle_done(re);
+            fx::middle_done(im);
+#pragma unroll
+            for (int b = 0; b < 3; b++) {
+                const int e = s * 3 + b;
+                fx::wide_add(re, u[b].x, rh[e]);
+                fx::wide_add(re, sgn * u[b].z, ih[e]);
+                fx::wide_add(im, u[b].x, ih[e]);
+                fx::wide_add(im, -sgn * u[b].z, rh[e]);
+            }
+            w[s * 3 + q].re = re;
+            w[s * 3 + q].im = im;
             if (fx::guard_large(w[s * 3 + q].re, w[s * 3 + q].im)) large |= 1u << (s * 3 + q);
         }
     }
@@ -369,9 +378,10 @@ __global__ void __launch_bounds__(FX_TPB, 4) k_dslash_fx(const __grid_constant__
 #pragma unroll 1
                 for (int h = 0; h < 8; h++) {
                     const bool bwd = h & 1;
-                    // ask L1 for the next hop's data while this one is computed
+                    // ask L1 for the next hop's data while this one is computed (the last hop asks for
+                    // its own again: a branch cost more)
                     const unsigned nx = h < 7 ? neighbour(h + 1) : nl;
-                    prefetch_hop_fx(args, (h + 1) >> 1, field_index(nx), bwd ? sl : nx);
+                    prefetch_hop_fx(args, ((h + 1) >> 1) & 3, field_index(nx), bwd ? sl : nx);
                     hop_fx(args, h >> 1, bwd, DAG != bwd, field_index(nl), bwd ? nl : sl, (int)(shifts & 63), acc, large);
                     shifts >>= 8;
                     nl = nx;

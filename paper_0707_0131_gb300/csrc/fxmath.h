@@ -10,26 +10,26 @@
 // Errors of one hop component w = sum over 3 colours of u (a +- b), in units of I (2^-57 of the
 // next power of two above the largest component M of the eight neighbours), for links whose rows
 // have norm 1:
-//   inputs     to_fixed rounds by 1/2, align by 1/2 of what is left: at most 3/4 per real, 3/2 per
-//              real of a +- b, and 3/2 sqrt(6) < 3.7 over a row of norm 1
+//   inputs     to_fixed rounds a and b by 1/2 each, align shifts that and rounds a +- b by 1/2: at
+//              most 1 per real of a +- b, and sqrt(6) < 2.5 over a row of norm 1
 //   links      1/2 2^-58 on six |a +- b| <= 2^58: 3
 //   products   1/4 each for lo lo: 1.5, and 1/2 for the rounding of the middle limb
-// 8.7 units for any one hop, 70 for the sum of eight (the integer sums are exact), one FP64
-// rounding at the end; random signs give 2 to 4 units.  70 units are 2^-50 M.
+// 7.5 units for any one hop, 60 for the sum of eight (the integer sums are exact), one FP64
+// rounding at the end; random signs give 2 to 4 units.  60 units are 2^-50 M.
 //
 // An error relative to M is not one relative to a component: FP64 keeps a component that its
 // neighbours' large ones never touch (other spins, or other colours where links do not mix them)
 // to its own precision.  So an element keeps the fixed-point result only if every output component
 // it forms is large enough (guard_bad): |re| or |im| of one of its x and y hop products, or of one
 // of its z and t hop products, reaches 2^GUARD_BIT units, a sixteenth of the power of two above M.
-// Then 70 units are below 70 times 2^-53 of the sum of the component's terms |u| |a +- b|; the
+// Then 60 units are below 60 times 2^-53 of the sum of the component's terms |u| |a +- b|; the
 // FP64 chain's own bound is 15 times.  Simulated against exact sums over fields spread by site,
 // spin, colour or component and point sources, with random, near-unit and unit links: the errors of
-// kept elements are 0.7 to 4.0 times 2^-53 of those terms at most, the FP64 chain's 1.8 to 6.0, and
+// kept elements are 0.7 to 3.9 times 2^-53 of those terms at most, the FP64 chain's 1.8 to 6.0, and
 // smaller than that in each class (with alignment by floor up to 6.8, and larger in three).  Of
 // Gaussian fields the guard leaves fewer than one element in 10^9 to FP64; twice the bound would
 // leave one in 10^5, and one in 500 where a source has a single colour (16^3x32, k = 4, such a
-// source: 397 us with this bound, 624 with twice it).
+// source: 8% over a dense one with this bound, 70% with twice it).
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -100,7 +100,7 @@ FX_HD double to_double(long long a, int emax) {
     return from_bits(out | ((uint64_t)s & 0x8000000000000000ull));
 }
 
-// I 2^-sh rounded to the nearest integer (ties up), 0 <= sh <= 63, |I| <= 2^57
+// I 2^-sh rounded to the nearest integer (ties up), 0 <= sh <= 63, |I| <= 2^58
 FX_HD long long align(long long I, int sh) {
     return (long long)((uint64_t)I + ((1ull << sh) >> 1)) >> sh;
 }
@@ -111,10 +111,6 @@ FX_HD void limbs(long long I, int &hi, int &lo) {
     lo = (int)((uint32_t)(uint64_t)I << (32 - LIMB)) >> (32 - LIMB);
 }
 
-// the sums of hi hi and of hi lo + lo hi products, and their value in units of I
-struct Acc {
-    long long hh, mid;
-};
 // acc + a b, one wide multiply-add (written out: left to itself the compiler widens the limbs
 // first and multiplies 64 by 64 bits, four instructions instead of one)
 FX_HD void wide_add(long long &acc, int a, int b) {
@@ -124,12 +120,15 @@ FX_HD void wide_add(long long &acc, int a, int b) {
     acc += (long long)a * b;
 #endif
 }
-FX_HD void mul_add(Acc &a, int uh, int ul, int h, int l) {
-    wide_add(a.hh, uh, h);
-    wide_add(a.mid, uh, l);
-    wide_add(a.mid, ul, h);
+// A sum of products u I in units of I: acc starts as MIDDLE (half a unit of the result), takes the hi lo
+// + lo hi products (mid_add), is brought to units of I (middle_done), and takes the hi hi products
+// (wide_add).  One accumulator in turn for both needs fewer registers and no addition at the end.
+constexpr long long MIDDLE = 1ll << (LIMB - 1);
+FX_HD void mid_add(long long &acc, int uh, int ul, int h, int l) {
+    wide_add(acc, uh, l);
+    wide_add(acc, ul, h);
 }
-FX_HD long long value(long long hh, long long mid) { return hh + ((mid + (1ll << (LIMB - 1))) >> LIMB); }
+FX_HD void middle_done(long long &acc) { acc >>= LIMB; }
 
 // The power of two that links are held relative to: the largest squared norm of a row or column, as
 // its high word top, then lies between 1/2 and 2 (a norm of sqrt 2 keeps the sums of eight hops below

@@ -47,38 +47,47 @@ extern "C" int fx_element(const double *psi, const double *u, int scale, double 
         const double *v = psi + h * 24, *g = u + h * 18;
         long long H[6][2], W[6][2];
         Q hq[6][2], wq[6][2], t[6];
-        auto in = [&](int e, int c) { return fx::align(fx::to_fixed(v[2 * e + c], ex[h]), sh); };
+        auto in = [&](int e, int c) { return fx::to_fixed(v[2 * e + c], ex[h]); };
         for (int s = 0; s < 2; s++)
             for (int c = 0; c < 3; c++) {
                 const int e = 3 * s + c, p = 6 + 3 * part[mu][s] + c, fr = sg * fre[mu][s], fi = sg * fim[mu][s];
-                H[e][0] = in(e, 0) + fr * in(p, 0) - fi * in(p, 1);
-                H[e][1] = in(e, 1) + fr * in(p, 1) + fi * in(p, 0);
+                H[e][0] = fx::align(in(e, 0) + fr * in(p, 0) - fi * in(p, 1), sh);
+                H[e][1] = fx::align(in(e, 1) + fr * in(p, 1) + fi * in(p, 0), sh);
                 hq[e][0] = (Q)v[2 * e] + fr * (Q)v[2 * p] - fi * (Q)v[2 * p + 1];
                 hq[e][1] = (Q)v[2 * e + 1] + fr * (Q)v[2 * p + 1] + fi * (Q)v[2 * p];
             }
         for (int s = 0; s < 2; s++)
             for (int q = 0; q < 3; q++) {
-                fx::Acc re{0, 0}, im{0, 0};
+                long long re = fx::MIDDLE, im = fx::MIDDLE;
+                int ah[3], bh[3], rh[3], ih[3];
                 const int w = 3 * s + q;
                 wq[w][0] = wq[w][1] = t[w] = 0;
                 for (int b = 0; b < 3; b++) {
                     const int e = 3 * s + b, l = (h & 1) ? 3 * b + q : 3 * q + b;
                     const double ur = g[2 * l], ui = (h & 1) ? -g[2 * l + 1] : g[2 * l + 1];
-                    int ah, al, bh, bl, rh, rl, ih, il;
-                    fx::limbs(std::llrint(ur * std::ldexp(1.0, 58 - scale)), ah, al);
-                    fx::limbs(std::llrint(ui * std::ldexp(1.0, 58 - scale)), bh, bl);
-                    fx::limbs(H[e][0], rh, rl);
-                    fx::limbs(H[e][1], ih, il);
-                    fx::mul_add(re, ah, al, rh, rl);
-                    fx::mul_add(re, bh, bl, -ih, -il);
-                    fx::mul_add(im, ah, al, ih, il);
-                    fx::mul_add(im, bh, bl, rh, rl);
+                    int al, bl, rl, il;
+                    fx::limbs(std::llrint(ur * std::ldexp(1.0, 58 - scale)), ah[b], al);
+                    fx::limbs(std::llrint(ui * std::ldexp(1.0, 58 - scale)), bh[b], bl);
+                    fx::limbs(H[e][0], rh[b], rl);
+                    fx::limbs(H[e][1], ih[b], il);
+                    fx::mid_add(re, ah[b], al, rh[b], rl);
+                    fx::mid_add(re, -bh[b], -bl, ih[b], il);
+                    fx::mid_add(im, ah[b], al, ih[b], il);
+                    fx::mid_add(im, bh[b], bl, rh[b], rl);
                     wq[w][0] += (Q)ur * hq[e][0] - (Q)ui * hq[e][1];
                     wq[w][1] += (Q)ur * hq[e][1] + (Q)ui * hq[e][0];
                     t[w] += (Q)(std::hypot(ur, ui) * std::hypot((double)hq[e][0], (double)hq[e][1]));
                 }
-                W[w][0] = fx::value(re.hh, re.mid);
-                W[w][1] = fx::value(im.hh, im.mid);
+                fx::middle_done(re);
+                fx::middle_done(im);
+                for (int b = 0; b < 3; b++) {
+                    fx::wide_add(re, ah[b], rh[b]);
+                    fx::wide_add(re, -bh[b], ih[b]);
+                    fx::wide_add(im, ah[b], ih[b]);
+                    fx::wide_add(im, bh[b], rh[b]);
+                }
+                W[w][0] = re;
+                W[w][1] = im;
                 if (fx::guard_large(W[w][0], W[w][1])) large |= 1u << w;
             }
         if (h == 3) large <<= 8;

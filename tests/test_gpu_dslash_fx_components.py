@@ -3,7 +3,7 @@ differ by many orders of magnitude, point sources and fields near the ends of th
 
 The same vectors alone (FP64 arithmetic) and two together (fixed point with FP64 where its guard asks
 for it).  A component's bound is relative to the sum of its own terms |u_ab| |h_b|, as fxmath.h derives
-it: 71 of 2^-53 for a kept element's hop sum and 16 for the FP64 chain's (a +- b, six products, eight
+it: 61 of 2^-53 for a kept element's hop sum and 16 for the FP64 chain's (a +- b, six products, eight
 hops), halved by the factor of the hop term, and four for the centre term and the last sum.
 """
 import numpy as np
@@ -87,7 +87,7 @@ def test_products_hold_every_component(api, links, kind):
             op.apply(which, np.ascontiguousarray(psi[r:r + 1]), one[r:r + 1], 1)
         op.apply(which, psi, two, 2)
         terms = _hop_terms(gauge, dims, psi, which == 1)
-        bar = U53 * (44 * terms + 4 * (4 + m_q) * np.abs(psi)) + 64 * 2.0 ** -1074
+        bar = U53 * (39 * terms + 4 * (4 + m_q) * np.abs(psi)) + 64 * 2.0 ** -1074
         err = np.abs(two - one)
         assert np.all(err <= bar), (which, (err / np.maximum(bar, 1e-320)).max())
         assert kind not in ("subnormal",) or np.abs(two - (4 + m_q) * psi).max() > 0  # the hop sum is there
@@ -129,7 +129,7 @@ def test_colours_of_unit_links_stay_apart(api, even_odd, prec):
 @pytest.mark.parametrize("sizes", [(3.0, 3.0, 3.0, 3.0), (0.06, 0.06, 0.06, 0.06), (1.0, 0.5, 1.2, 0.2), (1e30, 1e30, 1e30, 1e29)])
 def test_links_of_other_sizes(api, sizes):
     """Links that are not unitary (smeared, anisotropic): the bound of unit rows times sqrt 2 for the
-    power of two they are held relative to, as above, (71 sqrt 2 + 16) / 2 < 60."""
+    power of two they are held relative to, as above, (61 sqrt 2 + 16) / 2 < 52."""
     dims, m_q = (8, 8, 8, 8), 0.05
     gauge = fx.make_gauge(dims, 95) * np.array(sizes)[:, None, None]
     op = api.Op(gauge, dims, m_q, prec=64, max_rhs=2)
@@ -139,7 +139,7 @@ def test_links_of_other_sizes(api, sizes):
         for r in range(2):
             op.apply(which, np.ascontiguousarray(psi[r:r + 1]), one[r:r + 1], 1)
         op.apply(which, psi, two, 2)
-        bar = U53 * (60 * _hop_terms(gauge, dims, psi, which == 1) + 4 * (4 + m_q) * np.abs(psi))
+        bar = U53 * (52 * _hop_terms(gauge, dims, psi, which == 1) + 4 * (4 + m_q) * np.abs(psi))
         assert np.all(np.abs(two - one) <= bar), which
     op.close()
 
@@ -183,6 +183,6 @@ def test_device_vectors_on_both_sides_of_the_natural_rule(api, dims, k):
         vin = torch.from_numpy(psi).cuda()
         vout = torch.empty_like(vin)
         op.apply(which, vin, vout, k)
-        bar = U53 * (44 * _hop_terms(gauge, dims, psi, which == 1) + 4 * (4 + m_q) * np.abs(psi))
+        bar = U53 * (39 * _hop_terms(gauge, dims, psi, which == 1) + 4 * (4 + m_q) * np.abs(psi))
         assert np.all(np.abs(vout.cpu().numpy() - host) <= bar), which
     op.close()

@@ -1,9 +1,9 @@
 """The fixed-point arithmetic of the FP64 stencil on the host (fxmath.h, no GPU) against _Float128.
 
-Bounds (derived in fxmath.h): any element is within 70 units of the integers (2^-57 of the power of
+Bounds (derived in fxmath.h): any element is within 60 units of the integers (2^-57 of the power of
 two above the largest neighbour component) of the exact hop sum, plus one FP64 rounding.  An element
 that the guard keeps has, in every component it forms, a hop product of 2^53 units or more, so its error
-is below 70 of 2^-53 times the sum of the component's terms, plus that rounding: 71.
+is below 60 of 2^-53 times the sum of the component's terms, plus that rounding: 61.
 """
 import ctypes
 import math
@@ -108,12 +108,12 @@ def test_kept_elements_hold_every_component(lib, links, kind):
         v = np.ascontiguousarray(_psi(rng, kind)).view(np.float64)
         u = np.ascontiguousarray(_links(rng, links)).view(np.float64)
         keep = lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), 0, ctypes.byref(err), ctypes.byref(units))
-        assert units.value <= 70, (links, kind)
+        assert units.value <= 60, (links, kind)
         if kind in ("large", "small"):  # Gaussian fields: kept wherever their exponents are
             assert bool(keep) == _in_range(v)
         if keep:
             kept += 1
-            assert err.value <= 71, (links, kind, err.value)
+            assert err.value <= 61, (links, kind, err.value)
     if kind == "gauss":
         assert kept == 1500  # dense fields are not left to FP64
     if kind == "spins" or (kind == "colours" and links == "unit"):
@@ -147,9 +147,9 @@ def test_links_of_other_sizes(lib, size):
         u = np.ascontiguousarray(size * _links(rng, ("random", "near unit", "unit")[i // 200])).view(np.float64)
         v = np.ascontiguousarray(v)
         keep = lib.fx_element(v.ctypes.data_as(P), u.ctypes.data_as(P), scale, ctypes.byref(err), ctypes.byref(units))
-        assert units.value <= 70 * 2 ** 0.5
+        assert units.value <= 60 * 2 ** 0.5
         if keep:
-            assert err.value <= 71 * 2 ** 0.5
+            assert err.value <= 61 * 2 ** 0.5
 
 
 def test_links_that_do_not_suit(lib):
