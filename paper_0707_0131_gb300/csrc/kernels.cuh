@@ -166,12 +166,13 @@ cudaError_t launch_dslash_fx(const DslashCall &c, int epi, Field b, Field r, Fie
                              int iter, bool set_rho, RedScratch red, cudaStream_t s);
 // From this many (site, RHS) pairs on, FP64 launches of operators that have the limbs take it.
 // Per product, conversion to fixed point included, against the hops spread over lanes
-// (dslash_split.cuh): 4096 pairs 27 : 17 us, 6144 27 : 21, 8192 27 : 26, 16384 29 : 38, 41472
-// 31 : 78 (one wave of latency on this side, FP64 issue time on the other).
+// (dslash_split.cuh): 4096 pairs 26 : 17 us, 6144 25 : 21, 8192 25 : 26, 12288 25 : 33, 16384 25 :
+// 41, 41472 36 : 92 (one wave of latency on this side, FP64 issue time on the other).
 constexpr long FX_MIN = 8192;
 // Products of the API from this many pairs on (natural layout in and out): the split form reads and
 // writes that layout itself, the fixed-point one needs two packing launches.  M / A of one call: 8192
-// pairs 51 / 75 us against split 41 / 66, 12288 50 / 75 : 48 / 79, 24576 58 / 90 : 73 / 130.
+// pairs 47 / 70 us against split 40 / 65, 10240 47 / 70 : 43 / 70, 12288 47 / 70 : 48 / 79, 24576
+// 54 / 81 : 73 / 130.
 constexpr long FX_NAT_MIN = 10240;
 constexpr long FX_MAX = (1L << 32) / 12 - 1;  // 32-bit component offsets
 size_t fx_field_bytes(long n);
