@@ -10,11 +10,11 @@ from test_host_serving import _FakeWorker, _server
 
 
 @pytest.mark.parametrize("basis_s,gap_s,steady,least,most", [
-    (0.0, 0.0, True, 0.0, 0.02),     # nothing to lose
-    (0.03, 0.01, False, 0.02, 0.06),  # idle for as long as the basis took
-    (0.1, 0.01, True, 0.08, 0.2),    # in use all the time: the work of the basis and no longer
-    (0.03, 0.5, True, 0.0, 0.02),    # its next request comes too late to be worth the wait
-    (20.0, 0.01, True, 0.48, 0.7),   # a costly basis: the limits stay
+    (0.0, 0.0, True, 0.0, 0.2),      # nothing to lose
+    (0.01, 0.005, False, 0.005, 0.045),  # idle for as long as the basis took
+    (0.1, 0.01, True, 0.08, 0.4),    # in use all the time: the work of the basis and no longer
+    (0.03, 0.5, True, 0.0, 0.2),     # its next request comes too late to be worth the wait
+    (20.0, 0.01, True, 0.48, 2.0),   # a costly basis: the limits stay
 ])
 def test_wait_is_bounded_by_the_work_of_the_basis(basis_s, gap_s, steady, least, most):
     a, b = _FakeWorker("a", 20, 60, time.perf_counter()), _FakeWorker("b", 30, 40, 0.0)
