@@ -395,8 +395,8 @@ void cluster_config(long n, int k, int gformat, cudaStream_t s, cudaLaunchConfig
     cfg.numAttrs = 1;
 }
 
-// a cluster of 16 and its shared memory are opt-ins, per device; always those of the largest CTAs, so
-// that threads that launch at the same time set the same
+// a cluster of 16 and its shared memory are opt-ins, per device; those of the largest CTAs, so that one
+// setting does for every launch
 cudaError_t cluster_attributes(int gformat) {
     const void *kern = (const void *)cluster_kernel(gformat);
     cudaLaunchConfig_t cfg;
@@ -407,7 +407,8 @@ cudaError_t cluster_attributes(int gformat) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg.dynamicSmemBytes);
 }
 
-// whether the current GPU can hold a cluster of 16 with the largest CTAs
+// whether the current GPU can hold a cluster of 16 with the largest CTAs (asked, and the opt-ins set,
+// once per device)
 bool cluster_fits(int gformat) {
     static DeviceCache fits[2];
     int dev = 0;
@@ -470,8 +471,6 @@ cudaError_t launch_cg_cluster(const DslashCall &c, const CgCluster &q, CGScalars
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr;
     cluster_config((long)a.n, c.k, c.gformat, s, cfg, attr);
-    const cudaError_t e = cluster_attributes(c.gformat);
-    if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, cluster_kernel(c.gformat), a);
 }
 
